@@ -12,8 +12,10 @@
 // one complex sequence (Z_k = -2i (A_k + i B_k)).  A pass transforms every line
 // of one axis, each CTA P line pairs in shared memory, natural order in and
 // out (self-sorting Stockham FFTs):
-//   * FP64 path (k_dst_pass<double>): radix-4 stages (and one radix-2 stage)
-//     over the shared buffer, FP64-ALU bound on GB300;
+//   * FP64 path, N = 64..1024 (k_dst_mma, dst_mma.cuh): exact fixed-point
+//     matrix products on the tensor cores; other N (k_dst_pass<double>):
+//     radix-4 stages (and one radix-2 stage) over the shared buffer, bound by
+//     GB300's FP64 pipe;
 //   * FP32 path (k_dst32<LOGL, P>): a thread owns 16 points per stage,
 //     radix-16 register DFTs, per-stage twiddle tables, a padded buffer.
 // The pass along the slowest axis applies the spectral division in place
@@ -54,6 +56,7 @@ struct BoxSolver {
   double* s64 = nullptr;      // sin^2(k pi / 2N), k = 0..N
   float* s32 = nullptr;
   double* scale64 = nullptr;  // FP64 path: (2/N)^d / lambda on the mode grid (N-1)^d
+  uint4* frag = nullptr;      // FP64 path: digits of the sine matrix in fragment order (dst_mma.cuh)
   double* work64 = nullptr;   // grid of doubles
   float* work32 = nullptr;    // grid of floats
   double* res = nullptr;      // FP64 residual grid
@@ -86,6 +89,7 @@ struct PassArgs {
   int n;                    // N
   int logL;
   const void* tw;
+  const void* frag;         // FP64 path: sine-matrix digits (null: the FFT kernel)
   // spectral scaling (fused pass only)
   const double* cosv;
   const float* s32;           // sin^2(k pi/2N) for the FP32 path
@@ -657,6 +661,12 @@ __device__ __forceinline__ long long d2ll_pow2(double x, int F) {
   if (hi >> 31) neg32pair(rl, rh);
   return join64(rl, rh);
 }
+
+}  // namespace
+}  // namespace kfbi
+#include "dst_mma.cuh"
+namespace kfbi {
+namespace {
 
 template <int LOGL, int P>
 struct Reg {
@@ -1376,12 +1386,57 @@ cudaError_t set_smem_reg(int max_optin) {
                               max_optin);
 }
 
+// The FP64 pass on the tensor cores (dst_mma.cuh), N = 64..1024; below and
+// above (2D 2048: the dense products would cost 1.2 ms a solve, the FFT 1.9 ms,
+// but its lines do not fit beside their digits) the FFT kernel stays.
+// Measured, FFT -> products, FP64 box solve: 256^3 6709 -> 2127 us, 128^3 845 ->
+// 234, 64^3 124 -> 50, 1024^2 414 -> 412, 512^2 116 -> 85, 256^2 52 -> 35, 64^2
+// 33 -> 27; relative error against a quad-precision solve 4e-16..9e-16 -> 1e-16..3e-16.
+template <int LOGN, int W>
+void launch_mma(kfbi_problem* p, const PassArgs& A, int na, int split, cudaStream_t st) {
+  using M = Mma<LOGN, W>;
+  cudaLaunchAttribute cl;
+  cl.id = cudaLaunchAttributeClusterDimension;
+  cl.val.clusterDim = {1, 1, (unsigned)split};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)div_up(A.n - 1, M::NL), (unsigned)na, (unsigned)split);
+  cfg.blockDim = dim3(M::THREADS);
+  cfg.dynamicSmemBytes = M::SMEM;
+  cfg.stream = st;
+  cfg.attrs = &cl;
+  cfg.numAttrs = 1;
+  KFBI_LAUNCH(p, KFBI_KC_DST, cudaLaunchKernelEx(&cfg, k_dst_mma<LOGN, W>, A));
+}
+
+void launch_pass_mma(kfbi_problem* p, const PassArgs& A, int na, cudaStream_t st) {
+  const int n = A.n;
+  const long long ctas = (long long)div_up(n - 1, 8) * na;
+  // few lines (2D): clusters share a line group's modes while they fit on the
+  // SMs at one CTA each and every SM partition keeps a tile (512^2: 110 -> 85 us)
+  int split = 1;
+  while (2 * split * ctas <= 152 && (n >> 4) / (2 * split) >= 4) split *= 2;
+  // many line groups: four CTAs of four warps per SM overlap their phases
+  // (256^3: 2127 us; two of eight 2190)
+  const bool many = ctas >= 4 * 152;
+  switch (n) {
+    case 64: launch_mma<6, 4>(p, A, na, split, st); break;
+    case 128: many ? launch_mma<7, 4>(p, A, na, split, st) : launch_mma<7, 8>(p, A, na, split, st); break;
+    case 256: many ? launch_mma<8, 4>(p, A, na, split, st) : launch_mma<8, 8>(p, A, na, split, st); break;
+    case 512: launch_mma<9, 8>(p, A, na, split, st); break;
+    default: launch_mma<10, 8>(p, A, na, split, st); break;
+  }
+}
+
 // pairs per CTA: enough butterflies for 256 threads (P L / 4 >= 256), at least
 // `pmin` (strided passes read 2 P adjacent lines per row)
 template <typename T>
 void launch_pass(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st, int pmin) {
   if (sizeof(T) == 4) {
     launch_pass32(p, A, npairs_b, na, st);
+    return;
+  }
+  if (A.frag) {
+    launch_pass_mma(p, A, na, st);
     return;
   }
   const int L = 2 * A.n;
@@ -1402,6 +1457,12 @@ template <typename T, int P>
 cudaError_t set_smem(int max_optin) {
   return cudaFuncSetAttribute(k_dst_pass<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               max_optin);
+}
+
+template <int LOGN, int W>
+cudaError_t set_smem_mma() {
+  return cudaFuncSetAttribute(k_dst_mma<LOGN, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)Mma<LOGN, W>::SMEM);
 }
 
 // The passes of one DST solve of `src` (grid, FP64 or FP32) into `dst` (grid,
@@ -1432,6 +1493,7 @@ PassPlan plan_passes(kfbi_problem* p, const void* src, int src64, double* dst, i
   A.cosv = B->cosv;
   A.s32 = B->s32;
   A.scale64 = B->scale64;
+  A.frag = std::is_same<T, double>::value ? B->frag : nullptr;
   A.ih2 = 1.0 / (g.h * g.h);
   A.kt = p->kt * g.h * g.h;   // kappa h^2
   A.d = g.d;
@@ -1574,6 +1636,22 @@ kfbi_status box_create(kfbi_problem* p) {
     k_scale_table<<<std::min(div_up(nm, 256), 152 * 16), 256>>>(g.d, p->cfg.order, n, p->kt * g.h * g.h,
                                                                 gh2, B->s64, B->scale64);
     KFBI_CUDA(p, cudaGetLastError());
+    if (n >= kMmaMinN && n <= kMmaMaxN) {
+      // round(2^62 sin(pi i / N)), i = 0..N
+      std::vector<long long> sq(n + 1);
+      const long double pi = acosl(-1.0L);
+      for (int i = 0; i <= n / 2; ++i) sq[i] = sq[n - i] = llroundl(ldexpl(sinl(pi * i / n), 62));
+      sq[0] = sq[n] = 0;
+      long long* dsq = nullptr;
+      KFBI_CUDA(p, dalloc(&dsq, n + 1));
+      KFBI_CUDA(p, cudaMemcpy(dsq, sq.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice));
+      const long long cnt = mma_frag_count(n);
+      KFBI_CUDA(p, dalloc(&B->frag, cnt));
+      k_mma_table<<<std::min(div_up(cnt, 256), 152 * 8), 256>>>(n, dsq, B->frag);
+      KFBI_CUDA(p, cudaGetLastError());
+      KFBI_CUDA(p, cudaDeviceSynchronize());
+      cudaFree(dsq);
+    }
     KFBI_CUDA(p, cudaDeviceSynchronize());
   }
   KFBI_CUDA(p, dalloc(&B->nrm, 9));
@@ -1605,6 +1683,13 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, (set_smem<double, 2>(optin)));
   KFBI_CUDA(p, (set_smem<double, 4>(optin)));
   KFBI_CUDA(p, (set_smem<double, 8>(optin)));
+  KFBI_CUDA(p, (set_smem_mma<6, 4>()));
+  KFBI_CUDA(p, (set_smem_mma<7, 4>()));
+  KFBI_CUDA(p, (set_smem_mma<8, 4>()));
+  KFBI_CUDA(p, (set_smem_mma<7, 8>()));
+  KFBI_CUDA(p, (set_smem_mma<8, 8>()));
+  KFBI_CUDA(p, (set_smem_mma<9, 8>()));
+  KFBI_CUDA(p, (set_smem_mma<10, 8>()));
   KFBI_CUDA(p, (set_smem<float, 1>(optin)));
   KFBI_CUDA(p, (set_smem<float, 2>(optin)));
   KFBI_CUDA(p, (set_smem<float, 4>(optin)));
@@ -1633,6 +1718,7 @@ void box_destroy(kfbi_problem* p) {
   cudaFree(B->s64);
   cudaFree(B->s32);
   cudaFree(B->scale64);
+  cudaFree(B->frag);
   cudaFree(B->work64);
   cudaFree(B->work32);
   cudaFree(B->res);
