@@ -55,16 +55,6 @@ __global__ void k_reduce(const double* __restrict__ part, int nchunk, double* __
   }
 }
 
-// w -= sum_{i<count} h[i] V_i
-__global__ void k_project(const double* __restrict__ V, int nb, int count,
-                          const double* __restrict__ h, double* __restrict__ w) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += gridDim.x * blockDim.x) {
-    double s = w[k];
-    for (int i = 0; i < count; ++i) s -= h[i] * V[(size_t)i * nb + k];
-    w[k] = s;
-  }
-}
-
 __global__ void k_scale(double* __restrict__ w, int nb, const double* __restrict__ s, int invert) {
   double f = invert ? 1.0 / s[0] : s[0];
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += gridDim.x * blockDim.x)
@@ -77,35 +67,6 @@ __global__ void k_sub(const double* __restrict__ b, double* __restrict__ w, int 
 }
 
 __global__ void k_sqrt(double* s) { s[0] = sqrt(s[0]); }
-
-__global__ void k_add(double* __restrict__ a, const double* __restrict__ b, int k) {
-  for (int i = threadIdx.x; i < k; i += blockDim.x) a[i] += b[i];
-}
-
-// Hessenberg column j: H[0..j] = h1 + h2, H[j+1] = sqrt(nn); Givens update; res = |g[j+1]|
-__global__ void k_givens(double* __restrict__ H, int ld, int j, const double* __restrict__ h1,
-                         const double* __restrict__ hn2, double* __restrict__ cs,
-                         double* __restrict__ sn, double* __restrict__ g, double* __restrict__ res,
-                         double* __restrict__ hnorm) {
-  double* col = H + (size_t)j * ld;
-  for (int i = 0; i <= j; ++i) col[i] = h1[i];
-  double hn = sqrt(hn2[0]);
-  col[j + 1] = hn;
-  hnorm[0] = hn;
-  for (int i = 0; i < j; ++i) {
-    double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  double rr = hypot(col[j], col[j + 1]);
-  cs[j] = col[j] / rr;
-  sn[j] = col[j + 1] / rr;
-  col[j] = rr;
-  col[j + 1] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  res[0] = fabs(g[j + 1]);
-}
 
 __global__ void k_init_g(double* g, int m, const double* beta) {
   for (int i = threadIdx.x; i <= m; i += blockDim.x) g[i] = (i == 0) ? beta[0] : 0.0;
@@ -131,11 +92,9 @@ __global__ void k_update_x(const double* __restrict__ V, int nb, int k, const do
   }
 }
 
-// One Arnoldi step in one CTA (N_b moderate): w = V_{j+1} holds A v_j on entry.
-// CGS2 projections, norm, normalisation and the Givens update of column j.
 constexpr int kArnThreads = 1024;
 
-// One Arnoldi step by one CTA (N_b moderate): w = V_{j+1} holds A v_j on entry.
+// One Arnoldi step by one CTA (an instance of a batch): w = V_{j+1} holds A v_j on entry.
 // CGS2 projections (each warp owns whole dot products), norm, normalisation
 // and the Givens update of column j; res = |g_{j+1}|.
 __device__ void arnoldi_step(double* __restrict__ V, int nb, int j, double* __restrict__ H, int ld,
@@ -200,14 +159,6 @@ __device__ void arnoldi_step(double* __restrict__ V, int nb, int j, double* __re
   for (int k = tid; k < nb; k += kArnThreads) w[k] *= inv;
 }
 
-__global__ void __launch_bounds__(kArnThreads) k_arnoldi_small(
-    double* __restrict__ V, int nb, int j, double* __restrict__ H, int ld,
-    double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-    double* __restrict__ res) {
-  extern __shared__ double sm[];
-  arnoldi_step(V, nb, j, H, ld, cs, sn, g, res, sm);
-}
-
 }  // namespace
 
 // ---- batched Arnoldi over instances (iteration counters on the device) -------
@@ -257,22 +208,27 @@ __global__ void __launch_bounds__(kArnThreads) k_arnoldi_batched(const ArnDesc* 
 
 namespace {
 
-// ---- one GMRES iteration as a graph (moderate N_b) ----------------------------
-// CGS2 across many CTAs with the step index j on the device: the Arnoldi step
-// of one CTA is bound by that SM's FP64 rate (2 FMA/clk), so the projections
-// run on every SM and the Givens update on one CTA.
+// ---- one GMRES iteration on the device ----------------------------------------
+// CGS2 across many CTAs with the step index j on the device: an Arnoldi step
+// in one CTA is bound by that SM's FP64 rate (2 FMA/clk; at N_b = 29704 it took
+// 0.60 ms an iteration), so each product V_i . w is cut into chunks of
+// 2048 elements, a CTA each, and the update, which first adds its products'
+// partial sums in a fixed order, runs on every SM (0.04 ms).
 constexpr int kCgsThreads = 256;
 
-// h[i] = V_i . V_{j+1} for i <= j (CTA i; CTAs beyond j exit)
+// part[i nchunk + c] = V_i . V_{j+1} over chunk c, i <= j (CTAs beyond j exit)
 __global__ void __launch_bounds__(kCgsThreads) k_cgs_dots(const double* __restrict__ V, int nb,
-                                                          const int* __restrict__ jdev, double* __restrict__ h) {
+                                                          const int* __restrict__ jdev, int nchunk,
+                                                          double* __restrict__ part) {
   const int j = jdev[0];
-  const int i = blockIdx.x;
+  const int i = blockIdx.y, c = blockIdx.x;
   if (i > j) return;
   const double* v = V + (size_t)i * nb;
   const double* w = V + (size_t)(j + 1) * nb;
+  const int per = (nb + nchunk - 1) / nchunk;
+  const int b = c * per, e = min(nb, b + per);
   double s = 0.0;
-  for (int k = threadIdx.x; k < nb; k += kCgsThreads) s += v[k] * w[k];
+  for (int k = b + threadIdx.x; k < e; k += kCgsThreads) s += v[k] * w[k];
   s = warp_sum(s);
   __shared__ double ws[kCgsThreads / 32];
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
@@ -280,19 +236,31 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_dots(const double* __restri
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int q = 0; q < kCgsThreads / 32; ++q) t += ws[q];
-    h[i] = t;
+    part[(size_t)i * nchunk + c] = t;
   }
 }
 
-// V_{j+1} -= sum_{i <= j} h[i] V_i; with part: the CTA's sum of squares of the result
+// h[i] = sum_c part[i nchunk + c]; V_{j+1} -= sum_{i <= j} h[i] V_i; with npart:
+// the CTA's sum of squares of the result
 __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__ V, int nb,
                                                             const int* __restrict__ jdev,
-                                                            const double* __restrict__ h,
-                                                            double* __restrict__ part) {
+                                                            const double* __restrict__ part, int nchunk,
+                                                            double* __restrict__ h, double* __restrict__ npart) {
   const int j = jdev[0];
   __shared__ double hs[kMaxKrylov + 1];
-  for (int i = threadIdx.x; i <= j; i += kCgsThreads) hs[i] = h[i];
+  if (nchunk == 1) {
+    for (int i = threadIdx.x; i <= j; i += kCgsThreads) hs[i] = part[i];
+  } else {
+    for (int i = threadIdx.x >> 5; i <= j; i += kCgsThreads / 32) {
+      double s = 0.0;
+      for (int c = threadIdx.x & 31; c < nchunk; c += 32) s += part[(size_t)i * nchunk + c];
+      s = warp_sum(s);
+      if ((threadIdx.x & 31) == 0) hs[i] = s;
+    }
+  }
   __syncthreads();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i <= j; i += kCgsThreads) h[i] = hs[i];
   double* w = V + (size_t)(j + 1) * nb;
   double acc = 0.0;
   for (int k = blockIdx.x * kCgsThreads + threadIdx.x; k < nb; k += gridDim.x * kCgsThreads) {
@@ -301,7 +269,7 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__
     w[k] = s;
     acc += s * s;
   }
-  if (!part) return;
+  if (!npart) return;
   acc = warp_sum(acc);
   __shared__ double ws[kCgsThreads / 32];
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
@@ -309,7 +277,7 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int q = 0; q < kCgsThreads / 32; ++q) t += ws[q];
-    part[blockIdx.x] = t;
+    npart[blockIdx.x] = t;
   }
 }
 
@@ -599,8 +567,6 @@ kfbi_status gmres_finish(kfbi_problem* p, int k, double* x) {
   return KFBI_OK;
 }
 
-constexpr int kSmallArnoldi = 32768;   // N_b up to which one CTA runs the Arnoldi step
-
 kfbi_status gmres_create(kfbi_problem* p, int m) {
   Gmres& G = p->gm;
   G.nb = p->nx;   // the BIE's unknowns (2 N_b for the general interface kind)
@@ -614,7 +580,6 @@ kfbi_status gmres_create(kfbi_problem* p, int m) {
   KFBI_CUDA(p, dalloc(&G.y, m));
   KFBI_CUDA(p, dalloc(&G.part, (size_t)(m + 1) * G.nchunk));
   KFBI_CUDA(p, dalloc(&G.scal, 8));
-  KFBI_CUDA(p, dalloc(&G.hcol, 2 * (m + 1)));
   KFBI_CUDA(p, cudaMallocHost(reinterpret_cast<void**>(&G.host_res), 4 * sizeof(double)));
   KFBI_CUDA(p, dalloc(&G.jdev, 4));
   KFBI_CUDA(p, cudaMemset(G.jdev, 0, 4 * sizeof(int)));
@@ -634,10 +599,7 @@ void gmres_destroy(kfbi_problem* p) {
   cudaFree(G.y);
   cudaFree(G.part);
   cudaFree(G.scal);
-  cudaFree(G.hcol);
   if (G.host_res) cudaFreeHost(G.host_res);
-  if (G.it_exec) cudaGraphExecDestroy(G.it_exec);
-  if (G.it_graph) cudaGraphDestroy(G.it_graph);
   if (G.loop_exec) cudaGraphExecDestroy(G.loop_exec);
   if (G.loop_graph) cudaGraphDestroy(G.loop_graph);
   cudaFree(G.jdev);
@@ -680,10 +642,12 @@ static kfbi_status iteration_body(kfbi_problem* p, cudaGraphConditionalHandle co
   KFBI_TRY(apply_operator_impl(p, p->xbuf, p->ybuf));
   cudaStream_t cs = p->stream;
   KFBI_LAUNCH(p, KFBI_KC_GMRES, k_copy_out_batched<<<dim3(div_up(nb, 256), 1), 256, 0, cs>>>(d, G.jdev, done));
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_dots<<<G.m + 1, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.h1));
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_update<<<eb, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.h1, nullptr));
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_dots<<<G.m + 1, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.h2));
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_update<<<eb, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.h2, G.npart));
+  const dim3 dg(G.nchunk, G.m + 1);
+  for (int pass = 0; pass < 2; ++pass) {
+    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_dots<<<dg, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.nchunk, G.part));
+    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_update<<<eb, kCgsThreads, 0, cs>>>(
+        G.V, nb, G.jdev, G.part, G.nchunk, pass ? G.h2 : G.h1, pass ? G.npart : nullptr));
+  }
   KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_finish<<<1, 256, 0, cs>>>(G.H, G.m + 1, G.cs, G.sn, G.g, G.scal + 2, G.h1,
                                                                  G.h2, G.npart, eb, G.jdev, G.scal + 3, cond,
                                                                  use_cond, G.scal + 5));
@@ -739,23 +703,11 @@ static kfbi_status capture_body(kfbi_problem* p, cudaGraph_t into, cudaGraph_t* 
   return KFBI_OK;
 }
 
-// One GMRES iteration of problem p as a graph, replayed once per iteration.
-static kfbi_status iteration_graph(kfbi_problem* p) {
-  Gmres& G = p->gm;
-  if (G.it_exec) return KFBI_OK;
-  KFBI_TRY(ensure_desc(p));
-  cudaGraph_t gr = nullptr;
-  KFBI_TRY(capture_body(p, nullptr, &gr, 0, 0));
-  G.it_graph = gr;
-  KFBI_CUDA(p, cudaGraphInstantiate(&G.it_exec, gr, 0));
-  return KFBI_OK;
-}
-
 // The whole Arnoldi cycle on the device: a conditional WHILE node whose body is
 // one iteration; the finish kernel ends the loop when the residual estimate
 // reaches the threshold or after the iteration limit jdev[2], so the host
 // synchronises once per cycle instead of once per iteration.  Returns false
-// (the caller then replays the single-iteration graph) if the driver refuses
+// (the caller then launches the iterations one by one) if the driver refuses
 // conditional nodes.
 static bool loop_graph(kfbi_problem* p) {
   Gmres& G = p->gm;
@@ -796,16 +748,11 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
   Gmres& G = p->gm;
   const int nb = G.nb;
   const int m = std::max(1, std::min(restart, G.m));
-  const int ld = G.m + 1;
   cudaStream_t st = p->stream;
   const int eb = std::min(div_up(nb, 256), 152 * 4);
   double* beta = G.scal + 0;
   double* bn2 = G.scal + 1;
   double* res = G.scal + 2;
-  double* hn2 = G.scal + 3;
-  double* hnorm = G.scal + 4;
-  double* h1 = G.hcol;
-  double* h2 = G.hcol + (G.m + 1);
   KFBI_TRY(dot_self(p, b, bn2));
   double bnorm2;
   KFBI_TRY(read_scalar(p, bn2, &bnorm2));
@@ -864,7 +811,7 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
     }
     int jend = 0;
     double hres = hbeta;
-    const bool graph_it = nb <= kGraphArnoldi && p->use_graphs && !p->prof.on;
+    const bool graph_it = p->use_graphs && !p->prof.on;
     if (graph_it && loop_graph(p)) {
       // one launch runs the cycle: at most min(m, max_iter - total) iterations
       const int jmax = std::min(m, max_iter - total);
@@ -883,56 +830,19 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
       total += jdone;
       jend = jdone;
       if (!std::isfinite(hres)) return fail(p, KFBI_ERR_NONFINITE, "non-finite GMRES residual");
-    } else if (graph_it) {
-      KFBI_TRY(iteration_graph(p));
+    } else {
+      KFBI_TRY(ensure_desc(p));
       KFBI_CUDA(p, cudaMemsetAsync(G.jdev, 0, 3 * sizeof(int), st));
-    }
-    const bool stepwise = !(graph_it && G.loop_exec);
-    for (int j = 0; stepwise && j < m; ++j) {
-      double* Vj = G.V + (size_t)j * nb;
-      double* w = G.V + (size_t)(j + 1) * nb;
-      if (graph_it) {
-        KFBI_CUDA(p, cudaGraphLaunch(G.it_exec, st));
-        for (int k = 0; k < KFBI_KC_COUNT; ++k) p->prof.launches[k] += G.it_counts[k];
+      for (int j = 0; j < m; ++j) {
+        KFBI_TRY(iteration_body(p, 0, 0));
         ++total;
         KFBI_TRY(read_scalar(p, res, &hres));
         jend = j + 1;
         if (!std::isfinite(hres)) return fail(p, KFBI_ERR_NONFINITE, "non-finite GMRES residual");
         if (hres <= rtol * bnorm || total >= max_iter) break;
-        continue;
       }
-      KFBI_TRY(relax_box_tol(p));
-      KFBI_TRY(apply_operator_fast(p, Vj, w));
-      ++total;
-      if (nb <= kSmallArnoldi) {
-        size_t smem = sizeof(double) * ((size_t)(j + 2) * (kArnThreads / 32) + 2 * (size_t)(j + 2));
-        KFBI_LAUNCH(p, KFBI_KC_GMRES, k_arnoldi_small<<<1, kArnThreads, smem, st>>>(
-            G.V, nb, j, G.H, ld, G.cs, G.sn, G.g, res));
-        KFBI_CUDA(p, cudaGetLastError());
-        KFBI_TRY(read_scalar(p, res, &hres));
-        jend = j + 1;
-        if (!std::isfinite(hres)) return fail(p, KFBI_ERR_NONFINITE, "non-finite GMRES residual");
-        if (hres <= rtol * bnorm || total >= max_iter) break;
-        continue;
-      }
-      // CGS2: h1 = V^T w, w -= V h1, h2 = V^T w, w -= V h2
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_dots<<<dim3(G.nchunk, j + 1), kDotThreads, 0, st>>>(G.V, nb, j + 1, w, G.nchunk, G.part));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_reduce<<<j + 1, kDotThreads, 0, st>>>(G.part, G.nchunk, h1, 0));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_project<<<eb, 256, 0, st>>>(G.V, nb, j + 1, h1, w));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_dots<<<dim3(G.nchunk, j + 1), kDotThreads, 0, st>>>(G.V, nb, j + 1, w, G.nchunk, G.part));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_reduce<<<j + 1, kDotThreads, 0, st>>>(G.part, G.nchunk, h2, 0));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_project<<<eb, 256, 0, st>>>(G.V, nb, j + 1, h2, w));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_add<<<1, 128, 0, st>>>(h1, h2, j + 1));
-      KFBI_TRY(dot_self(p, w, hn2));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_givens<<<1, 1, 0, st>>>(G.H, ld, j, h1, hn2, G.cs, G.sn, G.g, res, hnorm));
-      KFBI_LAUNCH(p, KFBI_KC_GMRES, k_scale<<<eb, 256, 0, st>>>(w, nb, hnorm, 1));
-      KFBI_CUDA(p, cudaGetLastError());
-      KFBI_TRY(read_scalar(p, res, &hres));
-      jend = j + 1;
-      if (!std::isfinite(hres)) return fail(p, KFBI_ERR_NONFINITE, "non-finite GMRES residual");
-      if (hres <= rtol * bnorm || total >= max_iter) break;
     }
-    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_solve_y<<<1, 1, 0, st>>>(G.H, ld, jend, G.g, G.y));
+    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_solve_y<<<1, 1, 0, st>>>(G.H, G.m + 1, jend, G.g, G.y));
     KFBI_LAUNCH(p, KFBI_KC_GMRES, k_update_x<<<eb, 256, 0, st>>>(G.V, nb, jend, G.y, x));
     KFBI_CUDA(p, cudaGetLastError());
     nonzero_x = true;

@@ -34,7 +34,6 @@ constexpr double kTieEps = 1e-12;     // closest-point tie tolerance (units of h
 constexpr double kRootTol = 1e-15;    // root iteration stop |ds| <= tol N h (the box width)
 constexpr int kRootMaxIt = 64;
 constexpr int kMaxKrylov = 100;     // Krylov dimension of every problem (restart length)
-constexpr int kGraphArnoldi = 8192; // N_b up to which a GMRES iteration is one graph
 constexpr double kTraceWeightScale = 4.0;   // exp(-|xi|^2 / 4)
 
 // Status codes written by setup kernels into Problem::d_flags.
@@ -112,18 +111,15 @@ struct Gmres {
   double* y = nullptr;       // m
   double* part = nullptr;    // partial sums
   double* scal = nullptr;    // device scalars: [0] beta, [1] bnorm, [2] res, [3] tmp
-  double* hcol = nullptr;    // (m+1) coefficient scratch
   double* host_res = nullptr;  // pinned
   int nchunk = 0;
-  // one GMRES iteration (operator + Arnoldi step) as a CUDA graph with the
-  // step index on the device, for N_b <= kGraphArnoldi
+  // one GMRES iteration (operator + Arnoldi step) with the step index on the
+  // device
   int* jdev = nullptr;          // [0] j, [1] done flag (always 0 here), [2] iteration limit
   double* h1 = nullptr;         // (m+1)
   double* h2 = nullptr;         // (m+1)
   double* npart = nullptr;      // partial norms (one per CTA of the update)
   void* desc = nullptr;         // ArnDesc of this problem (device)
-  cudaGraphExec_t it_exec = nullptr;
-  cudaGraph_t it_graph = nullptr;
   // the whole Arnoldi cycle as a conditional WHILE node around that iteration
   cudaGraphExec_t loop_exec = nullptr;
   cudaGraph_t loop_graph = nullptr;
