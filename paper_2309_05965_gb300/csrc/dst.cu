@@ -16,8 +16,9 @@
 //     matrix products on the tensor cores; other N (k_dst_pass<double>):
 //     radix-4 stages (and one radix-2 stage) over the shared buffer, bound by
 //     GB300's FP64 pipe;
-//   * FP32 path (k_dst32<LOGL, P>): a thread owns 16 points per stage,
-//     radix-16 register DFTs, per-stage twiddle tables, a padded buffer.
+//   * FP32 path (k_dst32<LOGL, P, STR>): register DFTs of radix 16, a thread
+//     16 points per stage, only the half of the transform that the odd
+//     symmetry leaves (see odd_stage).
 // The pass along the slowest axis applies the spectral division in place
 // between the forward and the inverse transform (Z_{L-k} = -Z_k keeps the
 // rescaled sequence the odd extension of the next input), so 2D takes 3
@@ -371,15 +372,10 @@ __global__ void __launch_bounds__(256) k_dst_pass(PassArgs A) {
 // FP32 passes of the mixed-precision path with register DFTs.
 //
 // Each CTA transforms P line pairs (sequences of length L = 2^LOGL); a thread
-// owns 16 points of one sequence per stage.  Stockham autosort stages of
-// radix 16 (and one of radix 2^(LOGL mod 4)): a thread reads its R inputs at
-// stride L/R, multiplies by the stage twiddles, runs the R-point DFT in
-// registers and writes the R outputs at stride NS (the product of the earlier
-// radices), natural order in and out.  The shared buffer is padded by one
-// element per 16 so that the stride-R writes of the first stage and the
-// stride-L/R reads are free of bank conflicts.  Compared with the radix-4
-// shared-memory kernel above this takes 2-3 exchanges instead of 5-6 and all
-// index arithmetic is compile-time.
+// owns 16 points per stage: Stockham autosort stages, radix-R DFTs in
+// registers, natural order in and out, all index arithmetic compile-time.  The
+// shared buffer is padded by one element per 16 so that the strided accesses
+// of a stage are free of bank conflicts.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int padi(int i) { return i + (i >> 4); }
 
@@ -456,79 +452,94 @@ __device__ __forceinline__ void dftr(Cx<float>* v, Cx<float>* out) {
   }
 }
 
-// One radix-R Stockham stage in place on the padded buffer s (one sequence).
+// One radix-R Stockham stage of a sequence of length G in the padded buffer s.
 // tw is this stage's twiddle table T[r NS + k] = exp(-2 pi i r k / (NS R)):
-// the lanes of a warp have consecutive k, so each load is coalesced.
-template <int L, int R, int NS>
-__device__ __forceinline__ void reg_stage(Cx<float>* s, int tid, const Cx<float>* __restrict__ tw) {
-  constexpr int G = L / R;    // R-point DFTs per stage
-  constexpr int T = L / 16;   // threads per sequence
-  constexpr int Q = 16 / R;   // DFTs per thread
-  Cx<float> v[16];
+// the lanes of a warp have consecutive k, so each load is coalesced.  Output
+// index i goes to out(i, r, value); with INPLACE that is s again, and the
+// reads of all threads come first.
+template <int G, int R, int NS, bool INPLACE, class Out>
+__device__ __forceinline__ void reg_stage(bool act, const Cx<float>* s, int tid, const Cx<float>* __restrict__ tw,
+                                          Out&& out) {
+  constexpr int T = G >= 16 ? G / 16 : 1;   // threads per sequence
+  constexpr int Q = G / (R * T);            // DFTs per thread
+  Cx<float> v[Q * R];
+  if (act) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int j = tid + q * T;
+    for (int q = 0; q < Q; ++q)
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[q * R + r] = s[padi(j + r * G)];
+      for (int r = 0; r < R; ++r) v[q * R + r] = s[padi(tid + q * T + r * (G / R))];
   }
-  __syncthreads();
+  if (INPLACE) __syncthreads();
+  if (act) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int j = tid + q * T;
-    const int k = j & (NS - 1);
-    Cx<float>* x = v + q * R;
-    if constexpr (NS > 1) {
+    for (int q = 0; q < Q; ++q) {
+      const int j = tid + q * T;
+      const int k = j & (NS - 1);
+      Cx<float>* x = v + q * R;
+      if constexpr (NS > 1) {
 #pragma unroll
-      for (int r = 1; r < R; ++r) {
-        const float2 w = __ldg(reinterpret_cast<const float2*>(tw) + r * NS + k);
-        x[r] = cmul(x[r], Cx<float>{w.x, w.y});
+        for (int r = 1; r < R; ++r) {
+          const float2 w = __ldg(reinterpret_cast<const float2*>(tw) + r * NS + k);
+          x[r] = cmul(x[r], Cx<float>{w.x, w.y});
+        }
       }
-    }
-    Cx<float> y[R];
-    dftr<R>(x, y);
-    const int base = (j - k) * R + k;
+      Cx<float> y[R];
+      dftr<R>(x, y);
+      const int base = (j - k) * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) s[padi(base + r * NS)] = y[r];
+      for (int r = 0; r < R; ++r) out(base + r * NS, r >= R / 2, y[r]);
+    }
   }
-  __syncthreads();
+  if (INPLACE) __syncthreads();
 }
 
-// Stage plan of length 2^LOGL: radix-16 stages, then one of radix 2^(LOGL mod 4).
-// The twiddle tables of the stages after the first lie back to back.
-template <int LOGL>
-__device__ __forceinline__ void reg_fft(Cx<float>* s, int tid, const Cx<float>* __restrict__ tw) {
-  constexpr int L = 1 << LOGL;
-  constexpr int N16 = LOGL / 4, REM = LOGL % 4;
+// FFT of length G = 2^LOGG: radix-16 stages, then one of radix 2^(LOGG mod 4);
+// the twiddle tables of the stages after the first lie back to back.  All
+// stages but the last are in place; the last goes to `out` (LAST_INPLACE: s).
+// out's second argument tells whether the index is in the upper half.
+template <int LOGG, bool LAST_INPLACE, class Out>
+__device__ __forceinline__ void reg_fft(bool act, Cx<float>* s, int tid, const Cx<float>* __restrict__ tw,
+                                        Out&& out) {
+  constexpr int G = 1 << LOGG;
+  constexpr int N16 = LOGG / 4, REM = LOGG % 4;
   constexpr int NSF = 1 << (4 * N16);
-  constexpr int OFF3 = 16 * 16, OFFR = (N16 >= 2 ? 256 : 0) + (N16 >= 3 ? 16 * 256 : 0);
-  if constexpr (N16 >= 1) reg_stage<L, 16, 1>(s, tid, tw);
-  if constexpr (N16 >= 2) reg_stage<L, 16, 16>(s, tid, tw);
-  if constexpr (N16 >= 3) reg_stage<L, 16, 256>(s, tid, tw + OFF3);
-  if constexpr (REM == 1) reg_stage<L, 2, NSF>(s, tid, tw + OFFR);
-  if constexpr (REM == 2) reg_stage<L, 4, NSF>(s, tid, tw + OFFR);
-  if constexpr (REM == 3) reg_stage<L, 8, NSF>(s, tid, tw + OFFR);
+  constexpr int OFFR = N16 >= 2 ? 256 : 0;
+  static_assert(LOGG < 12, "two radix-16 stages at most");
+  auto inplace = [&](int i, bool, Cx<float> y) { s[padi(i)] = y; };
+  if constexpr (N16 >= 1) {
+    if constexpr (N16 == 1 && REM == 0) reg_stage<G, 16, 1, LAST_INPLACE>(act, s, tid, tw, out);
+    else reg_stage<G, 16, 1, true>(act, s, tid, tw, inplace);
+  }
+  if constexpr (N16 >= 2) {
+    if constexpr (REM == 0) reg_stage<G, 16, 16, LAST_INPLACE>(act, s, tid, tw, out);
+    else reg_stage<G, 16, 16, true>(act, s, tid, tw, inplace);
+  }
+  if constexpr (REM > 0) reg_stage<G, (1 << REM), NSF, LAST_INPLACE>(act, s, tid, tw + OFFR, out);
 }
 
-// Host copy of the same plan: the stage twiddle tables for length 2^logL.
+// Host copy of the same plan for transforms of length 2^logL: the twiddles
+// exp(-2 pi i j q / L) of the odd sequence's first stage, q = 1..8 by
+// j = 0..L/32, then the stage tables of length L/16.
 std::vector<float> stage_twiddles(int logL) {
-  const int L = 1 << logL;
-  std::vector<int> radix;
-  for (int k = 0; k < logL / 4; ++k) radix.push_back(16);
-  if (logL % 4) radix.push_back(1 << (logL % 4));
+  const int L = 1 << logL, logG = logL - 4;
   std::vector<float> out;
+  auto put = [&](long long num, long long den) {
+    const double ang = -2.0 * M_PI * (double)(num % den) / (double)den;
+    out.push_back((float)std::cos(ang));
+    out.push_back((float)std::sin(ang));
+  };
+  for (int q = 1; q <= 8; ++q)
+    for (int j = 0; j <= L / 32; ++j) put((long long)j * q, L);
+  std::vector<int> radix;
+  for (int k = 0; k < logG / 4; ++k) radix.push_back(16);
+  if (logG % 4) radix.push_back(1 << (logG % 4));
   int ns = 1;
   for (int R : radix) {
     if (ns > 1)
       for (int r = 0; r < R; ++r)
-        for (int k = 0; k < ns; ++k) {
-          const double ang = -2.0 * M_PI * (double)(r * k) / (double)(ns * R);
-          out.push_back((float)std::cos(ang));
-          out.push_back((float)std::sin(ang));
-        }
+        for (int k = 0; k < ns; ++k) put((long long)r * k, (long long)ns * R);
     ns *= R;
   }
-  (void)L;
-  if (out.empty()) out.assign(2, 0.f);
   return out;
 }
 
@@ -668,243 +679,299 @@ __device__ __forceinline__ long long d2ll_pow2(double x, int F) {
 namespace kfbi {
 namespace {
 
+// A line pair is one complex sequence of length L = 2N, the odd extension
+// z_{L-j} = -z_j.  Its FFT starts with a radix-16 stage over the columns
+// j, j + G, ..., j + 15 G (G = L/16), which gives 16 sequences q of length G;
+// oddness halves both parts:
+//   * column G - j is column j reversed and negated, so its outputs are those
+//     of column j: T[G-j][q] = -conj(w^{jq}) Y[j][16-q] beside
+//     T[j][q] = w^{jq} Y[j][q]; only columns 0..G/2 are transformed;
+//   * Z_{L-k} = -Z_k, so sequences 9..15 repeat 1..7; only q = 0..8 go on.
+// 9/16 of the full FFT's arithmetic and shared memory, the same operations on
+// what is left.  Inputs go from global memory to registers (each element is
+// read by one column); mode k = q + 16 k' lies at [q][k'], or, for k mod 16 > 8,
+// negated at [16 - q][G - 1 - k'].  Strided lines (STR) are dealt with the
+// CTA's adjacent pairs side by side, and their modes go from the last stage's
+// registers to global memory; contiguous lines pass the shared buffer once
+// more for coalesced stores.
+// The passes are bound by instruction issue (3D) and by latency (2D, 3 to 4
+// CTAs per SM).  Measured against the full transform (the same radix-16
+// stages over all 16 sequences), mixed box solve: 256^3 2489 -> 1688 us, 128^3
+// 459 -> 326, 2048^2 565 -> 470, 1024^2 219 -> 198, 64 batched stars 36.4 -> 31.6 ms.
 template <int LOGL, int P>
 struct Reg {
-  static constexpr int L = 1 << LOGL;
-  static constexpr int T = L / 16;          // threads per sequence
-  static constexpr int THREADS = P * T;
-  static constexpr int LP = L + L / 16;     // padded sequence length
-  static constexpr size_t SMEM = sizeof(Cx<float>) * (size_t)P * LP;
+  static constexpr int L = 1 << LOGL, N = L / 2, G = L / 16;
+  static constexpr int COLS = G / 2 + 1;
+  static constexpr int T = G >= 16 ? 9 * G / 16 : 9;   // FFT threads per pair: 16 points (G < 16: a sequence)
+  // one pair per CTA (2D): as many threads as the stores need
+  static constexpr int THREADS = P == 1 && G >= 32 ? G : (P * T + 31) / 32 * 32;
+  static constexpr int MINB = THREADS >= 128 && THREADS <= 160 ? 4 : 1;
+  static constexpr int GP = (G + G / 16) | 1;          // odd pitches: no bank conflicts across q or pairs
+  static constexpr int PP = 9 * GP;
+  static constexpr size_t SMEM = sizeof(Cx<float>) * (size_t)P * PP;
 };
 
-// Default pairs per CTA: 128 threads per CTA up to L = 2048.
-__host__ __device__ constexpr int reg_pairs(int logL) { return logL >= 11 ? 1 : (1 << (11 - logL)); }
+// buffer index of mode k of a pair; neg: the stored value is -Z_k
+template <int LOGL, int P>
+__device__ __forceinline__ int mode_at(int k, bool& neg) {
+  using F = Reg<LOGL, P>;
+  const int q = k & 15, c = k >> 4;
+  neg = q > 8;
+  return neg ? (16 - q) * F::GP + padi(F::G - 1 - c) : q * F::GP + padi(c);
+}
+
+// The radix-16 stage of column j0 from its 16 inputs, into the nine sequences.
+template <int LOGL, int P>
+__device__ __forceinline__ void odd_stage(Cx<float>* s, int j0, Cx<float>* v, const Cx<float>* __restrict__ tw) {
+  using F = Reg<LOGL, P>;
+  constexpr int G = F::G;
+  Cx<float> y[16];
+  dftr<16>(v, y);
+  const bool mir = j0 > 0 && 2 * j0 < G;               // columns 0 and G/2 are their own mirror images
+  const int a = padi(j0), b = padi(G - j0);
+  s[a] = y[0];
+  if (mir) s[b] = {-y[0].x, -y[0].y};
+#pragma unroll
+  for (int q = 1; q <= 8; ++q) {
+    const float2 w = __ldg(reinterpret_cast<const float2*>(tw) + (q - 1) * F::COLS + j0);
+    s[q * F::GP + a] = cmul(y[q], Cx<float>{w.x, w.y});
+    if (mir) {
+      const Cx<float> m = y[16 - q];
+      s[q * F::GP + b] = {-(m.x * w.x + m.y * w.y), m.x * w.y - m.y * w.x};
+    }
+  }
+}
 
 // One FP32 pass over the 2P lines b0 = 1 + 2 P bx ... of line family a = by + 1.
-// Offsets are 32-bit (grids up to 1025^3 nodes); each load/store item is one
-// complex pair (the same element of lines 2q and 2q+1).
-template <int LOGL, int P>
+// Offsets are 32-bit (grids up to 1025^3 nodes).
+template <int LOGL, int P, bool STR>
 __device__ __forceinline__ void dst32_body(const PassArgs& A, int bx, int by, Cx<float>* sm) {
   using F = Reg<LOGL, P>;
-  constexpr int L = F::L, LP = F::LP;
-  constexpr int n = L / 2, nm1 = n - 1;
-  if (A.zero_nrm && bx == 0 && by == 0 && threadIdx.x == 0) {
+  constexpr int n = F::N, nm1 = n - 1, G = F::G, T = F::T;
+  if (!STR && A.zero_nrm && bx == 0 && by == 0 && threadIdx.x == 0) {
     for (int k = 0; k < 7; ++k) A.zero_nrm[k] = 0ull;
     *A.zero_conv = 0;
   }
   const Cx<float>* tw = static_cast<const Cx<float>*>(A.twst);
   const int a = by + 1;
   const int b0 = 1 + 2 * P * bx;
-  const int sa = (int)A.sa, sb = (int)A.sb, es = (int)A.es;
+  const int sa = (int)A.sa, sb = STR ? 1 : (int)A.sb, es = STR ? (int)A.es : 1;
   const int abase = a * sa;
-  const bool contig = es == 1;
-  constexpr int nitem = nm1 * P;                      // (element, pair) items
-  constexpr int NIT = (nitem + F::THREADS - 1) / F::THREADS;
-  // contiguous lines: element fastest (coalesced along each line); strided
-  // lines: pair fastest (the 2P adjacent lines of a row together)
-  auto coords = [&](int t, int& j, int& q) {
-    if (contig) {
-      j = 1 + t % nm1;
-      q = t / nm1;
-    } else {
-      q = t % P;
-      j = 1 + t / P;
-    }
-  };
-  {
-    float2 vals[NIT];
+  const int t0 = threadIdx.x;
+  // the column of the first stage
+  const bool has = t0 < P * F::COLS;
+  const int c_pr = STR ? t0 % P : t0 / F::COLS, c_j = STR ? t0 / P : t0 % F::COLS;
+  Cx<float>* c_s = sm + c_pr * F::PP;
+  // the sequence of the later stages
+  constexpr int TS = G >= 16 ? G / 16 : 1;
+  const bool act = t0 < P * T;
+  const int f_pr = STR ? t0 % P : t0 / T, f_rem = STR ? t0 / P : t0 % T;
+  const int f_q = f_rem / TS, f_tid = f_rem % TS;
+  Cx<float>* f_s = sm + f_pr * F::PP + f_q * F::GP;
+  const Cx<float>* tw2 = tw + 8 * F::COLS;
+  auto keep = [&](int i, bool, Cx<float> y) { f_s[padi(i)] = y; };
+  if (has) {
+    const int bA = b0 + 2 * c_pr;
+    const bool okA = bA <= nm1, okB = bA + 1 <= nm1;
+    const int off = abase + bA * sb;
+    Cx<float> v[16];
+    // element j + G r, r < 8; -(G (16 - r) - j), r >= 8; 0 at both ends
+    auto fill = [&](auto* src) {
 #pragma unroll
-    for (int it = 0; it < NIT; ++it) {
-      const int t = threadIdx.x + it * F::THREADS;
-      int j, q;
-      coords(t < nitem ? t : 0, j, q);
-      const int bA = b0 + 2 * q;
-      const int off = abase + bA * sb + j * es;
-      float2 v = {0.f, 0.f};
-      if (t < nitem && bA <= nm1) {
-        if (A.src64) {
-          const double* src = static_cast<const double*>(A.src);
-          v.x = (float)__ldg(src + off);
-          if (bA + 1 <= nm1) v.y = (float)__ldg(src + off + sb);
-        } else {
-          const float* src = static_cast<const float*>(A.src);
-          v.x = __ldg(src + off);
-          if (bA + 1 <= nm1) v.y = __ldg(src + off + sb);
-        }
+      for (int r = 0; r < 16; ++r) {
+        const int j = r < 8 ? c_j + G * r : G * (16 - r) - c_j;
+        const bool in = (r != 0 || j > 0) && (r != 8 || j < n);
+        const int o = off + j * es;
+        const float x = (in && okA) ? (float)__ldg(src + o) : 0.f;
+        const float y = (in && okB) ? (float)__ldg(src + o + sb) : 0.f;
+        v[r] = r < 8 ? Cx<float>{x, y} : Cx<float>{-x, -y};
       }
-      vals[it] = v;
-    }
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) {
-      const int t = threadIdx.x + it * F::THREADS;
-      if (t < nitem) {
-        int j, q;
-        coords(t, j, q);
-        Cx<float>* zz = sm + q * LP;
-        zz[padi(j)] = {vals[it].x, vals[it].y};
-        zz[padi(L - j)] = {-vals[it].x, -vals[it].y};
-      }
-    }
-  }
-  for (int t = threadIdx.x; t < P; t += F::THREADS) {
-    sm[t * LP + padi(0)] = {0.f, 0.f};
-    sm[t * LP + padi(n)] = {0.f, 0.f};
+    };
+    if (!STR && A.src64) fill(static_cast<const double*>(A.src));
+    else fill(static_cast<const float*>(A.src));
+    odd_stage<LOGL, P>(c_s, c_j, v, tw);
   }
   __syncthreads();
-  const int pr = threadIdx.x / F::T, tid = threadIdx.x % F::T;
-  Cx<float>* s = sm + pr * LP;
-  reg_fft<LOGL>(s, tid, tw);
-  if (A.fused) {
-    // spectral division in place, then the same FFT gives the inverse
-    // transform.  lambda h^2 is affine in s_k along the line: alpha + beta s_k
-    // with alpha, beta fixed by the line's other mode indices.  Only k < n is
-    // divided; Z_{L-k} = -Z_k is written from it, so the rescaled sequence is
-    // exactly the odd extension of the next input.
-    const float kh2 = (float)A.kt, g = (float)A.gscale;
-    const int bA = b0 + 2 * pr, bB = min(bA + 1, nm1);
-    const float sa3 = A.d == 3 ? A.s32[a] : 0.f;
-    float alA, beA, alB, beB;
-    lam_affine(A.d, A.order, kh2, sa3, A.s32[min(bA, nm1)], alA, beA);
-    lam_affine(A.d, A.order, kh2, sa3, A.s32[bB], alB, beB);
-    const float gA = -0.5f * g, gB = 0.5f * g;
+  if (STR && A.fused) {
+    reg_fft<LOGL - 4, true>(act, f_s, f_tid, tw2, keep);
+    // spectral division of each mode on its way into the second transform's
+    // first stage.  lambda h^2 is affine in s_k along the line: alpha + beta
+    // s_k with alpha, beta fixed by the line's other mode indices.
+    Cx<float> v[16];
+    if (has) {
+      const float kh2 = (float)A.kt, g = (float)A.gscale;
+      const int bA = b0 + 2 * c_pr, bB = min(bA + 1, nm1);
+      const float sa3 = A.d == 3 ? A.s32[a] : 0.f;
+      float alA, beA, alB, beB;
+      lam_affine(A.d, A.order, kh2, sa3, A.s32[min(bA, nm1)], alA, beA);
+      lam_affine(A.d, A.order, kh2, sa3, A.s32[bB], alB, beB);
+      const float gA = -0.5f * g, gB = 0.5f * g;
 #pragma unroll
-    for (int i = 0; i < n / F::T; ++i) {
-      const int k = tid + i * F::T;
-      if (k == 0) {
-        s[padi(0)] = {0.f, 0.f};
-        s[padi(n)] = {0.f, 0.f};
-        continue;
+      for (int r = 0; r < 16; ++r) {
+        const int k = r < 8 ? c_j + G * r : G * (16 - r) - c_j;
+        if ((r != 0 || k > 0) && (r != 8 || k < n)) {
+          bool neg;
+          const Cx<float> Z = c_s[mode_at<LOGL, P>(k, neg)];
+          const float sk = __ldg(A.s32 + k);
+          const Cx<float> V = {__fdividef(gA, fmaf(beA, sk, alA)) * Z.y, __fdividef(gB, fmaf(beB, sk, alB)) * Z.x};
+          v[r] = (neg != (r >= 8)) ? Cx<float>{-V.x, -V.y} : V;
+        } else {
+          v[r] = {0.f, 0.f};
+        }
       }
-      const float sk = A.s32[k];
-      const Cx<float> Z = s[padi(k)];
-      const Cx<float> V = {__fdividef(gA, fmaf(beA, sk, alA)) * Z.y, __fdividef(gB, fmaf(beB, sk, alB)) * Z.x};
-      s[padi(k)] = V;
-      s[padi(L - k)] = {-V.x, -V.y};
     }
     __syncthreads();
-    reg_fft<LOGL>(s, tid, tw);
+    if (has) odd_stage<LOGL, P>(c_s, c_j, v, tw);
+    __syncthreads();
   }
-  // S_k = -Im(Z_k)/2 (line 2q), Re(Z_k)/2 (line 2q+1); in the accumulating
-  // modes all old values are loaded before the first store
-  float dmx = 0.f, umx = 0.f;
-  {
-    float2 vals[NIT];
-    int offs[NIT];
-    bool hasB[NIT];
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) {
-      const int t = threadIdx.x + it * F::THREADS;
-      int j, q;
-      coords(t < nitem ? t : 0, j, q);
-      const int bA = b0 + 2 * q;
-      offs[it] = (t < nitem && bA <= nm1) ? abase + bA * sb + j * es : -1;
-      hasB[it] = bA + 1 <= nm1;
-      const Cx<float> Z = sm[q * LP + padi(j)];
-      vals[it] = {-0.5f * Z.y, 0.5f * Z.x};
-    }
-    if (A.dstfix) {
-      long long oldA[NIT], oldB[NIT];
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        oldA[it] = offs[it] >= 0 ? A.dstfix[offs[it]] : 0ll;
-        oldB[it] = (offs[it] >= 0 && hasB[it]) ? A.dstfix[offs[it] + sb] : 0ll;
+  // S_k = -Im(Z_k)/2 (line 2q), Re(Z_k)/2 (line 2q+1)
+  if constexpr (STR) {
+    const int bA = b0 + 2 * f_pr;
+    const bool okA = bA <= nm1, okB = bA + 1 <= nm1;
+    float* o = static_cast<float*>(A.dst) + abase + bA;
+    const bool half = f_q == 0 || f_q == 8;            // modes below N only
+    auto store = [&](int i, bool up, Cx<float> y) {
+      int k = f_q + 16 * i;
+      float h = 0.5f;
+      if (up) {
+        k = F::L - k;
+        h = -0.5f;
       }
-      const float fa = A.fixf[0], fb = A.fixf[1], ia = A.fixf[2], ib = A.fixf[3];
-      const double isc = A.uout ? A.fixd[1] : 0.0;
-      // max|u| for the convergence check from the high words of u_fix alone
-      // (|u_fix| ~ 2^52, so to 2^-20 relative), converted once per thread
-      unsigned umi = 0u;
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        if (offs[it] >= 0) {
-          const long long nA = add64(oldA[it], f2ll((vals[it].x * fa) * fb));
-          A.dstfix[offs[it]] = nA;
-          if (A.uout) A.uout[offs[it]] = ll2d(nA) * isc;
-          dmx = fmax_nan(dmx, fabsf(vals[it].x));
-          umi = max(umi, (unsigned)abs((int)(nA >> 32)));
-          if (hasB[it]) {
-            const long long nB = add64(oldB[it], f2ll((vals[it].y * fa) * fb));
-            A.dstfix[offs[it] + sb] = nB;
-            if (A.uout) A.uout[offs[it] + sb] = ll2d(nB) * isc;
-            dmx = fmax_nan(dmx, fabsf(vals[it].y));
-            umi = max(umi, (unsigned)abs((int)(nB >> 32)));
-          }
-        }
-      }
-      umx = ((fmaf(u16f(umi >> 16), 65536.f, u16f(umi & 0xffffu)) * 4294967296.f) * ia) * ib;
-    } else if (A.dst64) {
-      double* o = static_cast<double*>(A.dst);
-      double oldA[NIT], oldB[NIT];
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        const bool acc = offs[it] >= 0 && A.accumulate;
-        oldA[it] = acc ? o[offs[it]] : 0.0;
-        oldB[it] = (acc && hasB[it]) ? o[offs[it] + sb] : 0.0;
-      }
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        if (offs[it] >= 0) {
-          const double nA = oldA[it] + (double)vals[it].x;
-          o[offs[it]] = nA;
-          dmx = fmax_nan(dmx, fabsf(vals[it].x));
-          umx = fmax_nan(umx, fabsf((float)nA));
-          if (hasB[it]) {
-            const double nB = oldB[it] + (double)vals[it].y;
-            o[offs[it] + sb] = nB;
-            dmx = fmax_nan(dmx, fabsf(vals[it].y));
-            umx = fmax_nan(umx, fabsf((float)nB));
-          }
-        }
-      }
+      if (up ? half : k == 0) return;
+      o[k * es] = -h * y.y;
+      if (okB) o[k * es + 1] = h * y.x;
+    };
+    if constexpr (G == 1) {
+      if (act && okA) store(0, f_q == 8, f_s[0]);
     } else {
-      float* o = static_cast<float*>(A.dst);
+      reg_fft<LOGL - 4, false>(act && okA, f_s, f_tid, tw2, store);
+    }
+    return;
+  } else {
+    reg_fft<LOGL - 4, true>(act, f_s, f_tid, tw2, keep);
+    // a few items (one mode of a pair) at a time; in the accumulating mode
+    // their old values are all loaded before the first store
+    float dmx = 0.f, umx = 0.f;
+    unsigned umi = 0u;
+    constexpr int nitem = n * P;
+    constexpr int NIT = (nitem + F::THREADS - 1) / F::THREADS;
+    constexpr int CH0 = P == 1 ? 8 : 4, CH = NIT < CH0 ? NIT : CH0;
+    float fa = 0.f, fb = 0.f;
+    double isc = 0.0;
+    if (A.dstfix) {
+      fa = A.fixf[0];
+      fb = A.fixf[1];
+      isc = A.uout ? A.fixd[1] : 0.0;
+    }
+#pragma unroll 1
+    for (int i0 = 0; i0 < NIT; i0 += CH) {
+      float2 vals[CH];
+      int offs[CH];
+      bool hasB[CH];
 #pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        if (offs[it] >= 0) {
-          o[offs[it]] = vals[it].x;
-          dmx = fmax_nan(dmx, fabsf(vals[it].x));
-          if (hasB[it]) {
-            o[offs[it] + sb] = vals[it].y;
-            dmx = fmax_nan(dmx, fabsf(vals[it].y));
+      for (int it = 0; it < CH; ++it) {
+        const int t = threadIdx.x + (i0 + it) * F::THREADS;
+        const bool in = t < nitem;
+        const int k = t & (n - 1), q = in ? t >> (LOGL - 1) : 0;
+        const int bA = b0 + 2 * q;
+        offs[it] = (in && k > 0 && bA <= nm1) ? abase + bA * sb + k : -1;
+        hasB[it] = bA + 1 <= nm1;
+        bool neg;
+        const Cx<float> Z = sm[q * F::PP + mode_at<LOGL, P>(k, neg)];
+        const float h = neg ? -0.5f : 0.5f;
+        vals[it] = {-h * Z.y, h * Z.x};
+      }
+      if (A.dstfix) {
+        long long oldA[CH], oldB[CH];
+#pragma unroll
+        for (int it = 0; it < CH; ++it) {
+          oldA[it] = offs[it] >= 0 ? A.dstfix[offs[it]] : 0ll;
+          oldB[it] = (offs[it] >= 0 && hasB[it]) ? A.dstfix[offs[it] + sb] : 0ll;
+        }
+        // max|u| for the convergence check from the high words of u_fix alone
+        // (|u_fix| ~ 2^52, so to 2^-20 relative), converted once per thread
+#pragma unroll
+        for (int it = 0; it < CH; ++it) {
+          if (offs[it] >= 0) {
+            const long long nA = add64(oldA[it], f2ll((vals[it].x * fa) * fb));
+            A.dstfix[offs[it]] = nA;
+            if (A.uout) A.uout[offs[it]] = ll2d(nA) * isc;
+            dmx = fmax_nan(dmx, fabsf(vals[it].x));
+            umi = max(umi, (unsigned)abs((int)(nA >> 32)));
+            if (hasB[it]) {
+              const long long nB = add64(oldB[it], f2ll((vals[it].y * fa) * fb));
+              A.dstfix[offs[it] + sb] = nB;
+              if (A.uout) A.uout[offs[it] + sb] = ll2d(nB) * isc;
+              dmx = fmax_nan(dmx, fabsf(vals[it].y));
+              umi = max(umi, (unsigned)abs((int)(nB >> 32)));
+            }
+          }
+        }
+      } else {
+        float* o = static_cast<float*>(A.dst);
+#pragma unroll
+        for (int it = 0; it < CH; ++it) {
+          if (offs[it] >= 0) {
+            o[offs[it]] = vals[it].x;
+            dmx = fmax_nan(dmx, fabsf(vals[it].x));
+            if (hasB[it]) {
+              o[offs[it] + sb] = vals[it].y;
+              dmx = fmax_nan(dmx, fabsf(vals[it].y));
+            }
           }
         }
       }
+    }
+    if (A.dstfix)
+      umx = ((fmaf(u16f(umi >> 16), 65536.f, u16f(umi & 0xffffu)) * 4294967296.f) * A.fixf[2]) * A.fixf[3];
+    else
       umx = dmx;
-    }
-  }
-  if (A.corr_max) {
-    for (int o = 16; o > 0; o >>= 1) {
-      dmx = fmax_nan(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
-      umx = fmax_nan(umx, __shfl_xor_sync(0xffffffffu, umx, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      if (!(dmx <= 0.f)) atomicMax(A.corr_max, (unsigned long long)__double_as_longlong((double)dmx));
-      if (!(umx <= 0.f)) atomicMax(A.corr_max + 1, (unsigned long long)__double_as_longlong((double)umx));
+    if (A.corr_max) {
+      for (int o = 16; o > 0; o >>= 1) {
+        dmx = fmax_nan(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+        umx = fmax_nan(umx, __shfl_xor_sync(0xffffffffu, umx, o));
+      }
+      if ((threadIdx.x & 31) == 0) {
+        if (!(dmx <= 0.f)) atomicMax(A.corr_max, (unsigned long long)__double_as_longlong((double)dmx));
+        if (!(umx <= 0.f)) atomicMax(A.corr_max + 1, (unsigned long long)__double_as_longlong((double)umx));
+      }
     }
   }
 }
 
-template <int LOGL, int P>
-__global__ void __launch_bounds__(Reg<LOGL, P>::THREADS) k_dst32(PassArgs A) {
+template <int LOGL, int P, bool STR>
+__global__ void __launch_bounds__(Reg<LOGL, P>::THREADS, Reg<LOGL, P>::MINB) k_dst32(PassArgs A) {
   if (A.skip && *A.skip) return;
   extern __shared__ unsigned char smraw[];
-  dst32_body<LOGL, P>(A, blockIdx.x, blockIdx.y, reinterpret_cast<Cx<float>*>(smraw));
+  dst32_body<LOGL, P, STR>(A, blockIdx.x, blockIdx.y, reinterpret_cast<Cx<float>*>(smraw));
 }
 
-// Each length compiled on its own (not inlined into the dispatching kernel, so
-// that the register allocation of one length does not spill another).
-template <int LOGL>
-__device__ __noinline__ void dst32_item(const PassArgs& A, int bx, int by, Cx<float>* sm) {
-  dst32_body<LOGL, reg_pairs(LOGL)>(A, bx, by, sm);
-}
+// Pairs per CTA: of the batched pass (all lengths in CTAs of one shape), of the
+// single passes over many line families (3D: 16 adjacent lines make 64-byte
+// segments; twice as many pairs measured 1880 against 1688 us at 256^3) and over
+// one (2D: as many CTAs as possible; strided passes two pairs, 16 bytes of
+// each sector: 1024^2 198 us, with one pair 219, with four 204).
+__host__ __device__ constexpr int batch_pairs(int logL) { return logL <= 8 ? 16 : 1 << (12 - logL); }
+__host__ __device__ constexpr int many_pairs(int logL) { return logL <= 8 ? 16 : logL >= 12 ? 1 : 1 << (12 - logL); }
+__host__ __device__ constexpr int few_pairs(int logL, bool str) { return str && logL < 13 ? 2 : 1; }
+
+constexpr int kBatchPassThreads = 160;
+constexpr size_t smax(size_t a, size_t b) { return a > b ? a : b; }
+constexpr size_t kBatchPassSmem =   // the largest of lengths up to 2048
+    smax(smax(Reg<8, batch_pairs(8)>::SMEM, Reg<9, batch_pairs(9)>::SMEM),
+         smax(Reg<10, batch_pairs(10)>::SMEM, Reg<11, batch_pairs(11)>::SMEM));
+static_assert(Reg<4, batch_pairs(4)>::THREADS == kBatchPassThreads && Reg<8, batch_pairs(8)>::THREADS == kBatchPassThreads &&
+              Reg<9, batch_pairs(9)>::THREADS == kBatchPassThreads && Reg<10, batch_pairs(10)>::THREADS == kBatchPassThreads &&
+              Reg<11, batch_pairs(11)>::THREADS == kBatchPassThreads, "one CTA shape for every length");
 
 // Persistent FP32 pass over many independent grids: every transform length
-// up to L = 2048 uses 128 threads and 17.4 KB per work item (P L / 16 = 128
-// with P = reg_pairs(LOGL)), so one kernel takes the work items of all
+// up to L = 2048 uses 160 threads and at most 20.2 KB per work item
+// (P = batch_pairs(LOGL)), so one kernel takes the work items of all
 // instances (item -> instance by binary search in `start`) and dispatches on
 // the instance's LOGL.
-__global__ void __launch_bounds__(128) k_dst32_batched(const PassArgs* __restrict__ args,
-                                                       const int* __restrict__ start, int ninst) {
+template <bool STR>
+__global__ void __launch_bounds__(kBatchPassThreads, STR ? 6 : 5)
+    k_dst32_batched(const PassArgs* __restrict__ args, const int* __restrict__ start, int ninst) {
   extern __shared__ unsigned char smraw[];
   Cx<float>* sm = reinterpret_cast<Cx<float>*>(smraw);
   const int total = start[ninst];
@@ -917,18 +984,18 @@ __global__ void __launch_bounds__(128) k_dst32_batched(const PassArgs* __restric
     const PassArgs& A = args[lo];
     if (A.skip && *A.skip) continue;
     const int local = item - start[lo];
-    const int p = reg_pairs(A.logL);
+    const int p = batch_pairs(A.logL);
     const int nbx = (A.n / 2 + p - 1) / p;
     const int bx = local % nbx, by = local / nbx;
     switch (A.logL) {
-      case 4: dst32_item<4>(A, bx, by, sm); break;
-      case 5: dst32_item<5>(A, bx, by, sm); break;
-      case 6: dst32_item<6>(A, bx, by, sm); break;
-      case 7: dst32_item<7>(A, bx, by, sm); break;
-      case 8: dst32_item<8>(A, bx, by, sm); break;
-      case 9: dst32_item<9>(A, bx, by, sm); break;
-      case 10: dst32_item<10>(A, bx, by, sm); break;
-      default: dst32_item<11>(A, bx, by, sm); break;
+      case 4: dst32_body<4, batch_pairs(4), STR>(A, bx, by, sm); break;
+      case 5: dst32_body<5, batch_pairs(5), STR>(A, bx, by, sm); break;
+      case 6: dst32_body<6, batch_pairs(6), STR>(A, bx, by, sm); break;
+      case 7: dst32_body<7, batch_pairs(7), STR>(A, bx, by, sm); break;
+      case 8: dst32_body<8, batch_pairs(8), STR>(A, bx, by, sm); break;
+      case 9: dst32_body<9, batch_pairs(9), STR>(A, bx, by, sm); break;
+      case 10: dst32_body<10, batch_pairs(10), STR>(A, bx, by, sm); break;
+      default: dst32_body<11, batch_pairs(11), STR>(A, bx, by, sm); break;
     }
     __syncthreads();
   }
@@ -1357,33 +1424,36 @@ void launch_pass_p(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cud
   KFBI_LAUNCH(p, KFBI_KC_DST, k_dst_pass<T, P><<<grid, 256, smem, st>>>(A));
 }
 
-template <int LOGL, int P>
+template <int LOGL, int P, bool STR>
 void launch_reg(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st) {
   using F = Reg<LOGL, P>;
   dim3 grid((unsigned)((npairs_b + P - 1) / P), (unsigned)na);
-  KFBI_LAUNCH(p, KFBI_KC_DST, k_dst32<LOGL, P><<<grid, F::THREADS, F::SMEM, st>>>(A));
-}
-
-// FP32 pass: P = reg_pairs(LOGL) line pairs per CTA (128-thread CTAs)
-void launch_pass32(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st) {
-  switch (A.logL) {
-    case 4: launch_reg<4, reg_pairs(4)>(p, A, npairs_b, na, st); break;
-    case 5: launch_reg<5, reg_pairs(5)>(p, A, npairs_b, na, st); break;
-    case 6: launch_reg<6, reg_pairs(6)>(p, A, npairs_b, na, st); break;
-    case 7: launch_reg<7, reg_pairs(7)>(p, A, npairs_b, na, st); break;
-    case 8: launch_reg<8, reg_pairs(8)>(p, A, npairs_b, na, st); break;
-    case 9: launch_reg<9, reg_pairs(9)>(p, A, npairs_b, na, st); break;
-    case 10: launch_reg<10, reg_pairs(10)>(p, A, npairs_b, na, st); break;
-    case 11: launch_reg<11, reg_pairs(11)>(p, A, npairs_b, na, st); break;
-    case 12: launch_reg<12, reg_pairs(12)>(p, A, npairs_b, na, st); break;
-    default: launch_reg<13, reg_pairs(13)>(p, A, npairs_b, na, st); break;
-  }
+  KFBI_LAUNCH(p, KFBI_KC_DST, k_dst32<LOGL, P, STR><<<grid, F::THREADS, F::SMEM, st>>>(A));
 }
 
 template <int LOGL>
-cudaError_t set_smem_reg(int max_optin) {
-  return cudaFuncSetAttribute(k_dst32<LOGL, reg_pairs(LOGL)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              max_optin);
+void launch_reg_l(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st) {
+  if (A.es == 1) {
+    if (na == 1) launch_reg<LOGL, few_pairs(LOGL, false), false>(p, A, npairs_b, na, st);
+    else launch_reg<LOGL, many_pairs(LOGL), false>(p, A, npairs_b, na, st);
+  } else {
+    if (na == 1) launch_reg<LOGL, few_pairs(LOGL, true), true>(p, A, npairs_b, na, st);
+    else launch_reg<LOGL, many_pairs(LOGL), true>(p, A, npairs_b, na, st);
+  }
+}
+void launch_pass32(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st) {
+  switch (A.logL) {
+    case 4: launch_reg_l<4>(p, A, npairs_b, na, st); break;
+    case 5: launch_reg_l<5>(p, A, npairs_b, na, st); break;
+    case 6: launch_reg_l<6>(p, A, npairs_b, na, st); break;
+    case 7: launch_reg_l<7>(p, A, npairs_b, na, st); break;
+    case 8: launch_reg_l<8>(p, A, npairs_b, na, st); break;
+    case 9: launch_reg_l<9>(p, A, npairs_b, na, st); break;
+    case 10: launch_reg_l<10>(p, A, npairs_b, na, st); break;
+    case 11: launch_reg_l<11>(p, A, npairs_b, na, st); break;
+    case 12: launch_reg_l<12>(p, A, npairs_b, na, st); break;
+    default: launch_reg_l<13>(p, A, npairs_b, na, st); break;
+  }
 }
 
 // The FP64 pass on the tensor cores (dst_mma.cuh), N = 64..1024; below and
@@ -1672,7 +1742,7 @@ kfbi_status box_create(kfbi_problem* p) {
   // shared memory per CTA: the FP64 passes hold two length-2N buffers per
   // line pair; the FP32 register passes one padded buffer per pair
   const size_t need = p->cfg.precision == KFBI_MIXED
-                          ? sizeof(Cx<float>) * (size_t)reg_pairs(B->logL) * (size_t)(2 * n + (2 * n) / 16)
+                          ? sizeof(Cx<float>) * (size_t)many_pairs(B->logL) * 9 * (size_t)(n / 8 + n / 128 + 1)
                           : sizeof(Cx<double>) * (size_t)(2 * n) * 2 * std::max(1, 1024 / (2 * n));
   if ((size_t)optin < need)
     return fail(p, KFBI_ERR_UNSUPPORTED,
@@ -1690,20 +1760,6 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, (set_smem_mma<8, 8>()));
   KFBI_CUDA(p, (set_smem_mma<9, 8>()));
   KFBI_CUDA(p, (set_smem_mma<10, 8>()));
-  KFBI_CUDA(p, (set_smem<float, 1>(optin)));
-  KFBI_CUDA(p, (set_smem<float, 2>(optin)));
-  KFBI_CUDA(p, (set_smem<float, 4>(optin)));
-  KFBI_CUDA(p, (set_smem<float, 8>(optin)));
-  KFBI_CUDA(p, set_smem_reg<4>(optin));
-  KFBI_CUDA(p, set_smem_reg<5>(optin));
-  KFBI_CUDA(p, set_smem_reg<6>(optin));
-  KFBI_CUDA(p, set_smem_reg<7>(optin));
-  KFBI_CUDA(p, set_smem_reg<8>(optin));
-  KFBI_CUDA(p, set_smem_reg<9>(optin));
-  KFBI_CUDA(p, set_smem_reg<10>(optin));
-  KFBI_CUDA(p, set_smem_reg<11>(optin));
-  KFBI_CUDA(p, set_smem_reg<12>(optin));
-  KFBI_CUDA(p, set_smem_reg<13>(optin));
   return KFBI_OK;
 }
 
@@ -2254,11 +2310,24 @@ struct BatchBox {
   int* dstart = nullptr;       // [ninst + 1] pass work items
   BoxDesc* dbox = nullptr;     // [ninst]
   int* drstart = nullptr;      // [ninst + 1] grid rows
-  int grid = 0, rgrid = 0;
+  bool str[5] = {};            // the pass's lines are strided
+  int grid = 0, rgrid = 0;     // CTAs of the contiguous passes and of the row kernels
+  int grid_s = 0;              // CTAs of the strided passes
+  int res_c = 0, res_s = 0;    // CTAs the GPU holds at once
 };
+
+void batch_launch_pass(kfbi_problem* p0, const BatchBox* bb, int v, const PassArgs* args, cudaStream_t st) {
+  if (bb->str[v])
+    KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<true><<<bb->grid_s, kBatchPassThreads, kBatchPassSmem, st>>>(
+        args, bb->dstart, bb->ninst));
+  else
+    KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<false><<<bb->grid, kBatchPassThreads, kBatchPassSmem, st>>>(
+        args, bb->dstart, bb->ninst));
+}
 
 void batch_box_copy_tiles(BatchBox* dst, const BatchBox* src) {
   dst->grid = src->grid;
+  dst->grid_s = src->grid_s;
   dst->rgrid = src->rgrid;
 }
 
@@ -2297,7 +2366,7 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
       last.fixf = B->fixf;
       last.corr_max = B->nrm + 3;
     }
-    const int pp = reg_pairs(B->logL);
+    const int pp = batch_pairs(B->logL);
     start[i + 1] = start[i] + ((plan0[i].npairs + pp - 1) / pp) * plan0[i].na;
     const int n1 = p->g.n + 1;
     rstart[i + 1] = rstart[i] + (d == 2 ? n1 : n1 * n1);
@@ -2323,9 +2392,14 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
   int dev = 0, sms = 0;
   KFBI_CUDA(p0, cudaGetDevice(&dev));
   KFBI_CUDA(p0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int per_sm = 0;
-  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dst32_batched, 128, Reg<11, 1>::SMEM));
-  bb->grid = sms * std::max(1, per_sm);
+  int per_c = 0, per_s = 0;
+  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_c, k_dst32_batched<false>, kBatchPassThreads,
+                                                              kBatchPassSmem));
+  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_s, k_dst32_batched<true>, kBatchPassThreads,
+                                                              kBatchPassSmem));
+  bb->grid = bb->res_c = sms * std::max(1, per_c);
+  bb->grid_s = bb->res_s = sms * std::max(1, per_s);
+  for (int v = 0; v < bb->npass; ++v) bb->str[v] = plan0[0].args[v].es != 1;
   bb->rgrid = sms * 8;
   return KFBI_OK;
 }
@@ -2368,12 +2442,13 @@ kfbi_status batch_box_autotune(kfbi_problem* p0, BatchBox* bb, kfbi_problem* con
     KFBI_CUDA(p0, cudaEventElapsedTime(ms, e0, e1));
     return KFBI_OK;
   };
-  const int resident = bb->grid;   // batch_box_create: SMs x resident CTAs per SM
+  const int resident = bb->res_c;
   kfbi_status s = KFBI_OK;
   float best = 1e30f;
   int best_grid = resident;
   for (int g : {std::max(1, resident / 2), resident, 2 * resident}) {
     bb->grid = g;
+    bb->grid_s = std::max(1, (int)((long long)g * bb->res_s / bb->res_c));
     float ms = 0.f;
     if ((s = time_solve(&ms)) != KFBI_OK) break;
     if (ms < best) {
@@ -2382,6 +2457,7 @@ kfbi_status batch_box_autotune(kfbi_problem* p0, BatchBox* bb, kfbi_problem* con
     }
   }
   bb->grid = best_grid;
+  bb->grid_s = std::max(1, (int)((long long)best_grid * bb->res_s / bb->res_c));
   best = 1e30f;
   int best_rgrid = 8 * sms;
   for (int per : {4, 8, 16, 32}) {
@@ -2421,20 +2497,17 @@ void batch_box_destroy(BatchBox* bb) {
 // mixed-precision steps of box_solve, every step one launch over all instances.
 kfbi_status batch_box_solve(kfbi_problem* p0, BatchBox* bb, const int* done, cudaStream_t st) {
   const int ni = bb->ninst;
-  const size_t smem = Reg<11, 1>::SMEM;
   const int cb = div_up(ni, 128);
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_zero_batched<<<cb, 128, 0, st>>>(bb->dbox, ni, done));
   for (int v = 0; v < bb->npass; ++v)
-    KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<<<bb->grid, 128, smem, st>>>(bb->dargs + (size_t)v * ni,
-                                                                               bb->dstart, ni));
+    batch_launch_pass(p0, bb, v, bb->dargs + (size_t)v * ni, st);
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_check_batched<<<cb, 128, 0, st>>>(bb->dbox, ni, 0));
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_fix_scale_batched<<<cb, 128, 0, st>>>(bb->dbox, ni));
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 0));
   for (int it = 1; it < bb->steps; ++it) {
     KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 1));
     for (int v = 0; v < bb->npass; ++v)
-      KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<<<bb->grid, 128, smem, st>>>(
-          bb->dargs + (size_t)(bb->npass + v) * ni, bb->dstart, ni));
+      batch_launch_pass(p0, bb, v, bb->dargs + (size_t)(bb->npass + v) * ni, st);
     KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_check_batched<<<cb, 128, 0, st>>>(bb->dbox, ni, it));
   }
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 2));
