@@ -48,6 +48,9 @@ struct Cx {
   T x, y;
 };
 
+constexpr int kMaxSteps = 8;             // FP32 solves of a mixed box solve, at most
+constexpr int kNrm = 9 + 2 * kMaxSteps;  // entries of BoxSolver::nrm
+
 struct BoxSolver {
   int L = 0, logL = 0;
   double* tw64 = nullptr;     // L/2 twiddles exp(-2 pi i t / L)
@@ -62,8 +65,9 @@ struct BoxSolver {
   float* work32 = nullptr;    // grid of floats
   double* res = nullptr;      // FP64 residual grid
   unsigned long long* nrm = nullptr;   // [0] max|R| [1] max|r| [2] last max|delta| [3] max|delta| [4] max|u| [5] last max|u|
-                                       // [6] correction steps of the last solve, [7] of all solves since reset,
-                                       // [8] relative size of the last first correction (FP32 error estimate)
+                                       // ([3], [4]: the batched solve), [6] correction steps of the last solve, [7] of all
+                                       // solves since reset, [8] relative size of the last first correction (FP32 error
+                                       // estimate), [9 + 2 s], [10 + 2 s] max|delta|, max|u| of step s
   double* tol_dev = nullptr;  // the refinement tolerance the checks read (relaxed inside GMRES)
   int* conv = nullptr;        // device flag
   int refine_steps = 4;
@@ -107,7 +111,7 @@ struct PassArgs {
   const float* fixf;              // [0..1] 2^Fa, 2^Fb; [2..3] 2^-Fa, 2^-Fb (k_fix_scale)
   const double* fixd;             // [1] mult h^2 2^-F (with uout)
   double* uout;                   // with dstfix: also u = u_fix mult h^2 2^-F in FP64
-  unsigned long long* zero_nrm;   // first pass of a mixed solve: CTA 0 clears nrm[0..6] and
+  unsigned long long* zero_nrm;   // first pass of a mixed solve: CTA 0 clears nrm (but [7], [8]) and
   int* zero_conv;                 // the convergence flag before anything reads them
 };
 
@@ -749,7 +753,8 @@ __device__ __forceinline__ void dst32_body(const PassArgs& A, int bx, int by, Cx
   using F = Reg<LOGL, P>;
   constexpr int n = F::N, nm1 = n - 1, G = F::G, T = F::T;
   if (!STR && A.zero_nrm && bx == 0 && by == 0 && threadIdx.x == 0) {
-    for (int k = 0; k < 7; ++k) A.zero_nrm[k] = 0ull;
+    for (int k = 0; k < kNrm; ++k)
+      if (k != 7 && k != 8) A.zero_nrm[k] = 0ull;
     *A.zero_conv = 0;
   }
   const Cx<float>* tw = static_cast<const Cx<float>*>(A.twst);
@@ -1008,30 +1013,43 @@ __global__ void __launch_bounds__(kBatchPassThreads, STR ? 6 : 5)
 // an estimate of the FP32 solve's error, 1 until one is observed) is within
 // tol, which a relaxed GMRES tolerance can reach.  The first correction of
 // every solve updates that estimate.
-__device__ __forceinline__ void check_body(unsigned long long* nrm, const double* tolp, int* conv, int step) {
-  const double tol = tolp[0];
-  if (*conv) return;
-  double dm = __longlong_as_double((long long)nrm[3]);
-  double um = __longlong_as_double((long long)nrm[4]);
-  nrm[2] = nrm[3];
-  nrm[5] = nrm[4];
+// The kernel after the step (the next residual) decides: every CTA from the
+// step's own maxima, so that no launch of one thread stands between them (19
+// launches instead of 24 with the scale in k_fix0, five steps enqueued: 1024^2
+// 198 -> 177 us, 64^2 121 -> 109); its first thread keeps the records.
+struct StepCheck {
+  unsigned long long* nrm;
+  const double* tol;
+  int* conv;
+  int step;        // the step to check
+};
+
+// whether the refinement is over at this check (or was before)
+__device__ __forceinline__ bool step_stop(const StepCheck& C, bool keeper) {
+  const int done = *C.conv;
+  const unsigned long long* slot = C.nrm + 9 + 2 * C.step;
+  const unsigned long long db = slot[0], ub = slot[1], eb = C.nrm[8];
+  const double tol = C.tol[0];
+  if (done) return true;
+  const double dm = __longlong_as_double((long long)db), um = __longlong_as_double((long long)ub);
   bool stop = dm <= tol * um;
-  if (step == 0 && 10.0 * __longlong_as_double((long long)nrm[8]) <= tol) stop = true;
-  if (step == 1 && um > 0.0) nrm[8] = (unsigned long long)__double_as_longlong(dm / um);
-  if (stop) {
-    *conv = 1;
-  } else {
-    nrm[6] += 1ull;   // one more refinement step will run
-    nrm[7] += 1ull;
+  if (C.step == 0 && 10.0 * __longlong_as_double((long long)eb) <= tol) stop = true;
+  if (keeper) {
+    C.nrm[2] = db;
+    C.nrm[5] = ub;
+    if (C.step == 1 && um > 0.0) C.nrm[8] = (unsigned long long)__double_as_longlong(dm / um);
+    if (stop) {
+      *C.conv = 1;
+    } else {
+      C.nrm[6] += 1ull;   // one more refinement step will run
+      C.nrm[7] += 1ull;
+    }
   }
-  nrm[3] = 0ull;
-  nrm[4] = 0ull;
+  return stop;
 }
 
-__global__ void k_check(unsigned long long* nrm, const double* tol, int* conv, int step) {
-  check_body(nrm, tol, conv, step);
-}
-
+// the check alone (a solve without refinement steps)
+__global__ void k_check(StepCheck C) { step_stop(C, true); }
 
 // ---- exact residual of the mixed path (fixed point) -------------------------
 // After the first FP32 solve u0, F is chosen so that max|u0| 2^F ~ 2^52; then
@@ -1042,71 +1060,100 @@ __global__ void k_check(unsigned long long* nrm, const double* tol, int* conv, i
 // FP64 stencil arithmetic, and is handed to the next FP32 solve as FP32.
 // Scales beyond the FP32 exponent range are applied as two factors
 // 2^Fa 2^Fb (Fa + Fb = F).
-__device__ __forceinline__ void fix_scale_body(const unsigned long long* __restrict__ umax, double multh2,
-                                               double kc, double* __restrict__ fixd, float* __restrict__ fixf) {
+struct FixScale {
+  int F;
+  double isc;      // u = U isc
+  float f[5];      // fixf
+};
+
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }
+
+__device__ __forceinline__ FixScale fix_scale_of(unsigned long long umax, double multh2, double inv_multh2) {
   // U = u 2^F / (mult h^2) with max|U| ~ 2^52; R_fix = R 2^F (an exact power of two)
-  const double um = __longlong_as_double((long long)umax[0]) / multh2;
-  int F = 0;
-  if (um > 0.0) F = 52 - (int)ceil(log2(um));
-  F = max(-120, min(F, 240));
-  const int Fa = F / 2, Fb = F - Fa;
-  fixd[1] = ldexp(multh2, -F);                  // u = U mult h^2 2^-F
-  fixd[2] = kc;
-  fixd[3] = (double)F;
-  fixf[0] = ldexpf(1.f, Fa);                    // U = (u 2^Fa) (2^Fb / mult h^2)
-  fixf[1] = (float)(ldexp(1.0, Fb) / multh2);
-  fixf[2] = ldexpf(1.f, -Fa);                   // u = (U 2^-Fa) (mult h^2 2^-Fb); r = (r_fix 2^-Fa) 2^-Fb
-  fixf[3] = (float)ldexp(multh2, -Fb);
-  fixf[4] = ldexpf(1.f, -Fb);
+  const double um = __longlong_as_double((long long)umax) * inv_multh2;
+  FixScale s;
+  s.F = 0;
+  if (um > 0.0) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(um);
+    s.F = 52 - ((int)((b >> 52) & 0x7ff) - 1023 + ((b & 0xfffffffffffffull) != 0ull));   // ceil(log2 um)
+  }
+  s.F = max(-120, min(s.F, 240));
+  const int Fa = s.F / 2, Fb = s.F - Fa;
+  s.isc = multh2 * pow2d(-s.F);                       // u = U mult h^2 2^-F
+  s.f[0] = pow2f(Fa);                                 // U = (u 2^Fa) (2^Fb / mult h^2)
+  s.f[1] = (float)(pow2d(Fb) * inv_multh2);
+  s.f[2] = pow2f(-Fa);                                // u = (U 2^-Fa) (mult h^2 2^-Fb); r = (r_fix 2^-Fa) 2^-Fb
+  s.f[3] = (float)(multh2 * pow2d(-Fb));
+  s.f[4] = pow2f(-Fb);
   if (!(um <= 1.7976931348623157e308)) {
     // a NaN or infinite first solve (non-finite data): the integer
     // conversions would turn it into finite values, so every conversion back
     // to floating point yields NaN instead and the caller sees a non-finite
     // result
-    const double qn = __longlong_as_double(0x7ff8000000000000LL);
-    fixd[1] = qn;
-    fixf[2] = __int_as_float(0x7fc00000);
-    fixf[3] = __int_as_float(0x7fc00000);
-    fixf[4] = __int_as_float(0x7fc00000);
+    s.isc = __longlong_as_double(0x7ff8000000000000LL);
+    s.f[2] = s.f[3] = s.f[4] = __int_as_float(0x7fc00000);
   }
+  return s;
 }
 
-__global__ void k_fix_scale(const unsigned long long* __restrict__ umax, double multh2, double kc,
-                            double* __restrict__ fixd, float* __restrict__ fixf) {
-  fix_scale_body(umax, multh2, kc, fixd, fixf);
+__device__ __forceinline__ void fix_scale_store(const FixScale& s, double kc, double* __restrict__ fixd,
+                                                float* __restrict__ fixf) {
+  fixd[1] = s.isc;
+  fixd[2] = kc;
+  fixd[3] = (double)s.F;
+  for (int k = 0; k < 5; ++k) fixf[k] = s.f[k];
 }
 
-// the check after the first FP32 solve and the fixed-point scale from its max|u|
-__global__ void k_check_scale(unsigned long long* nrm, const double* tol, int* conv, double multh2, double kc,
-                              double* __restrict__ fixd, float* __restrict__ fixf) {
-  check_body(nrm, tol, conv, 0);
-  fix_scale_body(nrm + 5, multh2, kc, fixd, fixf);
-}
-
-// u_fix = round(u0 2^F / (mult h^2)), R_fix = round(R 2^F); with u, also the
-// FP64 solution of the fixed-point u_fix (u0 is 0 on the boundary layer)
-__global__ void k_fix0(long long tot, const float* __restrict__ u0, const double* __restrict__ R, Grid g,
-                       const double* __restrict__ fixd, const float* __restrict__ fixf,
-                       long long* __restrict__ ufix, long long* __restrict__ rfix, double* __restrict__ u) {
-  const int F = (int)fixd[3];
-  const double isc = fixd[1];
-  const float fa = fixf[0], fb = fixf[1];
-  const int n1 = g.n + 1;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < (int)tot;
-       t += gridDim.x * blockDim.x) {
-    const long long uf = f2ll((u0[t] * fa) * fb);
+// The fixed-point scale from max|u0|, u_fix = round(u0 2^F / (mult h^2)),
+// R_fix = round(R 2^F); with u, also the FP64 solution of the fixed-point u_fix
+// (u0 is 0 on the boundary layer).  Every CTA derives the scale itself (a few
+// integer operations on the exponent; no launch of its own), the first writes
+// it for the later kernels.  A CTA takes kFixRows rows of 128 columns, all
+// their loads in flight together.
+constexpr int kFixRows = 8;
+__global__ void __launch_bounds__(128) k_fix0(Grid g, int rows, const float* __restrict__ u0,
+                                              const double* __restrict__ R,
+                                              const unsigned long long* __restrict__ umax, double multh2,
+                                              double inv_multh2, double kc, double* __restrict__ fixd,
+                                              float* __restrict__ fixf, long long* __restrict__ ufix,
+                                              long long* __restrict__ rfix, double* __restrict__ u) {
+  const int n = g.n, n1 = n + 1;
+  const int j = blockIdx.x * 128 + threadIdx.x;
+  const int r0 = blockIdx.y * kFixRows;
+  const bool in_j = j >= 1 && j < n;
+  float uv[kFixRows];
+  double rv[kFixRows];
+#pragma unroll
+  for (int k = 0; k < kFixRows; ++k) {
+    const bool ok = j <= n && r0 + k < rows;
+    uv[k] = ok ? u0[(r0 + k) * n1 + j] : 0.f;
+    rv[k] = ok && in_j ? R[(r0 + k) * n1 + j] : 0.0;
+  }
+  const FixScale s = fix_scale_of(umax[0], multh2, inv_multh2);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) fix_scale_store(s, kc, fixd, fixf);
+  if (j > n) return;
+#pragma unroll
+  for (int k = 0; k < kFixRows; ++k) {
+    const int r = r0 + k;
+    if (r >= rows) break;
+    const int i1 = g.d == 2 ? r : r % n1, i0 = g.d == 2 ? 1 : r / n1;
+    const bool interior = in_j && i1 >= 1 && i1 < n && i0 >= 1 && i0 < n;
+    const int t = r * n1 + j;
+    const long long uf = f2ll((uv[k] * s.f[0]) * s.f[1]);
     ufix[t] = uf;
-    if (u) u[t] = ll2d(uf) * isc;
-    int r = t;
-    bool interior = true;
-    for (int k = 0; k < g.d; ++k) {
-      const int q = r / n1;
-      const int i = r - q * n1;
-      r = q;
-      interior = interior && i >= 1 && i < g.n;
-    }
-    rfix[t] = interior ? d2ll_pow2(R[t], F) : 0ll;
+    if (u) u[t] = ll2d(uf) * s.isc;
+    rfix[t] = interior ? d2ll_pow2(rv[k], s.F) : 0ll;
   }
+}
+
+void launch_fix0(kfbi_problem* p, const Grid& g, const float* u0, const double* R, const unsigned long long* umax,
+                 double multh2, double kc, double* fixd, float* fixf, long long* ufix, long long* rfix, double* u,
+                 cudaStream_t st) {
+  const int rows = (int)(g.nodes() / (g.n + 1));
+  const dim3 grid((unsigned)div_up(g.n + 1, 128), (unsigned)div_up(rows, kFixRows));
+  KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_fix0<<<grid, 128, 0, st>>>(g, rows, u0, R, umax, multh2, 1.0 / multh2, kc,
+                                                                fixd, fixf, ufix, rfix, u));
 }
 
 struct FixStencil {
@@ -1205,12 +1252,12 @@ __device__ __forceinline__ long long kappa_int(const KappaFix& f, long long m) {
 constexpr int kResRows = 4;
 __global__ void k_res_fix2(Grid g, FixStencil W, const long long* __restrict__ R, const long long* __restrict__ u,
                            const double* __restrict__ fixd, const float* __restrict__ fixf,
-                           float* __restrict__ r32, const int* skip, double* __restrict__ uout) {
+                           float* __restrict__ r32, const int* skip, double* __restrict__ uout, StepCheck chk) {
   const int n = g.n, n1 = n + 1;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > n) return;
   const int i0 = blockIdx.y * kResRows, i1 = min(n1, i0 + kResRows);
-  if (skip && *skip) {
+  if (chk.nrm ? step_stop(chk, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) : (skip && *skip)) {
     if (uout)
       for (int i = i0; i < i1; ++i) uout[i * n1 + j] = ll2d(u[i * n1 + j]) * fixd[1];
     return;
@@ -1257,13 +1304,15 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
                                                             const long long* __restrict__ u,
                                                             const double* __restrict__ fixd,
                                                             const float* __restrict__ fixf, float* __restrict__ r32,
-                                                            const int* skip, double* __restrict__ uout, int kz) {
+                                                            const int* skip, double* __restrict__ uout, int kz,
+                                                            StepCheck chk) {
   const int n = g.n, n1 = n + 1, plane = n1 * n1;
   const int x = blockIdx.x * kR3X + (threadIdx.x % kR3X);
   const int yb = blockIdx.y * (kR3Y * kR3) + (threadIdx.x / kR3X) * kR3;
   if (x > n || yb > n) return;
   const int z0 = blockIdx.z * kz, z1 = min(n1, z0 + kz);
-  if (skip && *skip) {
+  const bool keeper = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0;
+  if (chk.nrm ? step_stop(chk, keeper) : (skip && *skip)) {
     if (uout) {
       const double isc = fixd[1];
       for (int z = z0; z < z1; ++z)
@@ -1357,16 +1406,17 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
 // launch of the fixed-point residual for the grid's dimension
 void launch_res_fix(kfbi_problem* p, const Grid& g, const FixStencil& W, const long long* R, const long long* u,
                     const double* fixd, const float* fixf, float* r32, const int* skip, double* uout,
-                    cudaStream_t st) {
+                    cudaStream_t st, const StepCheck& chk = StepCheck{nullptr, nullptr, nullptr, 0}) {
   if (g.d == 2) {
     const dim3 grid((unsigned)div_up(g.n + 1, 128), (unsigned)div_up(g.n + 1, kResRows), 1u);
-    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_res_fix2<<<grid, 128, 0, st>>>(g, W, R, u, fixd, fixf, r32, skip, uout));
+    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_res_fix2<<<grid, 128, 0, st>>>(g, W, R, u, fixd, fixf, r32, skip, uout,
+                                                                       chk));
   } else {
     const int kz = 16;
     const dim3 grid((unsigned)div_up(g.n + 1, kR3X), (unsigned)div_up(g.n + 1, kR3Y * kR3),
                     (unsigned)div_up(g.n + 1, kz));
     KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_res_fix3<<<grid, kR3Threads, 0, st>>>(g, W, R, u, fixd, fixf, r32, skip,
-                                                                               uout, kz));
+                                                                               uout, kz, chk));
   }
 }
 
@@ -1724,9 +1774,9 @@ kfbi_status box_create(kfbi_problem* p) {
     }
     KFBI_CUDA(p, cudaDeviceSynchronize());
   }
-  KFBI_CUDA(p, dalloc(&B->nrm, 9));
+  KFBI_CUDA(p, dalloc(&B->nrm, kNrm));
   {
-    unsigned long long init[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    unsigned long long init[kNrm] = {};
     const double one = 1.0;   // no FP32 error estimate yet
     memcpy(&init[8], &one, sizeof(one));
     KFBI_CUDA(p, cudaMemcpy(B->nrm, init, sizeof(init), cudaMemcpyHostToDevice));
@@ -1735,7 +1785,7 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, dalloc(&B->tol_dev, 1));
   B->tol = p->cfg.box_rtol > 0 ? p->cfg.box_rtol : 1e-13;
   KFBI_CUDA(p, cudaMemcpy(B->tol_dev, &B->tol, sizeof(double), cudaMemcpyHostToDevice));
-  B->refine_steps = p->cfg.box_max_iters > 0 ? std::min(p->cfg.box_max_iters, 8) : 5;
+  B->refine_steps = p->cfg.box_max_iters > 0 ? std::min(p->cfg.box_max_iters, kMaxSteps) : 5;
   int dev = 0, optin = 0;
   KFBI_CUDA(p, cudaGetDevice(&dev));
   KFBI_CUDA(p, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -1844,29 +1894,28 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   // output u is written once: by the last step's final pass, or, when the
   // convergence flag stops the refinement earlier, by the next residual
   // kernel in place of its skipped step (by the conversion kernel when there
-  // is no refinement step).  The check of the last step is left to the
-  // host-side diagnostics (box_last_residual), which read its maxima.
+  // is no refinement step).  Each step has its own maxima, which the next
+  // residual kernel checks (step_stop); the check of the last step is left to
+  // the host-side diagnostics (box_last_residual).
   cudaStream_t st = p->stream;
-  const long long nodes = g.nodes();
-  const int eb = (int)std::min<long long>(div_up(nodes, 256), 152 * 8);
+  unsigned long long* slot = B->nrm + 9;   // step s: slot + 2 s
   {
-    PassPlan P0 = plan_passes<float>(p, rhs, 1, u, 0, nullptr, B->nrm + 3);
+    PassPlan P0 = plan_passes<float>(p, rhs, 1, u, 0, nullptr, slot);
     P0.args[0].zero_nrm = B->nrm;
     P0.args[0].zero_conv = B->conv;
     PassArgs& last = P0.args[P0.npass - 1];
     last.dst = B->work32;
     last.dst64 = 0;
     last.accumulate = 0;
-    last.corr_max = B->nrm + 3;
+    last.corr_max = slot;
     for (int k = 0; k < P0.npass; ++k) launch_pass<float>(p, P0.args[k], P0.npairs, P0.na, st, P0.pmin[k]);
   }
-  KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check_scale<<<1, 1, 0, st>>>(B->nrm, B->tol_dev, B->conv, B->multh2, B->kc,
-                                                                      B->fixd, B->fixf));
-  KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_fix0<<<eb, 256, 0, st>>>(nodes, B->work32, rhs, g, B->fixd, B->fixf,
-                                                                 B->ufix, B->rfix,
-                                                                 B->refine_steps > 1 ? nullptr : u));
+  launch_fix0(p, g, B->work32, rhs, slot + 1, B->multh2, B->kc, B->fixd, B->fixf, B->ufix, B->rfix,
+              B->refine_steps > 1 ? nullptr : u, st);
+  if (B->refine_steps == 1)
+    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, 0}));
   float* r32 = reinterpret_cast<float*>(B->res);
-  PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, B->nrm + 3);
+  PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, nullptr);
   {
     PassArgs& last = PK.args[PK.npass - 1];
     last.dst = nullptr;
@@ -1875,17 +1924,15 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
     last.dstfix = B->ufix;
     last.fixf = B->fixf;
     last.fixd = B->fixd;
-    last.corr_max = B->nrm + 3;
   }
-  PassPlan PL = PK;   // the last step's final pass also writes the FP64 solution
-  PL.args[PL.npass - 1].uout = u;
   const FixStencil W{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB};
   for (int it = 1; it < B->refine_steps; ++it) {
-    launch_res_fix(p, g, W, B->rfix, B->ufix, B->fixd, B->fixf, r32, B->conv, u, st);
-    const PassPlan& P = it + 1 < B->refine_steps ? PK : PL;
-    for (int k = 0; k < P.npass; ++k) launch_pass<float>(p, P.args[k], P.npairs, P.na, st, P.pmin[k]);
-    if (it + 1 < B->refine_steps)
-      KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(B->nrm, B->tol_dev, B->conv, it));
+    launch_res_fix(p, g, W, B->rfix, B->ufix, B->fixd, B->fixf, r32, B->conv, u, st,
+                   StepCheck{B->nrm, B->tol_dev, B->conv, it - 1});
+    PassArgs& last = PK.args[PK.npass - 1];
+    last.corr_max = slot + 2 * it;
+    last.uout = it + 1 < B->refine_steps ? nullptr : u;   // the last step also writes the FP64 solution
+    for (int k = 0; k < PK.npass; ++k) launch_pass<float>(p, PK.args[k], PK.npairs, PK.na, st, PK.pmin[k]);
   }
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
@@ -1947,9 +1994,7 @@ kfbi_status fix_init(kfbi_problem* p, FixState* F, const float* u0, const double
   const int eb = (int)std::min<long long>(div_up(nodes, 256), 152 * 8);
   KFBI_CUDA(p, cudaMemsetAsync(F->umax, 0, sizeof(unsigned long long), st));
   KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_absmax32<<<eb, 256, 0, st>>>(nodes, u0, F->umax, nullptr));
-  KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_fix_scale<<<1, 1, 0, st>>>(F->umax, F->multh2, F->kc, F->fixd, F->fixf));
-  KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_fix0<<<eb, 256, 0, st>>>(nodes, u0, R, p->g, F->fixd, F->fixf, F->ufix,
-                                                                 F->rfix, nullptr));
+  launch_fix0(p, p->g, u0, R, F->umax, F->multh2, F->kc, F->fixd, F->fixf, F->ufix, F->rfix, nullptr, st);
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
 }
@@ -2000,7 +2045,7 @@ kfbi_status box_steps(kfbi_problem* p, int* steps, int* cycles) {
 kfbi_status box_last_residual(kfbi_problem* p, double* rel, int* converged) {
   if (p->mg) return mg_last_residual(p, rel, converged);
   BoxSolver* B = p->box;
-  unsigned long long h[6] = {0, 0, 0, 0, 0, 0};
+  unsigned long long h[kNrm] = {};
   int c = 1;
   if (p->cfg.precision == KFBI_MIXED) {
     KFBI_CUDA(p, cudaMemcpyAsync(h, B->nrm, sizeof(h), cudaMemcpyDeviceToHost, p->stream));
@@ -2008,11 +2053,12 @@ kfbi_status box_last_residual(kfbi_problem* p, double* rel, int* converged) {
     KFBI_CUDA(p, cudaStreamSynchronize(p->stream));
   }
   // the device checks every step but the last: with the flag unset after
-  // more than one step, the last step's maxima are still in h[3], h[4]
+  // more than one step, the last step's maxima count
   double dm, um;
   const bool last_open = p->cfg.precision == KFBI_MIXED && !c && B->refine_steps > 1;
-  memcpy(&dm, &h[last_open ? 3 : 2], 8);
-  memcpy(&um, &h[last_open ? 4 : 5], 8);
+  const int open = 9 + 2 * (B->refine_steps - 1);
+  memcpy(&dm, &h[last_open ? open : 2], 8);
+  memcpy(&um, &h[last_open ? open + 1 : 5], 8);
   if (last_open) c = dm <= B->tol * um ? 1 : 0;
   *rel = um > 0 ? dm / um : 0.0;
   *converged = c;
@@ -2254,7 +2300,7 @@ __global__ void k_check_batched(const BoxDesc* __restrict__ D, int ninst, int st
 __global__ void k_fix_scale_batched(const BoxDesc* __restrict__ D, int ninst) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ninst) return;
-  fix_scale_body(D[i].nrm + 5, D[i].multh2, D[i].kc, D[i].fixd, D[i].fixf);
+  fix_scale_store(fix_scale_of(D[i].nrm[5], D[i].multh2, 1.0 / D[i].multh2), D[i].kc, D[i].fixd, D[i].fixf);
 }
 
 // grid kernels over all instances' rows (one row of the last axis per item);
