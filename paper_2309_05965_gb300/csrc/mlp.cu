@@ -47,7 +47,6 @@ struct kfbi_mlp {
   float* d1 = nullptr;    // back-propagated signals [cap][width]
   float* d2 = nullptr;
   float* y = nullptr;     // [cap]
-  float* dy = nullptr;
   float* tb = nullptr;    // gathered targets [cap]
   float* loss = nullptr;  // [1]
 };
@@ -66,28 +65,113 @@ kfbi_status mfail(kfbi_mlp* m, kfbi_status s, const std::string& msg) {
     if (e_ != cudaSuccess) return mfail((m), KFBI_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-template <typename T>
-__device__ __forceinline__ float tof(T v);
-template <>
-__device__ __forceinline__ float tof<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float tof<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-
 // ---- tensor-core GEMM: mma.sync m16n8k16, bf16 operands, FP32 accumulation --
 // An FP32 operand enters as a sum of bfloat16 parts, x = hi + mid + lo with
 // each part the bf16 rounding of what the previous parts leave; every product
 // of two bf16 values is exact in FP32, so three parts carry an FP32 value's
 // 24 bits.  Weights already rounded to bf16 are one exact part.
-__device__ __forceinline__ void split3(float x, __nv_bfloat16& h, __nv_bfloat16& m, __nv_bfloat16& l) {
-  h = __float2bfloat16_rn(x);
-  const float r = x - __bfloat162float(h);
-  m = __float2bfloat16_rn(r);
-  l = __float2bfloat16_rn(r - __bfloat162float(m));
+//
+// C (M x N) = A (M x K) B (K x N), 64 x 64 tiles, four warps of 32 x 32 (2 x 4
+// mma tiles), K in steps of 32; blockIdx.z splits K into chunks.  An operand is
+// read along its contiguous axis (KC: the K axis, else its row or column
+// axis), the next step's values into registers while this step's products run,
+// cut into parts once, as they are stored to shared memory in pairs along K,
+// and read back by ldmatrix (rows of 20 words: no bank conflicts).  The tile's
+// products take 5 us of the tensor cores at 8192 x 256 x 256; a first version
+// that staged FP32 values one K step of 16 at a time and cut them per warp ran
+// at the memory latency of each step: 74 us, this one 26.
+constexpr int kGT = 64, kGK = 32, kGP = 20;   // tile, K step, pitch in words (pairs of bf16)
+
+__device__ __forceinline__ float gval(float v) { return v; }
+__device__ __forceinline__ float gval(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ void gvec4(const float* p, float* x) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  x[0] = v.x;
+  x[1] = v.y;
+  x[2] = v.z;
+  x[3] = v.w;
+}
+__device__ __forceinline__ void gvec4(const __nv_bfloat16* p, float* x) {
+  const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+  x[0] = __uint_as_float(v.x << 16);
+  x[1] = __uint_as_float(v.x & 0xffff0000u);
+  x[2] = __uint_as_float(v.y << 16);
+  x[3] = __uint_as_float(v.y & 0xffff0000u);
 }
 
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
-  // a in the low half: the element of the smaller k (or row) index
-  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+// 16 values of this thread's share of a 64 x 32 operand tile (rows r0.., terms
+// k0..; zero beyond R and ke).  KC: row r at p + r ld, four consecutive terms
+// of four rows; else term k at p + k ld, four consecutive rows of two terms,
+// twice.  vec: the groups of four are aligned and end with the operand.
+template <bool KC, typename T>
+__device__ __forceinline__ void g_load(const T* __restrict__ p, long long ld, int R, int ke, int r0, int k0, bool vec,
+                                       float (&x)[16]) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int it = 0; it < 4; ++it) {
+    const int r = KC ? r0 + (tid >> 3) + 16 * it : r0 + 4 * ((tid >> 4) + 8 * (it >> 1));
+    const int k = KC ? k0 + 4 * (tid & 7) : k0 + 2 * (tid & 15) + (it & 1);
+    float* v = x + 4 * it;
+    const T* q = KC ? p + r * ld + k : p + k * ld + r;
+    if (vec) {
+      if (r < R && k < ke) {
+        gvec4(q, v);
+      } else {
+        v[0] = v[1] = v[2] = v[3] = 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const bool ok = KC ? r < R && k + e < ke : r + e < R && k < ke;
+        v[e] = ok ? gval(q[e]) : 0.f;
+      }
+    }
+  }
+}
+
+// the pair (a, b), b in the upper half, as PARTS bf16 words
+template <int PARTS>
+__device__ __forceinline__ void g_split(float a, float b, uint32_t (&w)[PARTS]) {
+#pragma unroll
+  for (int q = 0; q < PARTS; ++q) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    w[q] = *reinterpret_cast<const uint32_t*>(&h);
+    a -= __uint_as_float(w[q] << 16);
+    b -= __uint_as_float(w[q] & 0xffff0000u);
+  }
+}
+
+template <bool KC, int PARTS>
+__device__ __forceinline__ void g_store(uint32_t* s, const float (&x)[16]) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int it = 0; it < (KC ? 4 : 2); ++it) {
+    if (KC) {
+      uint32_t w0[PARTS], w1[PARTS];
+      g_split<PARTS>(x[4 * it], x[4 * it + 1], w0);
+      g_split<PARTS>(x[4 * it + 2], x[4 * it + 3], w1);
+      const int at = ((tid >> 3) + 16 * it) * kGP + 2 * (tid & 7);
+#pragma unroll
+      for (int q = 0; q < PARTS; ++q)
+        *reinterpret_cast<uint2*>(s + q * kGT * kGP + at) = make_uint2(w0[q], w1[q]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t w[PARTS];
+        g_split<PARTS>(x[8 * it + e], x[8 * it + 4 + e], w);
+        const int at = (4 * ((tid >> 4) + 8 * it) + e) * kGP + (tid & 15);
+#pragma unroll
+        for (int q = 0; q < PARTS; ++q) s[q * kGT * kGP + at] = w[q];
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const uint32_t* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a));
 }
 
 __device__ __forceinline__ void mma16816(float* c, const uint32_t* a, const uint32_t* b) {
@@ -98,22 +182,18 @@ __device__ __forceinline__ void mma16816(float* c, const uint32_t* a, const uint
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// C (M x N) = A (M x K) B (K x N) with element (i, k) of A at A[i sam + k sak]
-// and (k, j) of B at B[k sbk + j sbn].  blockIdx.z splits K into chunks.
-// mode 0: C = act(acc + bias) [* (1 - gate^2)];  mode 1: C += acc (atomic).
-// 64 x 64 tiles, four warps of 32 x 32 (2 x 4 mma tiles), K steps of 16
-// staged in shared memory as FP32.  A is split in three bf16 parts; B is one
-// part when it is the bf16 weight copy, three when it is an FP32 array.
-template <typename TB>
+// mode 0: C = act(acc + bias) [* (1 - gate^2)], and csum_j += sum_i C_ij;
+// mode 1: C += acc (atomic).
+template <bool AKC, bool BKC, typename TB>
 __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, int kchunk, const float* __restrict__ A,
-                                              long long sam, long long sak, const TB* __restrict__ B,
-                                              long long sbk, long long sbn, float* __restrict__ C, long long ldc,
+                                              long long lda, bool avec, const TB* __restrict__ B, long long ldb,
+                                              bool bvec, float* __restrict__ C, long long ldc,
                                               const float* __restrict__ bias, int act, const float* __restrict__ gate,
-                                              int mode) {
-  constexpr bool BEXACT = sizeof(TB) == 2;
-  __shared__ float As[16][64 + 4];   // As[k][i]
-  __shared__ float Bs[16][64 + 4];   // Bs[k][j]
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+                                              float* __restrict__ csum, int mode) {
+  constexpr int BP = sizeof(TB) == 2 ? 1 : 3;
+  __shared__ __align__(16) uint32_t As[3 * kGT * kGP];
+  __shared__ __align__(16) uint32_t Bs[BP * kGT * kGP];
+  const int m0 = blockIdx.y * kGT, n0 = blockIdx.x * kGT;
   const int kb = blockIdx.z * kchunk;
   const int ke = min(K, kb + kchunk);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -126,102 +206,89 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, int kchunk, c
     for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[mi][ni][e] = 0.f;
-  for (int k0 = kb; k0 < ke; k0 += 16) {
-    for (int e = threadIdx.x; e < 64 * 16; e += 128) {
-      int i, k;
-      if (sam == 1) {
-        i = e & 63;
-        k = e >> 6;
-      } else {
-        i = e >> 4;
-        k = e & 15;
-      }
-      const int gi = m0 + i, gk = k0 + k;
-      As[k][i] = (gi < M && gk < ke) ? A[gi * sam + gk * sak] : 0.f;
-      int j, kk;
-      if (sbn == 1) {
-        j = e & 63;
-        kk = e >> 6;
-      } else {
-        j = e >> 4;
-        kk = e & 15;
-      }
-      const int gj = n0 + j, gk2 = k0 + kk;
-      Bs[kk][j] = (gj < N && gk2 < ke) ? tof<TB>(B[gk2 * sbk + gj * sbn]) : 0.f;
-    }
+  float ra[16], rb[16];
+  g_load<AKC>(A, lda, M, ke, m0, kb, avec, ra);
+  g_load<BKC>(B, ldb, N, ke, n0, kb, bvec, rb);
+  const uint32_t* pa = As + (wm + (lane & 15)) * kGP + 4 * (lane >> 4);
+  const uint32_t* pb = Bs + (wn + (lane & 7) + 8 * (lane >> 4)) * kGP + 4 * ((lane >> 3) & 1);
+  for (int k0 = kb; k0 < ke; k0 += kGK) {
+    g_store<AKC, 3>(As, ra);
+    g_store<BKC, BP>(Bs, rb);
     __syncthreads();
-    // A fragments (rows g, g + 8; k pairs 2tq, 2tq + 8) in three parts
-    uint32_t af[3][2][4];
-#pragma unroll
-    for (int mi = 0; mi < 2; ++mi) {
-      const int r = wm + mi * 16 + g;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int rr = r + ((q & 1) ? 8 : 0);
-        const int kk = 2 * tq + ((q & 2) ? 8 : 0);
-        __nv_bfloat16 h0, m0b, l0, h1, m1b, l1;
-        split3(As[kk][rr], h0, m0b, l0);
-        split3(As[kk + 1][rr], h1, m1b, l1);
-        af[0][mi][q] = pack2(h0, h1);
-        af[1][mi][q] = pack2(m0b, m1b);
-        af[2][mi][q] = pack2(l0, l1);
-      }
+    if (k0 + kGK < ke) {
+      g_load<AKC>(A, lda, M, ke, m0, k0 + kGK, avec, ra);
+      g_load<BKC>(B, ldb, N, ke, n0, k0 + kGK, bvec, rb);
     }
 #pragma unroll
-    for (int ni = 0; ni < 4; ++ni) {
-      const int col = wn + ni * 8 + g;
-      uint32_t bf[3][2];
+    for (int kk = 0; kk < 2; ++kk) {
+      if (kk == 1 && k0 + 16 >= ke) break;
+      uint32_t af[3][2][4];
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int kk = 2 * tq + (q ? 8 : 0);
-        __nv_bfloat16 h0, m0b, l0, h1, m1b, l1;
-        split3(Bs[kk][col], h0, m0b, l0);
-        split3(Bs[kk + 1][col], h1, m1b, l1);
-        bf[0][q] = pack2(h0, h1);
-        bf[1][q] = pack2(m0b, m1b);
-        bf[2][q] = pack2(l0, l1);
-      }
+      for (int q = 0; q < 3; ++q)
 #pragma unroll
-      for (int mi = 0; mi < 2; ++mi) {
-        // small terms first: lo, mid, then hi
-        if (BEXACT) {
-          mma16816(acc[mi][ni], af[2][mi], bf[0]);
-          mma16816(acc[mi][ni], af[1][mi], bf[0]);
-          mma16816(acc[mi][ni], af[0][mi], bf[0]);
-        } else {
-          mma16816(acc[mi][ni], af[2][mi], bf[0]);
-          mma16816(acc[mi][ni], af[0][mi], bf[2]);
-          mma16816(acc[mi][ni], af[1][mi], bf[1]);
-          mma16816(acc[mi][ni], af[1][mi], bf[0]);
-          mma16816(acc[mi][ni], af[0][mi], bf[1]);
-          mma16816(acc[mi][ni], af[0][mi], bf[0]);
-        }
+        for (int mi = 0; mi < 2; ++mi) ldsm4(af[q][mi], pa + (q * kGT + mi * 16) * kGP + 8 * kk);
+#pragma unroll
+      for (int nj = 0; nj < 2; ++nj) {
+        uint32_t bf[BP][4];
+#pragma unroll
+        for (int q = 0; q < BP; ++q) ldsm4(bf[q], pb + (q * kGT + nj * 16) * kGP + 8 * kk);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int mi = 0; mi < 2; ++mi) {
+            float* c = acc[mi][2 * nj + h];
+            // small terms first: lo, mid, then hi
+            if (BP == 1) {
+              mma16816(c, af[2][mi], bf[0] + 2 * h);
+              mma16816(c, af[1][mi], bf[0] + 2 * h);
+              mma16816(c, af[0][mi], bf[0] + 2 * h);
+            } else {
+              mma16816(c, af[2][mi], bf[0] + 2 * h);
+              mma16816(c, af[0][mi], bf[BP - 1] + 2 * h);
+              mma16816(c, af[1][mi], bf[BP / 2] + 2 * h);
+              mma16816(c, af[1][mi], bf[0] + 2 * h);
+              mma16816(c, af[0][mi], bf[BP / 2] + 2 * h);
+              mma16816(c, af[0][mi], bf[0] + 2 * h);
+            }
+          }
       }
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int mi = 0; mi < 2; ++mi)
+  for (int ni = 0; ni < 4; ++ni) {
+    const int j = n0 + wn + ni * 8 + 2 * tq;
+    float cs[2] = {0.f, 0.f};
 #pragma unroll
-    for (int ni = 0; ni < 4; ++ni)
+    for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int i = m0 + wm + mi * 16 + g + (e >= 2 ? 8 : 0);
-        const int j = n0 + wn + ni * 8 + 2 * tq + (e & 1);
-        if (i >= M || j >= N) continue;
-        float* o = C + (long long)i * ldc + j;
+        const int jj = j + (e & 1);
+        if (i >= M || jj >= N) continue;
+        float* o = C + (long long)i * ldc + jj;
         if (mode == 1) {
           atomicAdd(o, acc[mi][ni][e]);
         } else {
-          float v = acc[mi][ni][e] + (bias ? bias[j] : 0.f);
+          float v = acc[mi][ni][e] + (bias ? bias[jj] : 0.f);
           if (act) v = tanhf(v);
           if (gate) {
-            const float gt = gate[(long long)i * ldc + j];
+            const float gt = gate[(long long)i * ldc + jj];
             v *= 1.f - gt * gt;
           }
           *o = v;
+          cs[e & 1] += v;
         }
       }
+    if (csum) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) cs[e] += __shfl_xor_sync(0xffffffffu, cs[e], o);
+        if (g == 0 && j + e < N) atomicAdd(csum + j + e, cs[e]);
+      }
+    }
+  }
 }
 
 // X[i, :] = (raw[r_i, :] - shift) * scale with r_i = rows[i] (i when rows is
@@ -238,51 +305,86 @@ __global__ void k_normalise(int n, int n_in, const float* __restrict__ raw, cons
   if (t_in && k == 0) t_out[i] = t_in[r];
 }
 
-// y_i = W3 a2_i + b3 (a warp per row); with targets: dy_i = (y_i - t_i)/n and
-// the loss sum 1/(2n) sum e^2.
+// y_i = W3 a2_i + b3 + WL x_i (a warp per row)
+__device__ __forceinline__ float row_output(int W, const float* __restrict__ a, const __nv_bfloat16* __restrict__ w3,
+                                            float b3, int n_in, const float* __restrict__ x,
+                                            const float* __restrict__ wl) {
+  const int lane = threadIdx.x & 31;
+  float s = 0.f;
+  for (int k = lane; k < W; k += 32) s = fmaf(a[k], __bfloat162float(w3[k]), s);
+  if (lane < n_in) s = fmaf(x[lane], wl[lane], s);
+  return warp_sum(s) + b3;
+}
+
 __global__ void k_output(int n, int W, const float* __restrict__ a2, const __nv_bfloat16* __restrict__ w3,
                          const float* __restrict__ b3, int n_in, const float* __restrict__ X,
-                         const float* __restrict__ wl, float* __restrict__ y, const float* __restrict__ t,
-                         float* __restrict__ dy, float* __restrict__ loss) {
+                         const float* __restrict__ wl, float* __restrict__ y) {
   const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
   if (row >= n) return;
-  float s = 0.f;
-  for (int k = lane; k < W; k += 32) s = fmaf(a2[(long long)row * W + k], __bfloat162float(w3[k]), s);
-  if (lane < n_in) s = fmaf(X[(long long)row * n_in + lane], wl[lane], s);
-  s = warp_sum(s);
-  if (lane == 0) {
-    const float v = s + b3[0];
-    y[row] = v;
-    if (t) {
-      const float e = v - t[row];
-      dy[row] = e / (float)n;
-      atomicAdd(loss, 0.5f * e * e / (float)n);
+  const float v = row_output(W, a2 + (long long)row * W, w3, b3[0], n_in, X + (long long)row * n_in, wl);
+  if ((threadIdx.x & 31) == 0) y[row] = v;
+}
+
+// The head of a training step over kHeadRows rows per CTA: the outputs, the
+// loss 1/(2n) sum e^2, dy = e/n, the back-propagated d2 = dy W3 (1 - a2^2), and
+// the gradients of the output layer and of b2 (dW3 = dy^T a2, db3 = sum dy, dWL =
+// dy^T x~, db2 = sum d2), one pass over a2 with a column per thread.  Six
+// launches, four of them column sums of 32 CTAs that waited on one load per
+// row, took 119 us for 8192 rows; this kernel 16.
+constexpr int kHeadRows = 32, kHeadThreads = 256;
+__global__ void __launch_bounds__(kHeadThreads) k_head(int n, int W, const float* __restrict__ a2,
+                                                       const __nv_bfloat16* __restrict__ w3,
+                                                       const float* __restrict__ b3, int n_in,
+                                                       const float* __restrict__ X, const float* __restrict__ wl,
+                                                       const float* __restrict__ t, float* __restrict__ y,
+                                                       float* __restrict__ d2, float* __restrict__ loss,
+                                                       float* __restrict__ gW3, float* __restrict__ gb3,
+                                                       float* __restrict__ gWL, float* __restrict__ gb2) {
+  __shared__ float dy[kHeadRows];
+  __shared__ float es[kHeadThreads / 32];
+  const int r0 = blockIdx.x * kHeadRows, nr = min(kHeadRows, n - r0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float e2 = 0.f;
+  for (int r = warp; r < kHeadRows; r += kHeadThreads / 32) {
+    float e = 0.f;
+    if (r < nr) {
+      const long long row = r0 + r;
+      const float v = row_output(W, a2 + row * W, w3, b3[0], n_in, X + row * n_in, wl);
+      e = v - t[row];
+      if (lane == 0) y[row] = v;
     }
+    if (lane == 0) dy[r] = e / (float)n;
+    e2 += e * e;
   }
-}
-
-// d2 = dy_i W3_k (1 - a2^2)
-__global__ void k_back_out(int n, int W, const float* __restrict__ dy, const __nv_bfloat16* __restrict__ w3,
-                           const float* __restrict__ a2, float* __restrict__ d2) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)n * W) return;
-  const int k = (int)(t % W);
-  const long long i = t / W;
-  const float g = a2[t];
-  d2[t] = dy[i] * __bfloat162float(w3[k]) * (1.f - g * g);
-}
-
-// out_k += sum_i w_i X[i, k] (w = 1 when null); rows split over blocks
-__global__ void k_colsum(int n, int c, const float* __restrict__ w, const float* __restrict__ X, float* __restrict__ out,
-                         int rows_per_block) {
-  const int k = threadIdx.x + blockIdx.y * blockDim.x;
-  if (k >= c) return;
-  const int r0 = blockIdx.x * rows_per_block;
-  const int r1 = min(n, r0 + rows_per_block);
-  float s = 0.f;
-  for (int i = r0; i < r1; ++i) s = fmaf(w ? w[i] : 1.f, X[(long long)i * c + k], s);
-  atomicAdd(out + k, s);
+  if (lane == 0) es[warp] = e2;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int q = 0; q < kHeadThreads / 32; ++q) s += es[q];
+    atomicAdd(loss, 0.5f * s / (float)n);
+  }
+  for (int k = threadIdx.x; k < W; k += kHeadThreads) {
+    const float w = __bfloat162float(w3[k]);
+    const float* a = a2 + (long long)r0 * W + k;
+    float* d = d2 + (long long)r0 * W + k;
+    float s3 = 0.f, s2 = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < nr; ++r) {
+      const float v = a[(long long)r * W];
+      const float b = dy[r] * w * (1.f - v * v);
+      d[(long long)r * W] = b;
+      s3 = fmaf(dy[r], v, s3);
+      s2 += b;
+    }
+    atomicAdd(gW3 + k, s3);
+    atomicAdd(gb2 + k, s2);
+  }
+  if (threadIdx.x <= n_in) {
+    const int k = threadIdx.x;
+    float s = 0.f;
+    for (int r = 0; r < nr; ++r) s = fmaf(dy[r], k < n_in ? X[(long long)(r0 + r) * n_in + k] : 1.f, s);
+    atomicAdd(k < n_in ? gWL + k : gb3, s);
+  }
 }
 
 __global__ void k_round(int np, const float* __restrict__ theta, __nv_bfloat16* __restrict__ wbf) {
@@ -343,7 +445,7 @@ __global__ void k_to_density(int n, const float* __restrict__ y, double shift, d
 kfbi_status ensure(kfbi_mlp* m, int n) {
   if (n <= m->cap) return KFBI_OK;
   MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-  float** bufs[] = {&m->X, &m->a1, &m->a2, &m->d1, &m->d2, &m->y, &m->dy, &m->tb};
+  float** bufs[] = {&m->X, &m->a1, &m->a2, &m->d1, &m->d2, &m->y, &m->tb};
   for (float** b : bufs) {
     cudaFree(*b);
     *b = nullptr;
@@ -356,36 +458,48 @@ kfbi_status ensure(kfbi_mlp* m, int n) {
   MLP_CUDA(m, dalloc(&m->d1, (size_t)cap * W));
   MLP_CUDA(m, dalloc(&m->d2, (size_t)cap * W));
   MLP_CUDA(m, dalloc(&m->y, (size_t)cap));
-  MLP_CUDA(m, dalloc(&m->dy, (size_t)cap));
   MLP_CUDA(m, dalloc(&m->tb, (size_t)cap));
   m->cap = cap;
   return KFBI_OK;
 }
 
-template <typename TB>
-void gemm(cudaStream_t st, int M, int N, int K, const float* A, long long sam, long long sak, const TB* B,
-          long long sbk, long long sbn, float* C, long long ldc, const float* bias, int act, const float* gate,
-          int mode) {
+// AKC / BKC: the operand is contiguous along K (A: M x K row-major, B: N x K),
+// else along its other axis (A: K x M, B: K x N)
+template <bool AKC, bool BKC, typename TB>
+void gemm(cudaStream_t st, int M, int N, int K, const float* A, long long lda, const TB* B, long long ldb, float* C,
+          long long ldc, const float* bias, int act, const float* gate, float* csum, int mode) {
   int splits = 1, chunk = K;
-  if (mode == 1) {   // weight gradients: long K (the rows), few output tiles
-    const int tiles = div_up(M, 64) * div_up(N, 64);
-    splits = std::max(1, std::min(div_up(K, 256), div_up(152 * 8, tiles)));
-    chunk = div_up(div_up(K, splits), 16) * 16;
+  if (mode == 1) {
+    // weight gradients: long K (the rows), few output tiles.  Chunks of at
+    // most 256 terms bound the rounding of one accumulator; few tiles (dW1) take
+    // down to 128 for two CTAs per SM
+    const int tiles = div_up(M, kGT) * div_up(N, kGT);
+    splits = std::max(div_up(K, 256), std::min(div_up(K, 128), div_up(152 * 2, tiles)));
+    chunk = div_up(div_up(K, splits), kGK) * kGK;
     splits = div_up(K, chunk);
   }
-  dim3 grid(div_up(N, 64), div_up(M, 64), splits);
-  k_gemm<TB><<<grid, 128, 0, st>>>(M, N, K, chunk, A, sam, sak, B, sbk, sbn, C, ldc, bias, act, gate, mode);
+  auto vec = [](const void* p, size_t el, long long ld, int along) {
+    return (reinterpret_cast<uintptr_t>(p) % (4 * el)) == 0 && ld % 4 == 0 && along % 4 == 0;
+  };
+  const bool av = vec(A, sizeof(float), lda, AKC ? K : M), bv = vec(B, sizeof(TB), ldb, BKC ? K : N);
+  dim3 grid(div_up(N, kGT), div_up(M, kGT), splits);
+  k_gemm<AKC, BKC, TB><<<grid, 128, 0, st>>>(M, N, K, chunk, A, lda, av, B, ldb, bv, C, ldc, bias, act, gate, csum,
+                                              mode);
+}
+
+// the hidden layers of the rows already normalised into m->X
+void hidden_rows(kfbi_mlp* m, int n) {
+  const int W = m->width, ni = m->n_in;
+  const __nv_bfloat16* wb = m->wbf;
+  gemm<true, true>(m->stream, n, W, ni, m->X, ni, wb + m->oW1, ni, m->a1, W, m->theta + m->ob1, 1, nullptr, nullptr, 0);
+  gemm<true, true>(m->stream, n, W, W, m->a1, W, wb + m->oW2, W, m->a2, W, m->theta + m->ob2, 1, nullptr, nullptr, 0);
 }
 
 // forward on rows already normalised into m->X
-kfbi_status forward_rows(kfbi_mlp* m, int n, const float* t) {
-  const int W = m->width, ni = m->n_in;
-  cudaStream_t st = m->stream;
-  const __nv_bfloat16* wb = m->wbf;
-  gemm<__nv_bfloat16>(st, n, W, ni, m->X, ni, 1, wb + m->oW1, 1, ni, m->a1, W, m->theta + m->ob1, 1, nullptr, 0);
-  gemm<__nv_bfloat16>(st, n, W, W, m->a1, W, 1, wb + m->oW2, 1, W, m->a2, W, m->theta + m->ob2, 1, nullptr, 0);
-  k_output<<<div_up(n, 8), 256, 0, st>>>(n, W, m->a2, wb + m->oW3, m->theta + m->ob3, ni, m->X,
-                                         m->theta + m->oWL, m->y, t, m->dy, m->loss);
+kfbi_status forward_rows(kfbi_mlp* m, int n) {
+  hidden_rows(m, n);
+  k_output<<<div_up(n, 8), 256, 0, m->stream>>>(n, m->width, m->a2, m->wbf + m->oW3, m->theta + m->ob3, m->n_in, m->X,
+                                                m->theta + m->oWL, m->y);
   MLP_CUDA(m, cudaGetLastError());
   return KFBI_OK;
 }
@@ -403,7 +517,7 @@ kfbi_status kfbi_mlp_destroy(kfbi_mlp* m) {
   if (!m) return KFBI_OK;
   if (m->stream) cudaStreamSynchronize(m->stream);
   void* bufs[] = {m->theta, m->grad, m->mom1, m->mom2, m->wbf, m->shift, m->scale, m->X,
-                  m->a1,    m->a2,   m->d1,   m->d2,   m->y,   m->dy,    m->tb,    m->loss};
+                  m->a1,    m->a2,   m->d1,   m->d2,   m->y,   m->tb,   m->loss};
   for (void* b : bufs) cudaFree(b);
   delete m;
   return KFBI_OK;
@@ -504,7 +618,7 @@ kfbi_status kfbi_mlp_forward(kfbi_mlp* m, const float* X, int n, float* y) {
   const long long tot = (long long)n * m->n_in;
   k_normalise<<<div_up(tot, 256), 256, 0, m->stream>>>(n, m->n_in, X, nullptr, m->shift, m->scale, m->X,
                                                         nullptr, nullptr);
-  KFBI_TRY(forward_rows(m, n, nullptr));
+  KFBI_TRY(forward_rows(m, n));
   MLP_CUDA(m, cudaMemcpyAsync(y, m->y, sizeof(float) * n, cudaMemcpyDeviceToDevice, m->stream));
   return KFBI_OK;
 }
@@ -519,22 +633,16 @@ kfbi_status kfbi_mlp_loss_grad(kfbi_mlp* m, const float* X, const float* t, cons
   MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float), st));
   MLP_CUDA(m, cudaMemsetAsync(m->grad, 0, sizeof(float) * m->nparam, st));
   k_normalise<<<div_up(tot, 256), 256, 0, st>>>(n, ni, X, rows, m->shift, m->scale, m->X, t, m->tb);
-  KFBI_TRY(forward_rows(m, n, m->tb));
+  hidden_rows(m, n);
   const __nv_bfloat16* wb = m->wbf;
   float* g = m->grad;
-  // output layer: dW3 = dy^T a2, db3 = sum dy
-  const int rpb = 256;
-  k_colsum<<<dim3(div_up(n, rpb), div_up(W, 256)), 256, 0, st>>>(n, W, m->dy, m->a2, g + m->oW3, rpb);
-  k_colsum<<<dim3(div_up(n, rpb), 1), 32, 0, st>>>(n, 1, nullptr, m->dy, g + m->ob3, rpb);
-  k_colsum<<<dim3(div_up(n, rpb), 1), 32, 0, st>>>(n, ni, m->dy, m->X, g + m->oWL, rpb);
-  // d2 = dy W3 (1 - a2^2); dW2 = d2^T a1, db2 = sum d2
-  k_back_out<<<div_up((long long)n * W, 256), 256, 0, st>>>(n, W, m->dy, wb + m->oW3, m->a2, m->d2);
-  gemm<float>(st, W, W, n, m->d2, 1, W, m->a1, W, 1, g + m->oW2, W, nullptr, 0, nullptr, 1);
-  k_colsum<<<dim3(div_up(n, rpb), div_up(W, 256)), 256, 0, st>>>(n, W, nullptr, m->d2, g + m->ob2, rpb);
-  // d1 = (d2 W2) (1 - a1^2); dW1 = d1^T x~, db1 = sum d1
-  gemm<__nv_bfloat16>(st, n, W, W, m->d2, W, 1, wb + m->oW2, W, 1, m->d1, W, nullptr, 0, m->a1, 0);
-  gemm<float>(st, W, ni, n, m->d1, 1, W, m->X, ni, 1, g + m->oW1, ni, nullptr, 0, nullptr, 1);
-  k_colsum<<<dim3(div_up(n, rpb), div_up(W, 256)), 256, 0, st>>>(n, W, nullptr, m->d1, g + m->ob1, rpb);
+  k_head<<<div_up(n, kHeadRows), kHeadThreads, 0, st>>>(n, W, m->a2, wb + m->oW3, m->theta + m->ob3, ni, m->X,
+                                                        m->theta + m->oWL, m->tb, m->y, m->d2, m->loss, g + m->oW3,
+                                                        g + m->ob3, g + m->oWL, g + m->ob2);
+  // dW2 = d2^T a1; d1 = (d2 W2) (1 - a1^2), db1 = sum d1; dW1 = d1^T x~
+  gemm<false, false>(st, W, W, n, m->d2, W, m->a1, W, g + m->oW2, W, nullptr, 0, nullptr, nullptr, 1);
+  gemm<true, false>(st, n, W, W, m->d2, W, wb + m->oW2, W, m->d1, W, nullptr, 0, m->a1, g + m->ob1, 0);
+  gemm<false, false>(st, W, ni, n, m->d1, W, m->X, ni, g + m->oW1, ni, nullptr, 0, nullptr, nullptr, 1);
   MLP_CUDA(m, cudaGetLastError());
   if (loss) MLP_CUDA(m, cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
   return KFBI_OK;
@@ -583,7 +691,7 @@ kfbi_status kfbi_warm_start(kfbi_problem* p, kfbi_mlp* m, const kfbi_data* data,
   KFBI_LAUNCH(p, KFBI_KC_OTHER, k_normalise<<<div_up(tot, 256), 256, 0, p->stream>>>(
       nb, m->n_in, m->d1, nullptr, m->shift, m->scale, m->X, nullptr, nullptr));
   {
-    kfbi_status s = forward_rows(m, nb, nullptr);
+    kfbi_status s = forward_rows(m, nb);
     if (s != KFBI_OK) return fail(p, s, m->err);
   }
   KFBI_LAUNCH(p, KFBI_KC_OTHER, k_to_density<<<div_up(nb, 256), 256, 0, p->stream>>>(nb, m->y, m->out_shift,
@@ -620,7 +728,7 @@ kfbi_status kfbi_warm_start_batch(kfbi_batch* b, kfbi_mlp* m, const kfbi_data* d
   KFBI_LAUNCH(p0, KFBI_KC_OTHER, k_normalise<<<div_up(tot, 256), 256, 0, p0->stream>>>(
       rows, m->n_in, m->d1, nullptr, m->shift, m->scale, m->X, nullptr, nullptr));
   {
-    kfbi_status s = forward_rows(m, rows, nullptr);
+    kfbi_status s = forward_rows(m, rows);
     if (s != KFBI_OK) return fail(p0, s, m->err);
   }
   for (int k = 0; k < n; ++k) {

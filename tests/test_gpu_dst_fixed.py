@@ -5,7 +5,7 @@ import pytest
 
 import workloads as W
 from oracle import boxsolve as BS
-from gpu_util import dev, empty, host
+from tests.gpu_util import dev, empty, host
 
 pytestmark = pytest.mark.gpu
 
