@@ -1160,22 +1160,31 @@ struct FixStencil {
   int w0, w1, w2, w3, kA, kB;
 };
 
-// S U of the integer stencil and the kappa combination kA U_P + kB e, with
-// the weights of the three operators as shifts and adds on 32-bit pieces
-__device__ __forceinline__ long long fix_apply(const FixStencil& W, long long c, long long e, long long k2,
-                                               long long k3, long long& m) {
+// a + w b for a small weight: one 32 x 32 -> 64 multiply-add and one for the
+// high word, where shifts and adds of 64-bit numbers take two instructions each
+// (27 for the three weights of the 27-point operator)
+__device__ __forceinline__ long long mad64(long long a, unsigned w, long long b) {
+  unsigned bl, bh, rl, rh;
+  split64(b, bl, bh);
+  long long t;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(t) : "r"(bl), "r"(w), "l"(a));
+  split64(t, rl, rh);
+  return join64(rl, bh * w + rh);
+}
+
+// R - S U of the integer stencil and the kappa combination m = kA U_P + kB e
+__device__ __forceinline__ long long fix_residual_at(const FixStencil& W, long long R, long long c, long long e,
+                                                     long long k2, long long k3, long long& m) {
   if (W.w0 == -20) {          // 2D 4th order: -20 c + 4 e + k2; kappa: 8 c + e
-    m = add64(shl64<3>(c), e);
-    return add64(shl64<2>(sub64(e, add64(shl64<2>(c), c))), k2);
+    m = mad64(e, 8u, c);
+    return sub64(mad64(R, 20u, c), mad64(k2, 4u, e));
   }
   if (W.w0 == -200) {         // 3D 4th order: -200 c + 20 e + 6 k2 + k3; kappa: 6 c + e
-    m = add64(add64(shl64<2>(c), shl64<1>(c)), e);
-    const long long fifty_c = add64(add64(shl64<5>(c), shl64<4>(c)), shl64<1>(c));
-    const long long t = sub64(add64(shl64<2>(e), e), fifty_c);           // 5 e - 50 c
-    return add64(add64(shl64<2>(t), add64(shl64<2>(k2), shl64<1>(k2))), k3);
+    m = mad64(e, 6u, c);
+    return sub64(mad64(R, 200u, c), mad64(mad64(k3, 6u, k2), 20u, e));
   }
   m = c;                      // 2nd order: -2 d c + e; kappa: c
-  return W.w0 == -4 ? sub64(e, shl64<2>(c)) : sub64(e, add64(shl64<2>(c), shl64<1>(c)));
+  return sub64(mad64(R, W.w0 == -4 ? 4u : 6u, c), e);
 }
 
 // the 9/27 neighbour sums of a fixed-point grid at index t (32-bit indices)
@@ -1281,7 +1290,7 @@ __global__ void k_res_fix2(Grid g, FixStencil W, const long long* __restrict__ R
     const long long e = add64(cH, add64(mC, qC));   // edge neighbours
     const long long k2 = add64(mH, qH);             // corners
     long long m;
-    long long r = sub64(Ri, fix_apply(W, cC, e, k2, 0, m));
+    long long r = fix_residual_at(W, Ri, cC, e, k2, 0, m);
     if (!kf.zero) r = add64(r, kappa_int(kf, m));
     r32[i * n1 + j] = (ll2f(r) * f2) * f4;
     mC = cC;
@@ -1388,7 +1397,7 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
         const long long k2 = add64(cS2[r], add64(mS1[r], qS1[r]));
         const long long k3 = add64(mS2[r], qS2[r]);
         long long m;
-        long long res = sub64(Rcur[r], fix_apply(W, cC[r], e, k2, k3, m));
+        long long res = fix_residual_at(W, Rcur[r], cC[r], e, k2, k3, m);
         if (!kf.zero) res = add64(res, kappa_int(kf, m));
         r32[tb + r * n1] = (ll2f(res) * f2) * f4;
       }
@@ -2339,7 +2348,7 @@ __global__ void k_rows_batched(const BoxDesc* __restrict__ D, const int* __restr
         FIX_NEIGHBOURS(UP)
 #undef UP
         long long m;
-        long long r = sub64(B.rfix[t], fix_apply(W, c, e, k2, k3, m));
+        long long r = fix_residual_at(W, B.rfix[t], c, e, k2, k3, m);
         const KappaFix kf = kappa_fix(B.fixd[2]);
         if (!kf.zero) r = add64(r, kappa_int(kf, m));
         B.r32[t] = (ll2f(r) * B.fixf[2]) * B.fixf[4];
