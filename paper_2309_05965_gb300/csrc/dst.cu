@@ -2306,52 +2306,117 @@ __global__ void k_check_batched(const BoxDesc* __restrict__ D, int ninst, int st
   nrm[4] = 0ull;
 }
 
-__global__ void k_fix_scale_batched(const BoxDesc* __restrict__ D, int ninst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ninst) return;
-  fix_scale_store(fix_scale_of(D[i].nrm[5], D[i].multh2, 1.0 / D[i].multh2), D[i].kc, D[i].fixd, D[i].fixf);
-}
-
-// grid kernels over all instances' rows (one row of the last axis per item);
-// mode 0: u_fix = round(u0 2^F), R_fix = round(mult h^2 R 2^F);
-// mode 1: exact residual -> r32 (skips converged instances);
-// mode 2: u = u_fix 2^-F.
-__global__ void k_rows_batched(const BoxDesc* __restrict__ D, const int* __restrict__ rstart, int ninst, int mode) {
+// Grid kernels over all instances: an item is kFixRows rows of 128 columns of
+// one instance (its loads in flight together, as in the single solve).
+// MODE 0: the fixed-point scale, u_fix = round(u0 2^F / (mult h^2)), R_fix = round(R 2^F);
+// MODE 1: exact residual -> r32 (skips converged instances), in 2D marching
+// over the rows with k_res_fix2's three-row window;
+// MODE 2: u = u_fix mult h^2 2^-F of the instances that converged before the last
+// step; of the others, whose last pass writes u at the interior nodes, the
+// boundary layer (0); nothing of those in `done`.  MODE 3: u of every instance.
+template <int MODE>
+__global__ void __launch_bounds__(128) k_rows_batched(const BoxDesc* __restrict__ D, const int* __restrict__ rstart,
+                                                      int ninst, const int* __restrict__ done) {
   const int total = rstart[ninst];
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int inst = find_inst(rstart, ninst, item);
     const BoxDesc& B = D[inst];
-    if (mode == 1 && *B.conv) continue;
-    const Grid g = B.g;
-    const int n1 = g.n + 1;
-    const int row = item - rstart[inst];
-    const int i1 = row % n1, i0 = row / n1;   // 2D: i0 = 0
-    const bool row_in = i1 >= 1 && i1 < g.n && (g.d == 2 || (i0 >= 1 && i0 < g.n));
-    const int base = g.d == 2 ? i1 * n1 : (i0 * n1 + i1) * n1;
-    for (int j = threadIdx.x; j <= g.n; j += blockDim.x) {
-      const int t = base + j;
-      const bool interior = row_in && j >= 1 && j < g.n;
-      if (mode == 0) {
-        const float* ff = B.fixf;
-        B.ufix[t] = f2ll((B.u0[t] * ff[0]) * ff[1]);
-        B.rfix[t] = interior ? d2ll_pow2(B.R[t], (int)B.fixd[3]) : 0ll;
-      } else if (mode == 2) {
-        B.u[t] = ll2d(B.ufix[t]) * B.fixd[1];
-      } else {
-        if (!interior) {
-          B.r32[t] = 0.f;
-          continue;
+    const int conv = *B.conv;
+    if (MODE == 1 && conv) continue;
+    if (MODE == 2 && done && done[inst]) continue;
+    const int n = B.g.n, n1 = n + 1;
+    const bool d2 = B.g.d == 2;
+    const int rows = d2 ? n1 : n1 * n1;
+    const int ncb = (n1 + 127) / 128;
+    const int local = item - rstart[inst];
+    const int j = 128 * (local % ncb) + threadIdx.x, r0 = (local / ncb) * kFixRows;
+    if (j > n) continue;
+    const bool in_j = j >= 1 && j < n;
+    const int nr = min(kFixRows, rows - r0);
+    if (MODE == 0) {
+      float uv[kFixRows];
+      double rv[kFixRows];
+#pragma unroll
+      for (int k = 0; k < kFixRows; ++k) {
+        uv[k] = k < nr ? B.u0[(r0 + k) * n1 + j] : 0.f;
+        rv[k] = k < nr && in_j ? B.R[(r0 + k) * n1 + j] : 0.0;
+      }
+      const FixScale s = fix_scale_of(B.nrm[5], B.multh2, 1.0 / B.multh2);
+      if (local == 0 && threadIdx.x == 0) fix_scale_store(s, B.kc, B.fixd, B.fixf);
+      long long* uf = B.ufix;
+      long long* rf = B.rfix;
+#pragma unroll
+      for (int k = 0; k < kFixRows; ++k) {
+        if (k >= nr) break;
+        const int r = r0 + k;
+        const int i1 = d2 ? r : r % n1, i0 = d2 ? 1 : r / n1;
+        const bool interior = in_j && i1 >= 1 && i1 < n && i0 >= 1 && i0 < n;
+        uf[r * n1 + j] = f2ll((uv[k] * s.f[0]) * s.f[1]);
+        rf[r * n1 + j] = interior ? d2ll_pow2(rv[k], s.F) : 0ll;
+      }
+    } else if (MODE >= 2) {
+      const double isc = B.fixd[1];
+      const long long* __restrict__ uf = B.ufix;
+      double* __restrict__ u = B.u;
+      if (MODE == 2 && !conv) {
+        for (int k = 0; k < nr; ++k) {
+          const int r = r0 + k;
+          const int i1 = d2 ? r : r % n1, i0 = d2 ? 1 : r / n1;
+          if (!(in_j && i1 >= 1 && i1 < n && i0 >= 1 && i0 < n)) u[r * n1 + j] = 0.0;
         }
-        const FixStencil W = B.W;
-        const long long* ub = B.ufix;
+        continue;
+      }
+      long long v[kFixRows];
+#pragma unroll
+      for (int k = 0; k < kFixRows; ++k) v[k] = k < nr ? uf[(r0 + k) * n1 + j] : 0ll;
+#pragma unroll
+      for (int k = 0; k < kFixRows; ++k)
+        if (k < nr) u[(r0 + k) * n1 + j] = ll2d(v[k]) * isc;
+    } else {
+      if (!in_j) continue;
+      const FixStencil W = B.W;
+      const KappaFix kf = kappa_fix(B.fixd[2]);
+      const float f2 = B.fixf[2], f4 = B.fixf[4];
+      const long long* __restrict__ ub = B.ufix;
+      const long long* __restrict__ Rb = B.rfix;
+      float* __restrict__ out = B.r32;
+      if (d2) {
+        const int a = max(r0, 1), b = min(r0 + nr, n);
+        if (a >= b) continue;
+        const long long* p = ub + (a - 1) * n1 + j;
+        long long mC = p[0], mH = add64(p[-1], p[1]);
+        p += n1;
+        long long cC = p[0], cH = add64(p[-1], p[1]);
+#pragma unroll
+        for (int k = 0; k < kFixRows; ++k) {
+          const int i = a + k;
+          if (i >= b) break;
+          p += n1;
+          const long long qC = p[0], qH = add64(p[-1], p[1]);
+          const long long Ri = Rb[i * n1 + j];
+          long long m;
+          long long r = fix_residual_at(W, Ri, cC, add64(cH, add64(mC, qC)), add64(mH, qH), 0, m);
+          if (!kf.zero) r = add64(r, kappa_int(kf, m));
+          out[i * n1 + j] = (ll2f(r) * f2) * f4;
+          mC = cC;
+          mH = cH;
+          cC = qC;
+          cH = qH;
+        }
+      } else {
+        const Grid g = B.g;
+        for (int k = 0; k < nr; ++k) {
+          const int r = r0 + k, i1 = r % n1, i0 = r / n1;
+          if (i1 < 1 || i1 >= n || i0 < 1 || i0 >= n) continue;
+          const int t = r * n1 + j;
 #define UP(o) ub[t + (o)]
-        FIX_NEIGHBOURS(UP)
+          FIX_NEIGHBOURS(UP)
 #undef UP
-        long long m;
-        long long r = fix_residual_at(W, B.rfix[t], c, e, k2, k3, m);
-        const KappaFix kf = kappa_fix(B.fixd[2]);
-        if (!kf.zero) r = add64(r, kappa_int(kf, m));
-        B.r32[t] = (ll2f(r) * B.fixf[2]) * B.fixf[4];
+          long long m;
+          long long v = fix_residual_at(W, Rb[t], c, e, k2, k3, m);
+          if (!kf.zero) v = add64(v, kappa_int(kf, m));
+          out[t] = (ll2f(v) * f2) * f4;
+        }
       }
     }
   }
@@ -2361,10 +2426,10 @@ __global__ void k_rows_batched(const BoxDesc* __restrict__ D, const int* __restr
 
 struct BatchBox {
   int ninst = 0, npass = 0, steps = 3;
-  PassArgs* dargs = nullptr;   // [2 npass][ninst]: step 0 passes, then refinement-step passes
+  PassArgs* dargs = nullptr;   // [3 npass][ninst]: step 0's passes, a refinement step's, the last step's
   int* dstart = nullptr;       // [ninst + 1] pass work items
   BoxDesc* dbox = nullptr;     // [ninst]
-  int* drstart = nullptr;      // [ninst + 1] grid rows
+  int* drstart = nullptr;      // [ninst + 1] items of the row kernels
   bool str[5] = {};            // the pass's lines are strided
   int grid = 0, rgrid = 0;     // CTAs of the contiguous passes and of the row kernels
   int grid_s = 0;              // CTAs of the strided passes
@@ -2419,12 +2484,13 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
       last.accumulate = 1;
       last.dstfix = B->ufix;
       last.fixf = B->fixf;
+      last.fixd = B->fixd;
       last.corr_max = B->nrm + 3;
     }
     const int pp = batch_pairs(B->logL);
     start[i + 1] = start[i] + ((plan0[i].npairs + pp - 1) / pp) * plan0[i].na;
     const int n1 = p->g.n + 1;
-    rstart[i + 1] = rstart[i] + (d == 2 ? n1 : n1 * n1);
+    rstart[i + 1] = rstart[i] + div_up(n1, 128) * div_up(d == 2 ? n1 : n1 * n1, kFixRows);
     box[i] = BoxDesc{p->g, FixStencil{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB}, B->multh2, B->kc, B->tol,
                      rhs[i], p->ugrid, B->work32, B->ufix, B->rfix, r32, B->fixd, B->fixf, B->nrm, B->conv,
                      tol_dev ? tol_dev + i : nullptr};
@@ -2433,9 +2499,11 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
   for (int i = 0; i < ninst; ++i) bb->steps = std::max(bb->steps, ps[i]->box->refine_steps);
   bb->npass = plan0[0].npass;
   std::vector<PassArgs> args;
-  for (int v = 0; v < 2 * bb->npass; ++v)
-    for (int i = 0; i < ninst; ++i)
-      args.push_back(v < bb->npass ? plan0[i].args[v] : plank[i].args[v - bb->npass]);
+  for (int v = 0; v < 3 * bb->npass; ++v)
+    for (int i = 0; i < ninst; ++i) {
+      args.push_back(v < bb->npass ? plan0[i].args[v] : plank[i].args[v % bb->npass]);
+      if (v == 3 * bb->npass - 1) args.back().uout = ps[i]->ugrid;   // the last step also writes the solution
+    }
   KFBI_CUDA(p0, dalloc(&bb->dargs, args.size()));
   KFBI_CUDA(p0, dalloc(&bb->dstart, ninst + 1));
   KFBI_CUDA(p0, dalloc(&bb->dbox, ninst));
@@ -2557,15 +2625,20 @@ kfbi_status batch_box_solve(kfbi_problem* p0, BatchBox* bb, const int* done, cud
   for (int v = 0; v < bb->npass; ++v)
     batch_launch_pass(p0, bb, v, bb->dargs + (size_t)v * ni, st);
   KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_check_batched<<<cb, 128, 0, st>>>(bb->dbox, ni, 0));
-  KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_fix_scale_batched<<<cb, 128, 0, st>>>(bb->dbox, ni));
-  KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 0));
+  auto rows = [&](auto kernel) {
+    KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, kernel<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, done));
+  };
+  rows(k_rows_batched<0>);
   for (int it = 1; it < bb->steps; ++it) {
-    KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 1));
+    const bool last = it + 1 == bb->steps;
+    rows(k_rows_batched<1>);
     for (int v = 0; v < bb->npass; ++v)
-      batch_launch_pass(p0, bb, v, bb->dargs + (size_t)(bb->npass + v) * ni, st);
+      batch_launch_pass(p0, bb, v, bb->dargs + (size_t)((last ? 2 : 1) * bb->npass + v) * ni, st);
+    // before the last step's check: the instances that stopped earlier
+    if (last) rows(k_rows_batched<2>);
     KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_check_batched<<<cb, 128, 0, st>>>(bb->dbox, ni, it));
   }
-  KFBI_LAUNCH(p0, KFBI_KC_RESIDUAL, k_rows_batched<<<bb->rgrid, 128, 0, st>>>(bb->dbox, bb->drstart, ni, 2));
+  if (bb->steps == 1) rows(k_rows_batched<3>);   // no refinement: every solution from u_fix
   KFBI_CUDA(p0, cudaGetLastError());
   return KFBI_OK;
 }
