@@ -351,4 +351,11 @@ __device__ inline void ls_grad_iface(const LevelSet& L, int k, const double* X, 
   ls_grad(L, X, g);
 }
 
+// H_k and its gradient: one evaluation of a sampled level set gives both
+__device__ inline double ls_H_grad_iface(const LevelSet& L, int k, const double* X, double* g) {
+  if (L.kind == KFBI_LS_GRID) return ls_sampled(L, X, g);
+  ls_grad_iface(L, k, X, g);
+  return ls_H_iface(L, k, X);
+}
+
 }  // namespace kfbi

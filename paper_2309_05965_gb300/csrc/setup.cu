@@ -214,9 +214,8 @@ __device__ double edge_root(const Grid& g, const LevelSet& L, int k, const doubl
   for (int it = 0; it < kRootMaxIt; ++it) {
     double X[3] = {xa[0], xa[1], xa[2]};
     X[r] = xa[r] + s;
-    double f = ls_H_iface(L, k, X);
     double gr[3];
-    ls_grad_iface(L, k, X, gr);
+    double f = ls_H_grad_iface(L, k, X, gr);
     double df = gr[r];
     bool done_zero = f == 0.0;
     bool same = (f < 0.0) == neg_a;
@@ -352,21 +351,31 @@ __global__ void __launch_bounds__(32 * kLineWarps) k_cand_fill(Grid g, LevelSet 
 
 // One thread per candidate: the root of H_k on its edge (Sec. 5.1), the unit
 // normal, and whether the point is a DOF of this family (|n_r| > cos alpha).
-__global__ void k_cand_roots(Grid g, LevelSet L, LineDesc D, int ncand, double cos_alpha,
-                             const int32_t* __restrict__ cline, const int32_t* __restrict__ cedge,
-                             const int32_t* __restrict__ ciface, double* __restrict__ cx,
-                             double* __restrict__ cn, int32_t* __restrict__ keep) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncand) return;
+struct RootSet {
+  LineDesc D;
+  int n;
+  const int32_t *line, *edge, *iface;
+  double *x, *nv;
+  int32_t* keep;
+};
+struct RootSets {
+  RootSet s[3];
+  int block[4];   // first block of each family, a warp per block
+};
+__global__ void k_cand_roots(Grid g, LevelSet L, RootSets R, double cos_alpha) {
+  const int f = (int)blockIdx.x >= R.block[2] ? 2 : (int)blockIdx.x >= R.block[1] ? 1 : 0;
+  const RootSet& S = R.s[f];
+  const int c = (blockIdx.x - R.block[f]) * blockDim.x + threadIdx.x;
+  if (c >= S.n) return;
   int ia, ib;
-  line_other(g, D, cline[c], &ia, &ib);
+  line_other(g, S.D, S.line[c], &ia, &ib);
   double X[3], nv[3];
-  const bool k = crossing_point(g, L, ciface[c], D, ia, ib, cedge[c], cos_alpha, X, nv);
+  const bool k = crossing_point(g, L, S.iface[c], S.D, ia, ib, S.edge[c], cos_alpha, X, nv);
   for (int e = 0; e < 3; ++e) {
-    cx[(size_t)e * ncand + c] = X[e];
-    cn[(size_t)e * ncand + c] = nv[e];
+    S.x[(size_t)e * S.n + c] = X[e];
+    S.nv[(size_t)e * S.n + c] = nv[e];
   }
-  keep[c] = k ? 1 : 0;
+  S.keep[c] = k ? 1 : 0;
 }
 
 // The kept candidates in candidate order are the family's DOFs in DOF order:
@@ -622,15 +631,37 @@ __device__ __forceinline__ double mono_lap(const double pw[3][5], int e, int d) 
 // R: upper triangle of A plus rdiag; reflector v_k in A[k.., k];
 // vn2[k] = 2 / |v_k|^2 (0 for a zero column), so that applying H_k costs a
 // multiply: an FP64 divide is a long sequence on GB300's FP64 pipe (2 lanes
-// per clock per SM), and one per column pair made the fits FP64-bound.
+// per clock per SM), and one per column pair made the fits FP64-bound.  A warp
+// instruction takes that pipe 16 cycles, so products and sums are explicit FMAs
+// (the unit is compiled without contraction) and the dot products of a reflector
+// with kHG columns are reduced together by warp_sum_group, 9 additions for 8
+// columns instead of 40: the trace fits of a 1024^2 update 582 -> 337 us.
 // ---------------------------------------------------------------------------
+constexpr int kHG = 8;
+
+// the sum over the warp of each of eight values; lane l gets that of value l / 4
+__device__ __forceinline__ double warp_sum_group(const double (&v)[kHG]) {
+  const int lane = threadIdx.x & 31;
+  const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0, h2 = (lane & 4) != 0;
+  double a[4], b[2];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    a[q] = (h4 ? v[q + 4] : v[q]) + __shfl_xor_sync(0xffffffffu, h4 ? v[q] : v[q + 4], 16);
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    b[q] = (h3 ? a[q + 2] : a[q]) + __shfl_xor_sync(0xffffffffu, h3 ? a[q] : a[q + 2], 8);
+  double c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+
 __device__ bool warp_householder(double* A, int lda, int m, int n, double* rdiag, double* vn2) {
   const int lane = threadIdx.x & 31;
   bool ok = true;
   for (int k = 0; k < n; ++k) {
     double* ak = A + (size_t)k * lda;
     double s = 0.0;
-    for (int i = k + lane; i < m; i += 32) s += ak[i] * ak[i];
+    for (int i = k + lane; i < m; i += 32) s = fma(ak[i], ak[i], s);
     s = warp_sum(s);
     double akk = ak[k];
     double nrm = sqrt(s);
@@ -650,33 +681,57 @@ __device__ bool warp_householder(double* A, int lda, int m, int n, double* rdiag
       ok = false;
       continue;
     }
-    for (int j = k + 1; j < n; ++j) {
-      double* aj = A + (size_t)j * lda;
-      double t = 0.0;
-      for (int i = k + lane; i < m; i += 32) t += ak[i] * aj[i];
-      t = warp_sum(t);
-      double f = t * rv;
-      for (int i = k + lane; i < m; i += 32) aj[i] -= f * ak[i];
-      __syncwarp();
+    for (int j = k + 1; j < n; j += kHG) {
+      const int nj = min(kHG, n - j);
+      double t[kHG];
+#pragma unroll
+      for (int q = 0; q < kHG; ++q) t[q] = 0.0;
+      for (int i = k + lane; i < m; i += 32) {
+        const double v = ak[i];
+#pragma unroll
+        for (int q = 0; q < kHG; ++q)
+          if (q < nj) t[q] = fma(v, A[(size_t)(j + q) * lda + i], t[q]);
+      }
+      const double f = -(warp_sum_group(t) * rv);
+      double fq[kHG];
+#pragma unroll
+      for (int q = 0; q < kHG; ++q) fq[q] = __shfl_sync(0xffffffffu, f, 4 * q);
+      for (int i = k + lane; i < m; i += 32) {
+        const double v = ak[i];
+#pragma unroll
+        for (int q = 0; q < kHG; ++q)
+          if (q < nj) {
+            double* a = A + (size_t)(j + q) * lda + i;
+            *a = fma(fq[q], v, *a);
+          }
+      }
     }
+    __syncwarp();
   }
   return ok;
 }
 
-// y <- H_k y for k = n-1..0 (y = Q y) or k = 0..n-1 (y = Q^T y).
-__device__ void warp_apply_q(const double* A, int lda, int m, int n, const double* vn2, double* y,
-                             bool transpose) {
+// y <- Q y for two vectors: H_k for k = n-1..0
+__device__ void warp_apply_q2(const double* A, int lda, int m, int n, const double* vn2, double* y0, double* y1) {
   const int lane = threadIdx.x & 31;
-  for (int kk = 0; kk < n; ++kk) {
-    int k = transpose ? kk : n - 1 - kk;
+  const bool up = (lane & 16) != 0;
+  for (int k = n - 1; k >= 0; --k) {
     if (!(vn2[k] > 0.0)) continue;
     const double* ak = A + (size_t)k * lda;
-    double t = 0.0;
-    for (int i = k + lane; i < m; i += 32) t += ak[i] * y[i];
-    t = warp_sum(t);
-    double f = t * vn2[k];
+    double t0 = 0.0, t1 = 0.0;
+    for (int i = k + lane; i < m; i += 32) {
+      t0 = fma(ak[i], y0[i], t0);
+      t1 = fma(ak[i], y1[i], t1);
+    }
+    double t = (up ? t1 : t0) + __shfl_xor_sync(0xffffffffu, up ? t0 : t1, 16);
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const double f = -(t * vn2[k]);
+    const double f0 = __shfl_sync(0xffffffffu, f, 0), f1 = __shfl_sync(0xffffffffu, f, 16);
     __syncwarp();
-    for (int i = k + lane; i < m; i += 32) y[i] -= f * ak[i];
+    for (int i = k + lane; i < m; i += 32) {
+      y0[i] = fma(f0, ak[i], y0[i]);
+      y1[i] = fma(f1, ak[i], y1[i]);
+    }
     __syncwarp();
   }
 }
@@ -790,7 +845,7 @@ __global__ void k_collocation_factor(Grid g, double kt, DofView V, int nb,
       const double rk = t / piv;
       col[k] = rk;
       for (int r = 0; r < n; ++r)
-        if (r != k) col[r] = col[r] - fcol[r] * rk;
+        if (r != k) col[r] = fma(-fcol[r], rk, col[r]);
     }
     __syncwarp();
   }
@@ -1126,12 +1181,14 @@ struct TraceParams {
 // within R_s, and nodes of another label within R_o that are irregular and
 // hold C^(t) (need == nullptr: one interface, where they always do) or, where
 // another interface is close (`close`), every node of another label within R_o.
+// ax (optional): the window's offsets xi per axis from the point (trace_axes),
+// which spares the FP64 divisions of every candidate.
 __device__ __forceinline__ bool trace_select(const Grid& g, const TraceParams& T, const double* p,
                                              const int* n0, int o, int tlab, bool close,
                                              const uint8_t* inside, const uint8_t* irr,
                                              const uint32_t* need,
                                              long long* node_out, double* xi_out, double* r2_out,
-                                             bool* across) {
+                                             bool* across, const double* ax = nullptr) {
   int off[3] = {0, 0, 0};
   int rem = o;
   for (int k = g.d - 1; k >= 0; --k) {
@@ -1142,7 +1199,8 @@ __device__ __forceinline__ bool trace_select(const Grid& g, const TraceParams& T
   for (int k = 0; k < g.d; ++k)
     if (idx[k] < 0 || idx[k] > g.n) return false;
   double xi[3] = {0.0, 0.0, 0.0};
-  for (int k = 0; k < g.d; ++k) xi[k] = (coord(g, idx[k]) - p[k]) / g.h;
+  for (int k = 0; k < g.d; ++k)
+    xi[k] = ax ? ax[k * T.wside + off[k] + T.win] : (coord(g, idx[k]) - p[k]) / g.h;
   double r2 = xi[0] * xi[0];
   r2 = r2 + xi[1] * xi[1];
   if (g.d == 3) r2 = r2 + xi[2] * xi[2];
@@ -1167,6 +1225,17 @@ __device__ __forceinline__ void trace_centre(const Grid& g, const DofView& V, in
   p[2] = g.d == 3 ? V.x[2][i] : 0.0;
   n0[0] = n0[1] = n0[2] = 0;
   for (int k = 0; k < g.d; ++k) n0[k] = (int)floor((p[k] - g.lo) / g.h + 0.5);
+}
+
+// (coord(n0 + o) - p) / h for every window offset o of each axis, by a warp; ax
+// holds d wside values
+__device__ __forceinline__ void trace_axes(const Grid& g, const TraceParams& T, const double* p, const int* n0,
+                                           double* ax) {
+  for (int e = threadIdx.x & 31; e < g.d * T.wside; e += 32) {
+    const int k = e / T.wside, o = e - k * T.wside - T.win;
+    ax[e] = (coord(g, n0[k] + o) - p[k]) / g.h;
+  }
+  __syncwarp();
 }
 
 // Several interfaces: a DOF of interface k is close to another interface if a
@@ -1201,26 +1270,35 @@ __global__ void k_trace_close(Grid g, TraceParams T, DofView V, int nb,
   close[i] = c;
 }
 
-__global__ void k_trace_count(Grid g, TraceParams T, DofView V, int nb,
+// A warp per (DOF, side), kCountWarps per CTA.  (A thread per pair walked its
+// window of wside^d candidates alone, two or three FP64 divisions each: 223 us
+// of a 1024^2 update, now 21.)
+constexpr int kCountWarps = 4;
+__global__ void __launch_bounds__(32 * kCountWarps) k_trace_count(Grid g, TraceParams T, DofView V, int nb,
                               const uint8_t* __restrict__ inside, const uint8_t* __restrict__ irr,
                               const uint8_t* __restrict__ close, const uint32_t* __restrict__ need,
                               int32_t* __restrict__ count) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  extern __shared__ double sm[];
+  double* ax = sm + (threadIdx.x >> 5) * g.d * T.wside;
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * kCountWarps + (threadIdx.x >> 5);
   if (t >= 2 * nb) return;
   int side = t / nb, i = t % nb;
   double p[3];
   int n0[3];
   trace_centre(g, V, i, p, n0);
+  trace_axes(g, T, p, n0, ax);
   const int tlab = side == 0 ? V.iface[i] + 1 : 0;
   const bool cl = close && close[i];
   int c = 0;
-  for (int o = 0; o < T.wtotal; ++o) {
+  for (int o = lane; o < T.wtotal; o += 32) {
     long long node;
     double xi[3], r2;
     bool across;
-    if (trace_select(g, T, p, n0, o, tlab, cl, inside, irr, need, &node, xi, &r2, &across)) ++c;
+    if (trace_select(g, T, p, n0, o, tlab, cl, inside, irr, need, &node, xi, &r2, &across, ax)) ++c;
   }
-  count[t] = c;
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) count[t] = c;
 }
 
 // Several interfaces: the entries the trace stencils of close DOFs need,
@@ -1268,7 +1346,8 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
   double* rdiag = wt + lda;                  // n
   double* vn2 = rdiag + n;                   // n
   double* z = vn2 + n;                       // 2n
-  int* nodes = (int*)(z + 2 * n);            // lda ints
+  double* ax = z + 2 * n;                    // d wside
+  int* nodes = (int*)(ax + g.d * T.wside);   // lda ints
   int* acr = nodes + lda;                    // lda ints
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x;
@@ -1281,6 +1360,7 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
   for (int k = 0; k < d; ++k) n0[k] = (int)floor((p[k] - g.lo) / g.h + 0.5);
   const int tlab = side == 0 ? V.iface[i] + 1 : 0;
   const bool cl = close && close[i];
+  trace_axes(g, T, p, n0, ax);
   // ordered compaction of the selected window offsets
   int m = 0;
   for (int base = 0; base < T.wtotal; base += 32) {
@@ -1289,7 +1369,7 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
     double xi[3] = {0.0, 0.0, 0.0}, r2 = 0.0;
     bool across = false;
     bool sel = o < T.wtotal && trace_select(g, T, p, n0, o, tlab, cl, inside, irr, need, &node,
-                                            xi, &r2, &across);
+                                            xi, &r2, &across, ax);
     unsigned ball = __ballot_sync(0xffffffffu, sel);
     if (sel) {
       int pos = m + __popc(ball & ((1u << lane) - 1u));
@@ -1308,21 +1388,33 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
   __syncwarp();
   m = min(m, mmax);
   bool ok = m >= n && warp_householder(A, lda, m, n, rdiag, vn2);
-  // z0 = R^{-T} e_0, z1 = R^{-T} c_n  (forward substitution, lane 0)
-  if (lane == 0) {
-    for (int k = 0; k < n; ++k) {
-      double c0 = (k == 0) ? 1.0 : 0.0;
-      double c1 = 0.0;
-      if (k >= 1 && k <= d) c1 = nv[k - 1] / g.h;
-      double a0 = c0, a1 = c1;
-      for (int j = 0; j < k; ++j) {
-        double rjk = A[(size_t)k * lda + j];
-        a0 -= rjk * z[j];
-        a1 -= rjk * z[n + j];
+  // z0 = R^{-T} e_0, z1 = R^{-T} c_n: forward substitution by columns, lane k
+  // (and k + 32) holding the sums of unknowns k
+  {
+    double a0[2], a1[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int k = lane + 32 * q;
+      a0[q] = k == 0 ? 1.0 : 0.0;
+      a1[q] = k >= 1 && k <= d ? nv[k - 1] / g.h : 0.0;
+    }
+    for (int j = 0; j < n; ++j) {
+      const double ir = 1.0 / rdiag[j];
+      const double z0 = __shfl_sync(0xffffffffu, j < 32 ? a0[0] : a0[1], j & 31) * ir;
+      const double z1 = __shfl_sync(0xffffffffu, j < 32 ? a1[0] : a1[1], j & 31) * ir;
+      if (lane == 0) {
+        z[j] = z0;
+        z[n + j] = z1;
       }
-      const double ir = 1.0 / rdiag[k];
-      z[k] = a0 * ir;
-      z[n + k] = a1 * ir;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int k = lane + 32 * q;
+        if (k > j && k < n) {
+          const double r = A[(size_t)k * lda + j];
+          a0[q] = fma(-r, z0, a0[q]);
+          a1[q] = fma(-r, z1, a1[q]);
+        }
+      }
     }
   }
   __syncwarp();
@@ -1331,8 +1423,7 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
     y1[r] = r < n ? z[n + r] : 0.0;
   }
   __syncwarp();
-  warp_apply_q(A, lda, m, n, vn2, y0, false);
-  warp_apply_q(A, lda, m, n, vn2, y1, false);
+  warp_apply_q2(A, lda, m, n, vn2, y0, y1);
   int off = ptr_all[t];
   for (int r = lane; r < m; r += 32) {
     double a = y0[r] * wt[r], b = y1[r] * wt[r];
@@ -1492,9 +1583,10 @@ kfbi_status build_geometry(kfbi_problem* p) {
   auto free_cand = [&]() {
     for (int r = 0; r < 3; ++r) C[r] = Cand();
   };
-  int32_t* ccnt = nullptr;
-  KFBI_CUDA(p, galloc(p, &ccnt, nlines));
-  int32_t base = 0;
+  // each step is enqueued for all families before the host waits for its
+  // counts, and the root iterations of all families are one launch: a family's
+  // few warps are bound by the latency of their FP64 chains (two families of a
+  // sampled level set at 1024^2: 443 -> 190 us with one evaluation for value and gradient)
   for (int r = 0; r < d; ++r) {
     D[r].r = r;
     int o[2], no = 0;
@@ -1506,34 +1598,54 @@ kfbi_status build_geometry(kfbi_problem* p) {
     D[r].sa = strides[o[0]];
     D[r].sb = d == 3 ? strides[o[1]] : 0;
     Cand& c = C[r];
+    int32_t* ccnt = nullptr;
+    KFBI_CUDA(p, galloc(p, &ccnt, nlines));
     k_cand_count<<<div_up(nlines, kLineWarps), 32 * kLineWarps, 0, st>>>(g, L, D[r], p->inside, multi,
                                                                         nlines, ccnt);
     KFBI_CUDA(p, cudaGetLastError());
     KFBI_CUDA(p, galloc(p, &c.start, nlines + 1));
     KFBI_TRY(scan_exclusive(p, ccnt, c.start, nlines, 0, st));
     KFBI_CUDA(p, cudaMemcpyAsync(&c.n, c.start + nlines, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    KFBI_CUDA(p, cudaStreamSynchronize(st));
+  }
+  KFBI_CUDA(p, cudaStreamSynchronize(st));
+  RootSets RS;
+  memset(&RS, 0, sizeof(RS));
+  for (int r = 0; r < 3; ++r) {
+    Cand& c = C[r];
+    RS.block[r + 1] = RS.block[r] + div_up(c.n, 32);
+    if (r >= d) continue;
     KFBI_CUDA(p, galloc(p, &c.kpos, c.n + 1));
-    if (c.n > 0) {
-      KFBI_CUDA(p, galloc(p, &c.line, c.n));
-      KFBI_CUDA(p, galloc(p, &c.edge, c.n));
-      KFBI_CUDA(p, galloc(p, &c.iface, c.n));
-      KFBI_CUDA(p, galloc(p, &c.keep, c.n));
-      KFBI_CUDA(p, galloc(p, &c.x, 3 * (size_t)c.n));
-      KFBI_CUDA(p, galloc(p, &c.nv, 3 * (size_t)c.n));
-      k_cand_fill<<<div_up(nlines, kLineWarps), 32 * kLineWarps, 0, st>>>(g, L, D[r], p->inside, multi,
-                                                                         nlines, c.start, c.line, c.edge,
-                                                                         c.iface);
-      // one warp per block: the FP64-bound root iterations spread over all SMs
-      k_cand_roots<<<div_up(c.n, 32), 32, 0, st>>>(g, L, D[r], c.n, p->cos_alpha, c.line, c.edge, c.iface,
-                                                   c.x, c.nv, c.keep);
-      KFBI_CUDA(p, cudaGetLastError());
-      KFBI_TRY(scan_exclusive(p, c.keep, c.kpos, c.n, 0, st));
-      KFBI_CUDA(p, cudaMemcpyAsync(&c.kept, c.kpos + c.n, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      KFBI_CUDA(p, cudaStreamSynchronize(st));
-    } else {
+    if (c.n == 0) {
       KFBI_CUDA(p, cudaMemsetAsync(c.kpos, 0, sizeof(int32_t), st));
+      continue;
     }
+    KFBI_CUDA(p, galloc(p, &c.line, c.n));
+    KFBI_CUDA(p, galloc(p, &c.edge, c.n));
+    KFBI_CUDA(p, galloc(p, &c.iface, c.n));
+    KFBI_CUDA(p, galloc(p, &c.keep, c.n));
+    KFBI_CUDA(p, galloc(p, &c.x, 3 * (size_t)c.n));
+    KFBI_CUDA(p, galloc(p, &c.nv, 3 * (size_t)c.n));
+    k_cand_fill<<<div_up(nlines, kLineWarps), 32 * kLineWarps, 0, st>>>(g, L, D[r], p->inside, multi,
+                                                                       nlines, c.start, c.line, c.edge,
+                                                                       c.iface);
+    KFBI_CUDA(p, cudaGetLastError());
+    RS.s[r] = RootSet{D[r], c.n, c.line, c.edge, c.iface, c.x, c.nv, c.keep};
+  }
+  if (RS.block[3] > 0) {
+    // one warp per block: the FP64-bound root iterations spread over all SMs
+    k_cand_roots<<<RS.block[3], 32, 0, st>>>(g, L, RS, p->cos_alpha);
+    KFBI_CUDA(p, cudaGetLastError());
+  }
+  for (int r = 0; r < d; ++r) {
+    Cand& c = C[r];
+    if (c.n == 0) continue;
+    KFBI_TRY(scan_exclusive(p, c.keep, c.kpos, c.n, 0, st));
+    KFBI_CUDA(p, cudaMemcpyAsync(&c.kept, c.kpos + c.n, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  }
+  KFBI_CUDA(p, cudaStreamSynchronize(st));
+  int32_t base = 0;
+  for (int r = 0; r < d; ++r) {
+    Cand& c = C[r];
     KFBI_CUDA(p, galloc(p, &p->line_start[r], nlines + 1));
     k_cand_line_start<<<div_up(nlines + 1, 256), 256, 0, st>>>(nlines, base, c.start, c.kpos,
                                                                p->line_start[r]);
@@ -1785,8 +1897,8 @@ kfbi_status build_geometry(kfbi_problem* p) {
   int32_t *tcnt = nullptr, *tptr = nullptr;
   KFBI_CUDA(p, galloc(p, &tcnt, 2 * nb));
   KFBI_CUDA(p, galloc(p, &tptr, 2 * nb + 1));
-  k_trace_count<<<div_up(2 * nb, 128), 128, 0, st>>>(g, TP, V, nb, p->inside, p->irr_flag, close,
-                                                       need, tcnt);
+  k_trace_count<<<div_up(2 * nb, kCountWarps), 32 * kCountWarps, sizeof(double) * kCountWarps * d * TP.wside, st>>>(
+      g, TP, V, nb, p->inside, p->irr_flag, close, need, tcnt);
   KFBI_TRY(scan_exclusive(p, tcnt, tptr, 2 * nb, 0, st));
   KFBI_CUDA(p, cudaGetLastError());
   std::vector<int32_t> hptr(2 * nb + 1), hcnt(2 * nb);
@@ -1809,7 +1921,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
     double alpha = p->cfg.kind == KFBI_DIRICHLET_INTERIOR ? 0.5 : 0.0;
     double beta = p->cfg.kind == KFBI_DIRICHLET_INTERIOR ? 0.0 : 0.5;
     const int lda = mmax + 1;
-    size_t smem = sizeof(double) * ((size_t)lda * nc + 3 * (size_t)lda + 4 * nc) +
+    size_t smem = sizeof(double) * ((size_t)lda * nc + 3 * (size_t)lda + 4 * nc + d * TP.wside) +
                   sizeof(int) * 2 * (size_t)lda;
     int dev = 0, optin = 0;
     KFBI_CUDA(p, cudaGetDevice(&dev));
