@@ -142,7 +142,8 @@ typedef struct {
                              before application j inside kfbi_gmres_solve the
                              refinement stops at max(box_rtol, omega rtol ||b|| /
                              ||r_j||) (relaxation as the residual falls, after
-                             Simoncini & Szyld 2003); right-hand side, starts,
+                             Simoncini & Szyld 2003; half of omega for the
+                             interface kinds); right-hand side, starts,
                              restarts and evaluation stay at box_rtol           */
 } kfbi_config;
 

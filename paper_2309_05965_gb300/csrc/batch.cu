@@ -248,7 +248,7 @@ kfbi_status kfbi_create_batch(kfbi_problem* const* problems, int count, kfbi_bat
     return bail(s);
   // per-instance refinement tolerances of the loop's box solves (each
   // problem's box_rtol, relaxed inside GMRES when relax > 0)
-  b->omega = p0->cfg.relax;
+  b->omega = relax_omega(p0);
   {
     std::vector<double> base(count);
     for (int k = 0; k < count; ++k) base[k] = box_tol(b->ps[k]);

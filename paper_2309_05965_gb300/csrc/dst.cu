@@ -71,6 +71,7 @@ struct BoxSolver {
   double* tol_dev = nullptr;  // the refinement tolerance the checks read (relaxed inside GMRES)
   int* conv = nullptr;        // device flag
   int refine_steps = 4;
+  double margin = 10.0;       // first_margin of the problem
   double tol = 1e-13;
   // exact residual of the mixed path in fixed point: mult h^2 A_h = S - kappa h^2 K
   // with S integer weights w[c] by the number c of nonzero offsets and
@@ -1008,11 +1009,11 @@ __global__ void __launch_bounds__(kBatchPassThreads, STR ? 6 : 5)
 
 // The check after refinement step `step` (0: the first FP32 solve): stop when
 // the last correction max|delta| <= tol max|u|.  After the first solve there
-// is no correction yet; it stops there only when ten times the relative size
-// of the first correction observed in an earlier solve on this grid (nrm[8],
+// is no correction yet; it stops there only when `margin` times the relative
+// size of the first correction observed in an earlier solve on this grid (nrm[8],
 // an estimate of the FP32 solve's error, 1 until one is observed) is within
 // tol, which a relaxed GMRES tolerance can reach.  The first correction of
-// every solve updates that estimate.
+// every solve updates that estimate.  See first_margin for the margin.
 // The kernel after the step (the next residual) decides: every CTA from the
 // step's own maxima, so that no launch of one thread stands between them (19
 // launches instead of 24 with the scale in k_fix0, five steps enqueued: 1024^2
@@ -1021,6 +1022,7 @@ struct StepCheck {
   unsigned long long* nrm;
   const double* tol;
   int* conv;
+  double margin;
   int step;        // the step to check
 };
 
@@ -1033,7 +1035,7 @@ __device__ __forceinline__ bool step_stop(const StepCheck& C, bool keeper) {
   if (done) return true;
   const double dm = __longlong_as_double((long long)db), um = __longlong_as_double((long long)ub);
   bool stop = dm <= tol * um;
-  if (C.step == 0 && 10.0 * __longlong_as_double((long long)eb) <= tol) stop = true;
+  if (C.step == 0 && C.margin * __longlong_as_double((long long)eb) <= tol) stop = true;
   if (keeper) {
     C.nrm[2] = db;
     C.nrm[5] = ub;
@@ -1415,7 +1417,7 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
 // launch of the fixed-point residual for the grid's dimension
 void launch_res_fix(kfbi_problem* p, const Grid& g, const FixStencil& W, const long long* R, const long long* u,
                     const double* fixd, const float* fixf, float* r32, const int* skip, double* uout,
-                    cudaStream_t st, const StepCheck& chk = StepCheck{nullptr, nullptr, nullptr, 0}) {
+                    cudaStream_t st, const StepCheck& chk = StepCheck{nullptr, nullptr, nullptr, 0.0, 0}) {
   if (g.d == 2) {
     const dim3 grid((unsigned)div_up(g.n + 1, 128), (unsigned)div_up(g.n + 1, kResRows), 1u);
     KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_res_fix2<<<grid, 128, 0, st>>>(g, W, R, u, fixd, fixf, r32, skip, uout,
@@ -1682,6 +1684,17 @@ void mg_destroy(kfbi_problem* p);
 kfbi_status mg_solve(kfbi_problem* p, const double* rhs, double* u);
 kfbi_status mg_last_residual(kfbi_problem* p, double* rel, int* converged);
 
+// Margin between the error estimate of an unrefined FP32 solve and the relaxed
+// tolerance it may stop at: 10, times the contrast of an interface problem, whose
+// operator nearly annihilates the constants (by the contrast): the mean of the
+// rounding errors, of which the estimate (a maximum norm) says nothing, reaches the
+// solution larger by that.  See relax_omega for figures.
+static double first_margin(const kfbi_problem* p) {
+  if (p->cfg.kind != KFBI_INTERFACE_MU && p->cfg.kind != KFBI_INTERFACE_GENERAL) return 10.0;
+  const double a = std::fabs(p->cfg.sigma_in), b = std::fabs(p->cfg.sigma_out);
+  return 10.0 * std::max(a / b, b / a);
+}
+
 kfbi_status box_create(kfbi_problem* p) {
   if (p->cfg.box_solver == KFBI_BOX_MG) return mg_create(p);
   const Grid g = p->g;
@@ -1793,6 +1806,7 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, dalloc(&B->conv, 1));
   KFBI_CUDA(p, dalloc(&B->tol_dev, 1));
   B->tol = p->cfg.box_rtol > 0 ? p->cfg.box_rtol : 1e-13;
+  B->margin = first_margin(p);
   KFBI_CUDA(p, cudaMemcpy(B->tol_dev, &B->tol, sizeof(double), cudaMemcpyHostToDevice));
   B->refine_steps = p->cfg.box_max_iters > 0 ? std::min(p->cfg.box_max_iters, kMaxSteps) : 5;
   int dev = 0, optin = 0;
@@ -1922,7 +1936,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   launch_fix0(p, g, B->work32, rhs, slot + 1, B->multh2, B->kc, B->fixd, B->fixf, B->ufix, B->rfix,
               B->refine_steps > 1 ? nullptr : u, st);
   if (B->refine_steps == 1)
-    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, 0}));
+    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, 0}));
   float* r32 = reinterpret_cast<float*>(B->res);
   PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, nullptr);
   {
@@ -1937,7 +1951,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   const FixStencil W{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB};
   for (int it = 1; it < B->refine_steps; ++it) {
     launch_res_fix(p, g, W, B->rfix, B->ufix, B->fixd, B->fixf, r32, B->conv, u, st,
-                   StepCheck{B->nrm, B->tol_dev, B->conv, it - 1});
+                   StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, it - 1});
     PassArgs& last = PK.args[PK.npass - 1];
     last.corr_max = slot + 2 * it;
     last.uout = it + 1 < B->refine_steps ? nullptr : u;   // the last step also writes the FP64 solution
@@ -2254,7 +2268,7 @@ namespace {
 struct BoxDesc {
   Grid g;
   FixStencil W;
-  double multh2, kc, tol;
+  double multh2, kc, tol, margin;
   const double* R;         // right-hand side (FP64 grid)
   double* u;               // solution (FP64 grid)
   const float* u0;         // first FP32 solve (the work grid)
@@ -2299,7 +2313,7 @@ __global__ void k_check_batched(const BoxDesc* __restrict__ D, int ninst, int st
   nrm[2] = nrm[3];
   nrm[5] = nrm[4];
   bool stop = dm <= tol * um;
-  if (step == 0 && 10.0 * __longlong_as_double((long long)nrm[8]) <= tol) stop = true;
+  if (step == 0 && D[i].margin * __longlong_as_double((long long)nrm[8]) <= tol) stop = true;
   if (step == 1 && um > 0.0) nrm[8] = (unsigned long long)__double_as_longlong(dm / um);
   if (stop) *D[i].conv = 1;
   nrm[3] = 0ull;
@@ -2492,7 +2506,7 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
     const int n1 = p->g.n + 1;
     rstart[i + 1] = rstart[i] + div_up(n1, 128) * div_up(d == 2 ? n1 : n1 * n1, kFixRows);
     box[i] = BoxDesc{p->g, FixStencil{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB}, B->multh2, B->kc, B->tol,
-                     rhs[i], p->ugrid, B->work32, B->ufix, B->rfix, r32, B->fixd, B->fixf, B->nrm, B->conv,
+                     B->margin, rhs[i], p->ugrid, B->work32, B->ufix, B->rfix, r32, B->fixd, B->fixf, B->nrm, B->conv,
                      tol_dev ? tol_dev + i : nullptr};
   }
   bb->steps = 0;

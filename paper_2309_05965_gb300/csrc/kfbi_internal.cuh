@@ -366,6 +366,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u);
 kfbi_status box_last_residual(kfbi_problem* p, double* rel, int* converged);
 kfbi_status box_steps(kfbi_problem* p, int* steps, int* cycles);
 double* box_tol_dev(kfbi_problem* p);
+double relax_omega(const kfbi_problem* p);
 double box_tol(const kfbi_problem* p);
 kfbi_status box_tol_reset(kfbi_problem* p);
 kfbi_status box_steps_reset(kfbi_problem* p);
