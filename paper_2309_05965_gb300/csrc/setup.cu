@@ -901,31 +901,38 @@ __global__ void k_irregular_flags(Grid g, const uint8_t* __restrict__ inside,
 }
 
 // rows along the last axis
+// A warp per grid row, kLineWarps per CTA (a thread per row read its bytes one
+// by one: 40 and 75 us for the two kernels of a 1024^2 update, now 4.4 and 8.7).
 __global__ void k_row_count(Grid g, const uint8_t* __restrict__ flag, int nrows,
                             int32_t* __restrict__ count) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = blockIdx.x * kLineWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= nrows) return;
   const uint8_t* f = flag + (long long)r * (g.n + 1);
   int c = 0;
-  for (int j = 0; j <= g.n; ++j) c += f[j];
-  count[r] = c;
+  for (int j = lane; j <= g.n; j += 32) c += f[j];
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) count[r] = c;
 }
 
 __global__ void k_row_fill(Grid g, const uint8_t* __restrict__ flag,
                            const uint8_t* __restrict__ inside, int nrows,
                            const int32_t* __restrict__ start, int32_t* __restrict__ lin,
                            uint8_t* __restrict__ irr_inside, int32_t* __restrict__ map) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = blockIdx.x * kLineWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= nrows) return;
-  long long base = (long long)r * (g.n + 1);
+  const long long base = (long long)r * (g.n + 1);
   int pos = start[r];
-  for (int j = 0; j <= g.n; ++j) {
-    if (flag[base + j]) {
-      lin[pos] = (int32_t)(base + j);
-      irr_inside[pos] = inside[base + j];
-      map[base + j] = pos;
-      ++pos;
+  for (int j0 = 0; j0 <= g.n; j0 += 32) {
+    const int j = j0 + lane;
+    const bool on = j <= g.n && flag[base + j];
+    const unsigned ball = __ballot_sync(0xffffffffu, on);
+    if (on) {
+      const int at = pos + __popc(ball & ((1u << lane) - 1u));
+      lin[at] = (int32_t)(base + j);
+      irr_inside[at] = inside[base + j];
+      map[base + j] = at;
     }
+    pos += __popc(ball);
   }
 }
 
@@ -974,59 +981,66 @@ __device__ __forceinline__ double dist2(const DofView& V, int d, int q, const do
 
 // Per correction entry (node, interface k): the closest primary point among
 // the DOFs of interface k.
+// A warp per entry, its lanes over the 7^d cells: minima do not depend on the
+// order.  (1024^2 update: 53 us with a thread per entry, now 16.)
 __global__ void k_closest(Grid g, DofView V, int nb, int nent, const int32_t* __restrict__ lin,
                           const int32_t* __restrict__ ent_iface,
                           const int32_t* __restrict__ cstart, const int32_t* __restrict__ items,
                           int32_t* __restrict__ owner, int* flags) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
+  const int q = blockIdx.x * kLineWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (q >= nent) return;
   const int ifc = ent_iface[q];
-  const int K = 3;
+  const int K = 3, S = 2 * K + 1;
   int idx[3];
   node_multi(g, lin[q], idx);
   double X[3] = {coord(g, idx[0]), coord(g, idx[1]), g.d == 3 ? coord(g, idx[2]) : 0.0};
   int c0[3] = {min(idx[0], g.n - 1), min(idx[1], g.n - 1), g.d == 3 ? min(idx[2], g.n - 1) : 0};
-  double eps = kTieEps * g.h * g.h;
+  const double eps = kTieEps * g.h * g.h;
+  const int ncell = g.d == 3 ? S * S * S : S * S;
   double dmin = INFINITY;
-  int lo3 = g.d == 3 ? -K : 0, hi3 = g.d == 3 ? K : 0;
   for (int pass = 0; pass < 2; ++pass) {
     int best = INT_MAX;
-    for (int a = -K; a <= K; ++a)
-      for (int b = -K; b <= K; ++b)
-        for (int c = lo3; c <= hi3; ++c) {
-          int cc[3] = {c0[0] + a, c0[1] + b, c0[2] + c};
-          if (cc[0] < 0 || cc[0] >= g.n || cc[1] < 0 || cc[1] >= g.n) continue;
-          if (g.d == 3 && (cc[2] < 0 || cc[2] >= g.n)) continue;
-          long long ci = cell_index(g, cc);
-          for (int t = cstart[ci]; t < cstart[ci + 1]; ++t) {
-            int i = items[t];
-            if (V.iface[i] != ifc) continue;
-            double d2 = dist2(V, g.d, i, X);
-            if (pass == 0) dmin = fmin(dmin, d2);
-            else if (d2 <= dmin + eps && i < best) best = i;
-          }
-        }
+    for (int e = lane; e < ncell; e += 32) {
+      const int c2 = g.d == 3 ? e % S : 0, ab = g.d == 3 ? e / S : e;
+      const int cc[3] = {c0[0] + ab / S - K, c0[1] + ab % S - K, c0[2] + (g.d == 3 ? c2 - K : 0)};
+      if (cc[0] < 0 || cc[0] >= g.n || cc[1] < 0 || cc[1] >= g.n) continue;
+      if (g.d == 3 && (cc[2] < 0 || cc[2] >= g.n)) continue;
+      const long long ci = cell_index(g, cc);
+      for (int t = cstart[ci]; t < cstart[ci + 1]; ++t) {
+        const int i = items[t];
+        if (V.iface[i] != ifc) continue;
+        const double d2 = dist2(V, g.d, i, X);
+        if (pass == 0) dmin = fmin(dmin, d2);
+        else if (d2 <= dmin + eps && i < best) best = i;
+      }
+    }
+    if (pass == 0)
+      for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
     if (pass == 0 && !(dmin < (double)(K * K) * g.h * g.h)) {
       // nothing certain within K h: global search
-      atomicAdd(&flags[kFlagClosestFallback], 1);
+      if (lane == 0) atomicAdd(&flags[kFlagClosestFallback], 1);
       dmin = INFINITY;
-      for (int i = 0; i < nb; ++i)
+      for (int i = lane; i < nb; i += 32)
         if (V.iface[i] == ifc) dmin = fmin(dmin, dist2(V, g.d, i, X));
+      for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
       int b2 = INT_MAX;
-      for (int i = 0; i < nb; ++i)
-        if (V.iface[i] == ifc && dist2(V, g.d, i, X) <= dmin + eps) {
-          b2 = i;
-          break;
+      for (int i = lane; i < nb; i += 32)
+        if (V.iface[i] == ifc && dist2(V, g.d, i, X) <= dmin + eps && i < b2) b2 = i;
+      b2 = __reduce_min_sync(0xffffffffu, b2);
+      if (lane == 0) {
+        if (b2 == INT_MAX) {
+          // no DOF on this interface at all: reported, and an in-range owner
+          flag_min(flags, kFlagNoOwner, q + 1);
+          b2 = 0;
         }
-      if (b2 == INT_MAX) {
-        // no DOF on this interface at all: reported, and an in-range owner
-        flag_min(flags, kFlagNoOwner, q + 1);
-        b2 = 0;
+        owner[q] = b2;
       }
-      owner[q] = b2;
       return;
     }
-    if (pass == 1) owner[q] = best;
+    if (pass == 1) {
+      best = __reduce_min_sync(0xffffffffu, best);
+      if (lane == 0) owner[q] = best;
+    }
   }
 }
 
@@ -1796,7 +1810,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
   KFBI_CUDA(p, galloc(p, &rstart, nrows + 1));
   KFBI_CUDA(p, galloc(p, &map, nodes));
   KFBI_CUDA(p, cudaMemsetAsync(map, 0xff, sizeof(int32_t) * nodes, st));
-  k_row_count<<<div_up(nrows, 128), 128, 0, st>>>(g, p->irr_flag, nrows, rcnt);
+  k_row_count<<<div_up(nrows, kLineWarps), 32 * kLineWarps, 0, st>>>(g, p->irr_flag, nrows, rcnt);
   KFBI_TRY(scan_exclusive(p, rcnt, rstart, nrows, 0, st));
   int32_t nirr = 0;
   KFBI_CUDA(p, cudaMemcpyAsync(&nirr, rstart + nrows, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1805,7 +1819,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
   if (nirr == 0) return fail(p, KFBI_ERR_GEOMETRY, "no irregular nodes");
   KFBI_CUDA(p, galloc(p, &p->irr_lin, nirr));
   KFBI_CUDA(p, galloc(p, &p->irr_inside, nirr));
-  k_row_fill<<<div_up(nrows, 128), 128, 0, st>>>(g, p->irr_flag, p->inside, nrows, rstart,
+  k_row_fill<<<div_up(nrows, kLineWarps), 32 * kLineWarps, 0, st>>>(g, p->irr_flag, p->inside, nrows, rstart,
                                                   p->irr_lin, p->irr_inside, map);
   KFBI_CUDA(p, cudaGetLastError());
 
@@ -1874,7 +1888,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
     k_cell_count<<<div_up(nb, 256), 256, 0, st>>>(g, V, nb, ccnt);
     KFBI_TRY(scan_exclusive(p, ccnt, cstart, (int)ncell, 0, st));
     k_cell_fill<<<div_up(nb, 256), 256, 0, st>>>(g, V, nb, cstart, cur, items);
-    k_closest<<<div_up(nent, 128), 128, 0, st>>>(g, V, nb, nent, p->ent_lin, p->ent_iface, cstart,
+    k_closest<<<div_up(nent, kLineWarps), 32 * kLineWarps, 0, st>>>(g, V, nb, nent, p->ent_lin, p->ent_iface, cstart,
                                                  items, p->ent_owner, p->d_flags);
     KFBI_CUDA(p, cudaGetLastError());
   }
