@@ -8,6 +8,8 @@
 //   3.4   corrected interpolation of the traces (Sec. 5.5), fused with the BIE
 //         combination y = alpha x + beta t.
 // All arithmetic is FP64.
+#include <cooperative_groups.h>
+
 #include "kfbi_internal.cuh"
 
 namespace kfbi {
@@ -374,23 +376,32 @@ __global__ void k_trace_op(int nb, TraceCSR tp, TraceCSR tm, const double* __res
   if (lane == 0) y[i] = (x ? alpha * x[i] : 0.0) + beta * acc;
 }
 
-// y -= mean(y): one CTA, each thread a strided partial sum, then a fixed
-// warp/CTA tree, so the result does not depend on timing.
-__global__ void __launch_bounds__(1024) k_mean_project(int n, double* __restrict__ y) {
+// y -= mean(y) by one cluster of kMeanCtas CTAs: each thread a strided partial
+// sum, a fixed warp/CTA tree, then the CTAs' sums in rank order through
+// distributed shared memory, so the result does not depend on timing.  (One CTA
+// is bound by the latency of its own loads: 29 us at N_b = 29,700, 12.8 in a cluster.)
+constexpr int kMeanCtas = 8;
+__global__ void __cluster_dims__(kMeanCtas, 1, 1) __launch_bounds__(1024) k_mean_project(int n, double* __restrict__ y) {
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   __shared__ double part[32];
+  __shared__ double sum;
+  const int stride = kMeanCtas * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += y[i];
+  for (int i = t0; i < n; i += stride) s += y[i];
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x < 32) {
     double t = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
     t = warp_sum(t);
-    if (threadIdx.x == 0) part[0] = t;
+    if (threadIdx.x == 0) sum = t;
   }
-  __syncthreads();
-  const double m = part[0] / n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) y[i] -= m;
+  cluster.sync();
+  double t = 0.0;
+  for (int r = 0; r < kMeanCtas; ++r) t += *cluster.map_shared_rank(&sum, r);
+  const double m = t / n;
+  for (int i = t0; i < n; i += stride) y[i] -= m;
+  cluster.sync();   // no CTA leaves while another reads its sum
 }
 
 // ---- general interface problem, eq. (bie-ifp-1) ----------------------------
@@ -576,7 +587,7 @@ kfbi_status launch_operator_trace(kfbi_problem* p, const double* u, const double
 
 kfbi_status launch_mean_project(kfbi_problem* p, double* y) {
   if (p->cfg.kind != KFBI_NEUMANN_INTERIOR || p->kt != 0.0) return KFBI_OK;
-  KFBI_LAUNCH(p, KFBI_KC_TRACE, k_mean_project<<<1, 1024, 0, p->stream>>>(p->nb, y));
+  KFBI_LAUNCH(p, KFBI_KC_TRACE, k_mean_project<<<kMeanCtas, 1024, 0, p->stream>>>(p->nb, y));
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
 }
