@@ -213,12 +213,22 @@ __global__ void k_traces4(int nb, TraceCSR tp, TraceCSR tm, const double* __rest
   int lane = threadIdx.x & 31;
   if (i >= nb) return;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int e = tp.ptr[i] + lane; e < tp.ptr[i + 1]; e += 32) {
+  for (int e = tp.ptr[i] + lane; e < tp.mid[i]; e += 32) {
+    const double w = u[tp.node[e]];
+    s[0] += tp.wv[e] * w;
+    s[1] += tp.wn[e] * w;
+  }
+  for (int e = tp.mid[i] + lane; e < tp.ptr[i + 1]; e += 32) {
     const double w = trace_datum<MULTI, false>(tp, e, u, cv);
     s[0] += tp.wv[e] * w;
     s[1] += tp.wn[e] * w;
   }
-  for (int e = tm.ptr[i] + lane; e < tm.ptr[i + 1]; e += 32) {
+  for (int e = tm.ptr[i] + lane; e < tm.mid[i]; e += 32) {
+    const double w = u[tm.node[e]];
+    s[2] += tm.wv[e] * w;
+    s[3] += tm.wn[e] * w;
+  }
+  for (int e = tm.mid[i] + lane; e < tm.ptr[i + 1]; e += 32) {
     const double w = trace_datum<MULTI, true>(tm, e, u, cv);
     s[2] += tm.wv[e] * w;
     s[3] += tm.wn[e] * w;
@@ -297,13 +307,14 @@ __device__ __forceinline__ double df_value(DFlt a) { return (double)a.hi + (doub
 // One stencil entry into the pair sums of the value and normal-derivative
 // weights: w (u + corrections), the corrections C as in trace_datum, each its
 // own product.
-template <bool MULTI, bool MINUS>
+template <bool MULTI, bool MINUS, bool CORR>
 __device__ __forceinline__ void trace_entry2_df(const TraceCSR& T, int e, const double* __restrict__ u,
                                                 const double* __restrict__ cv, DFlt& av, DFlt& an) {
   const float2 wv = T.wv2[e], wn = T.wn2[e];
   const float2 uu = split_f64(u[T.node[e]]);
   df_fma(av, wv, uu);
   df_fma(an, wn, uu);
+  if (!CORR) return;
   const int j = T.irr[e];
   if (!MULTI) {
     if (j >= 0) {
@@ -338,10 +349,14 @@ __global__ void k_traces4_df(int nb, TraceCSR tp, TraceCSR tm, const double* __r
   int lane = threadIdx.x & 31;
   if (i >= nb) return;
   DFlt s[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (int e = tp.ptr[i] + lane; e < tp.ptr[i + 1]; e += 32)
-    trace_entry2_df<MULTI, false>(tp, e, u, cv, s[0], s[1]);
-  for (int e = tm.ptr[i] + lane; e < tm.ptr[i + 1]; e += 32)
-    trace_entry2_df<MULTI, true>(tm, e, u, cv, s[2], s[3]);
+  for (int e = tp.ptr[i] + lane; e < tp.mid[i]; e += 32)
+    trace_entry2_df<MULTI, false, false>(tp, e, u, cv, s[0], s[1]);
+  for (int e = tp.mid[i] + lane; e < tp.ptr[i + 1]; e += 32)
+    trace_entry2_df<MULTI, false, true>(tp, e, u, cv, s[0], s[1]);
+  for (int e = tm.ptr[i] + lane; e < tm.mid[i]; e += 32)
+    trace_entry2_df<MULTI, true, false>(tm, e, u, cv, s[2], s[3]);
+  for (int e = tm.mid[i] + lane; e < tm.ptr[i + 1]; e += 32)
+    trace_entry2_df<MULTI, true, true>(tm, e, u, cv, s[2], s[3]);
   for (int q = 0; q < 4; ++q) s[q] = df_add(s[q], DFlt{0.f, 0.f});
   const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0;
   DFlt k0 = h4 ? s[2] : s[0], k1 = h4 ? s[3] : s[1];
@@ -357,23 +372,39 @@ __global__ void k_traces4_df(int nb, TraceCSR tp, TraceCSR tm, const double* __r
   if ((lane & 7) == 0 && out) out[i] = df_value(k);
 }
 
+// One side of a DOF's operator trace by LPD lanes: the plain entries (their
+// loads batched), then those with corrections.
+template <bool MULTI, bool MINUS, int LPD>
+__device__ __forceinline__ double trace_side(const TraceCSR& T, int i, int lane, const double* __restrict__ u,
+                                             const double* __restrict__ cv) {
+  const int mid = T.mid[i], end = T.ptr[i + 1];
+  double acc = 0.0;
+#pragma unroll 4
+  for (int e = T.ptr[i] + lane; e < mid; e += LPD) acc += T.w[e] * u[T.node[e]];
+  for (int e = mid + lane; e < end; e += LPD) acc += T.w[e] * trace_datum<MULTI, MINUS>(T, e, u, cv);
+  return acc;
+}
+
 // The operator's trace quantity t (average value for the Dirichlet form,
 // average normal derivative for the mu-form; weights carry the 1/2) fused with
-// the BIE combination y = alpha x + beta t.
-template <bool MULTI>
-__global__ void k_trace_op(int nb, TraceCSR tp, TraceCSR tm, const double* __restrict__ u,
-                           const double* __restrict__ cv, const double* __restrict__ x,
-                           double alpha, double beta, double* __restrict__ y) {
-  int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  int lane = threadIdx.x & 31;
-  if (i >= nb) return;
+// the BIE combination y = alpha x + beta t, LPD lanes per DOF.  With few DOFs a
+// warp each keeps the chains of gathers short; with many the FP64 pipe counts (16
+// cycles per warp instruction), and eight lanes share one reduction among four
+// DOFs: 128^3 Neumann (29,700 DOFs) 59 -> 43 us, 256^3 torus 143 -> 94.
+template <bool MULTI, int LPD>
+__global__ void __launch_bounds__(256) k_trace_op(int nb, TraceCSR tp, TraceCSR tm, const double* __restrict__ u,
+                                                  const double* __restrict__ cv, const double* __restrict__ x,
+                                                  double alpha, double beta, double* __restrict__ y) {
+  const int i = (blockIdx.x * 256 + threadIdx.x) / LPD;
+  const int lane = threadIdx.x % LPD;
   double acc = 0.0;
-  for (int e = tp.ptr[i] + lane; e < tp.ptr[i + 1]; e += 32)
-    acc += tp.w[e] * trace_datum<MULTI, false>(tp, e, u, cv);
-  for (int e = tm.ptr[i] + lane; e < tm.ptr[i + 1]; e += 32)
-    acc += tm.w[e] * trace_datum<MULTI, true>(tm, e, u, cv);
-  acc = warp_sum(acc);
-  if (lane == 0) y[i] = (x ? alpha * x[i] : 0.0) + beta * acc;
+  if (i < nb) {
+    acc = trace_side<MULTI, false, LPD>(tp, i, lane, u, cv);
+    acc += trace_side<MULTI, true, LPD>(tm, i, lane, u, cv);
+  }
+#pragma unroll
+  for (int o = LPD / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0 && i < nb) y[i] = (x ? alpha * x[i] : 0.0) + beta * acc;
 }
 
 // y -= mean(y) by one cluster of kMeanCtas CTAs: each thread a strided partial
@@ -573,14 +604,19 @@ kfbi_status launch_traces(kfbi_problem* p, const double* u, const double* cvals,
   return KFBI_OK;
 }
 
+// DOFs from which eight lanes each come near filling the GPU (152 SMs x 1024
+// threads); at 1,766 DOFs a warp each: 1024^2 solve 3403 us against 3419.
+constexpr int kManyDofs = 16384;
+
 kfbi_status launch_operator_trace(kfbi_problem* p, const double* u, const double* cvals,
                                   const double* x, double alpha_x, double beta_t, double* y) {
-  if (p->n_iface > 1)
-    KFBI_LAUNCH(p, KFBI_KC_TRACE, k_trace_op<true><<<div_up(p->nb, 8), 256, 0, p->stream>>>(
+  auto launch = [&](auto kernel, int lpd) {
+    KFBI_LAUNCH(p, KFBI_KC_TRACE, kernel<<<div_up((long long)p->nb * lpd, 256), 256, 0, p->stream>>>(
         p->nb, p->tr[0], p->tr[1], u, cvals, x, alpha_x, beta_t, y));
-  else
-    KFBI_LAUNCH(p, KFBI_KC_TRACE, k_trace_op<false><<<div_up(p->nb, 8), 256, 0, p->stream>>>(
-        p->nb, p->tr[0], p->tr[1], u, cvals, x, alpha_x, beta_t, y));
+  };
+  const bool many = p->nb >= kManyDofs;
+  if (p->n_iface > 1) many ? launch(k_trace_op<true, 8>, 8) : launch(k_trace_op<true, 32>, 32);
+  else many ? launch(k_trace_op<false, 8>, 8) : launch(k_trace_op<false, 32>, 32);
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
 }
@@ -747,19 +783,8 @@ __global__ void k_trace_op_batched(const TrDesc* __restrict__ D, const int* __re
   const int k = inst_of(start, ninst, item);
   const TrDesc& t = D[k];
   const int i = item - start[k];
-  double acc = 0.0;
-  for (int e = t.tp.ptr[i] + lane; e < t.tp.ptr[i + 1]; e += 32) {
-    double w = t.u[t.tp.node[e]];
-    const int j = t.tp.irr[e];
-    if (j >= 0) w += t.cv[j];
-    acc += t.tp.w[e] * w;
-  }
-  for (int e = t.tm.ptr[i] + lane; e < t.tm.ptr[i + 1]; e += 32) {
-    double w = t.u[t.tm.node[e]];
-    const int j = t.tm.irr[e];
-    if (j >= 0) w -= t.cv[j];
-    acc += t.tm.w[e] * w;
-  }
+  double acc = trace_side<false, false, 32>(t.tp, i, lane, t.u, t.cv);
+  acc += trace_side<false, true, 32>(t.tm, i, lane, t.u, t.cv);
   acc = warp_sum(acc);
   if (lane == 0) t.y[i] = t.alpha * t.x[i] + t.beta * acc;
 }

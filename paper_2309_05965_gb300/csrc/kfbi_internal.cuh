@@ -71,6 +71,7 @@ struct LevelSet {
 // Trace stencil CSR for one side.
 struct TraceCSR {
   int32_t* ptr = nullptr;    // N_b + 1
+  int32_t* mid = nullptr;    // N_b: entries ptr..mid take no correction, mid..next ptr do
   int32_t* node = nullptr;   // grid linear index
   // correction entry added to the node's value, -1 if none: one interface,
   // the node's entry when it lies across Gamma (+C on the '+' side, -C on the

@@ -1346,7 +1346,8 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
                              const int32_t* __restrict__ map, const int32_t* __restrict__ ptr_all,
                              const uint8_t* __restrict__ close, const uint32_t* __restrict__ need,
                              const uint32_t* __restrict__ need2, const int32_t* __restrict__ emap,
-                             int mmax, double alpha, double beta, int32_t* __restrict__ node_out,
+                             int mmax, double alpha, double beta, int32_t* __restrict__ mid_out,
+                             int32_t* __restrict__ node_out,
                              int32_t* __restrict__ irr_out, int32_t* __restrict__ irr2_out,
                              double* __restrict__ wv_out,
                              double* __restrict__ wn_out, double* __restrict__ w_out, int* flags) {
@@ -1438,8 +1439,24 @@ __global__ void k_trace_fill(Grid g, TraceParams T, DofView V, int nb,
   }
   __syncwarp();
   warp_apply_q2(A, lda, m, n, vn2, y0, y1);
-  int off = ptr_all[t];
-  for (int r = lane; r < m; r += 32) {
+  // the entries that take corrections behind the others: the trace kernels read
+  // and add corrections for those alone
+  int nreg = 0;
+  for (int r = lane; r < m; r += 32) nreg += acr[r] ? 0 : 1;
+  nreg = __reduce_add_sync(0xffffffffu, nreg);
+  const int off0 = ptr_all[t];
+  if (lane == 0) mid_out[t] = off0 + nreg - (side ? ptr_all[nb] : 0);
+  int nr = 0, na = nreg;
+  for (int r0 = 0; r0 < m; r0 += 32) {
+    const int r = r0 + lane;
+    const bool in = r < m, ac = in && acr[r] != 0;
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned br = __ballot_sync(0xffffffffu, in && !ac), ba = __ballot_sync(0xffffffffu, ac);
+    const int at = off0 + (ac ? na + __popc(ba & below) : nr + __popc(br & below));
+    nr += __popc(br);
+    na += __popc(ba);
+    if (!in) continue;
+    const int off = at - r;
     double a = y0[r] * wt[r], b = y1[r] * wt[r];
     int node = nodes[r];
     node_out[off + r] = node;
@@ -1923,7 +1940,8 @@ kfbi_status build_geometry(kfbi_problem* p) {
   int mmax = 0;
   for (int k = 0; k < 2 * nb; ++k) mmax = std::max(mmax, hcnt[k]);
   const int nnz_all = hptr[2 * nb];
-  int32_t *tnode = nullptr, *tirr = nullptr, *tirr2 = nullptr;
+  int32_t *tmid = nullptr, *tnode = nullptr, *tirr = nullptr, *tirr2 = nullptr;
+  KFBI_CUDA(p, galloc(p, &tmid, 2 * nb));
   double *twv = nullptr, *twn = nullptr, *tw = nullptr;
   KFBI_CUDA(p, galloc(p, &tnode, nnz_all));
   KFBI_CUDA(p, galloc(p, &tirr, nnz_all));
@@ -1943,7 +1961,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
     if (smem > (size_t)optin)
       return fail(p, KFBI_ERR_UNSUPPORTED, "trace stencil too large for shared memory");
     k_trace_fill<<<2 * nb, 32, smem, st>>>(g, TP, V, nb, p->inside, p->irr_flag, map, tptr, close,
-                                           need, need2, emap, mmax, alpha, beta, tnode, tirr,
+                                           need, need2, emap, mmax, alpha, beta, tmid, tnode, tirr,
                                            tirr2, twv, twn, tw, p->d_flags);
     KFBI_CUDA(p, cudaGetLastError());
   }
@@ -1958,6 +1976,7 @@ kfbi_status build_geometry(kfbi_problem* p) {
     KFBI_CUDA(p, cudaMemcpyAsync(c.ptr, sp.data(), sizeof(int32_t) * (nb + 1),
                                  cudaMemcpyHostToDevice, st));
     c.nnz = sp[nb];
+    c.mid = tmid + (size_t)s * nb;
     c.node = tnode + b0;
     c.irr = tirr + b0;
     c.irr2 = multi ? tirr2 + b0 : nullptr;
