@@ -102,14 +102,18 @@ __device__ __forceinline__ void sum_digits(const float (&f)[8], long long& T, lo
   float m = 0.f;
 #pragma unroll
   for (int d = 0; d < 8; ++d) m = fmaxf(m, fabsf(f[d]));
-  int w[8];
   if (m <= 4194304.f) {
+    // pairs in 32 bits, the offsets 0x4B400000 of both taken off together
+    constexpr unsigned off = 0x4B400000u * 257u;
+    unsigned b[8];
 #pragma unroll
-    for (int d = 0; d < 8; ++d) w[d] = __float_as_int(__fadd_rn(f[d], magic)) - 0x4B400000;
-    const int p0 = w[0] * 256 + w[1], p1 = w[2] * 256 + w[3], p2 = w[4] * 256 + w[5], p3 = w[6] * 256 + w[7];
+    for (int d = 0; d < 8; ++d) b[d] = (unsigned)__float_as_int(__fadd_rn(f[d], magic));
+    const int p0 = (int)(b[0] * 256u + b[1] - off), p1 = (int)(b[2] * 256u + b[3] - off);
+    const int p2 = (int)(b[4] * 256u + b[5] - off), p3 = (int)(b[6] * 256u + b[7] - off);
     T = add64(join64((unsigned)p0 << 16, (unsigned)(p0 >> 16)), join64((unsigned)p1, (unsigned)(p1 >> 31)));
     L = add64(join64((unsigned)p2 << 16, (unsigned)(p2 >> 16)), join64((unsigned)p3, (unsigned)(p3 >> 31)));
   } else {
+    int w[8];
 #pragma unroll
     for (int d = 0; d < 8; ++d) w[d] = __float2int_rn(f[d]);
     T = (long long)(w[0] * 256 + w[1]) * 65536 + ((long long)w[2] * 256 + w[3]);
