@@ -138,7 +138,7 @@ static bool build_loop(kfbi_batch* b) {
 // Potentials with data of every instance: per instance the correction values
 // (a, b, f~ from data[k]) and the corrected right-hand side into the
 // problem's RHS buffer, then one batched box solve into each problem's grid,
-// then its boundary layer (the outer data g_b when use_gb).
+// whose boundary layer stays zero.
 static kfbi_status batch_potentials(kfbi_batch* b, const double* const* a, const double* const* bb,
                                     const kfbi_data* data, bool use_gb) {
   kfbi_problem* p0 = b->ps[0];
@@ -149,10 +149,7 @@ static kfbi_status batch_potentials(kfbi_batch* b, const double* const* a, const
     KFBI_TRY(launch_correction_values_data(p, a ? a[k] : nullptr, bb ? bb[k] : nullptr, &dd, p->cvals));
     KFBI_TRY(launch_rhs(p, p->cvals, &dd, p->rhs));
   }
-  KFBI_TRY(batch_box_solve(p0, b->bb_data, b->zeros, b->stream));
-  for (int k = 0; k < b->n; ++k)
-    KFBI_TRY(launch_set_boundary(b->ps[k], b->ps[k]->ugrid, use_gb ? data[k].g_b : nullptr));
-  return KFBI_OK;
+  return batch_box_solve(p0, b->bb_data, b->zeros, b->stream);
 }
 
 namespace kfbi {
@@ -329,11 +326,13 @@ kfbi_status kfbi_gmres_solve_batch(kfbi_batch* b, const kfbi_data* data, const k
     KFBI_TRY(batch_potentials(b, mu ? a.data() : nullptr, nullptr, data, mu));
     for (int k = 0; k < n; ++k) {
       kfbi_problem* p = b->ps[k];
+      if (mu && data[k].g_b) KFBI_TRY(launch_set_boundary(p, p->ugrid, data[k].g_b));
       if (p->cfg.kind == KFBI_DIRICHLET_INTERIOR)
         KFBI_TRY(launch_operator_trace(p, p->ugrid, p->cvals, data[k].g1, 1.0, -1.0, p->bvec));
       else
         KFBI_TRY(launch_operator_trace(p, p->ugrid, p->cvals, data[k].g2,
                                        1.0 / (p->cfg.sigma_in + p->cfg.sigma_out), p->mu, p->bvec));
+      if (mu) KFBI_TRY(reset_boundary(p, &data[k]));
     }
   }
   // starts: y = A x0 of every instance that has one (one batched operator
@@ -439,9 +438,11 @@ kfbi_status kfbi_evaluate_batch(kfbi_batch* b, const kfbi_data* data, const doub
     if (mu) bb[k] = densities[k];
   }
   KFBI_TRY(batch_potentials(b, a.data(), mu ? bb.data() : nullptr, data, mu));
-  for (int k = 0; k < n; ++k)
+  for (int k = 0; k < n; ++k) {
     KFBI_CUDA(p0, cudaMemcpyAsync(u_grids[k], b->ps[k]->ugrid, sizeof(double) * b->ps[k]->g.nodes(),
                                   cudaMemcpyDeviceToDevice, b->stream));
+    if (mu && data[k].g_b) KFBI_TRY(launch_set_boundary(b->ps[k], u_grids[k], data[k].g_b));
+  }
   return KFBI_OK;
 }
 

@@ -23,8 +23,8 @@ kfbi_status fail(kfbi_problem* p, kfbi_status s, const std::string& msg) {
 static kfbi_status potential_traces(kfbi_problem* q, const double* a, const double* b, double* T) {
   const int nb = q->nb;
   KFBI_TRY(launch_correction_values(q, a, b, nullptr, q->cvals));
-  KFBI_TRY(launch_rhs(q, q->cvals, nullptr, q->rhs));
-  KFBI_TRY(box_solve(q, q->rhs, q->ugrid));
+  KFBI_TRY(launch_rhs_operator(q, q->cvals));
+  KFBI_TRY(box_solve_interior(q, q->rhs_op, q->ugrid));
   return launch_traces(q, q->ugrid, q->cvals, T, T + nb, T + 2 * nb, T + 3 * nb);
 }
 
@@ -52,9 +52,9 @@ kfbi_status apply_operator_impl(kfbi_problem* p, const double* x, double* y) {
   // Step 3.1 (fitted and evaluated at the irregular nodes)
   KFBI_TRY(launch_correction_values(p, dir ? x : nullptr, dir ? nullptr : x, nullptr, p->cvals));
   // Step 3.2
-  KFBI_TRY(launch_rhs(p, p->cvals, nullptr, p->rhs));
+  KFBI_TRY(launch_rhs_operator(p, p->cvals));
   // Step 3.3
-  KFBI_TRY(box_solve(p, p->rhs, p->ugrid));
+  KFBI_TRY(box_solve_interior(p, p->rhs_op, p->ugrid));
   // Step 3.4 + BIE: Dirichlet y = x/2 + avg value; mu-form y = x/2 - mu avg d_n;
   // Neumann y = x/2 + avg d_n (= x/2 - K'x), projected when kappa~ = 0
   KFBI_TRY(launch_operator_trace(p, p->ugrid, p->cvals, x, 0.5, dir || neu ? 1.0 : -p->mu, y));
@@ -111,6 +111,10 @@ static kfbi_status potential_with_data(kfbi_problem* p, const double* a, const d
   return launch_set_boundary(p, u, use_gb ? dd.g_b : nullptr);
 }
 
+kfbi_status reset_boundary(kfbi_problem* p, const kfbi_data* data) {
+  return data && data->g_b ? launch_set_boundary(p, p->ugrid, nullptr) : KFBI_OK;
+}
+
 // The data of each side of the general interface problem: f_1 (Omega_1) for
 // the kappa_1 operator; f_2 (Omega_2) and the outer values g_b for kappa_2.
 static void side_data(const kfbi_data* data, kfbi_data* d1, kfbi_data* d2) {
@@ -142,6 +146,7 @@ static kfbi_status bie_rhs_general(kfbi_problem* p, const kfbi_data* data, doubl
   KFBI_TRY(potential_with_data(q, data->g1, nullptr, &d2, true, q->ugrid));
   KFBI_TRY(launch_traces(q, q->ugrid, q->cvals, T + 4 * (size_t)nb, T + 5 * (size_t)nb, T + 6 * (size_t)nb,
                          T + 7 * (size_t)nb));
+  KFBI_TRY(reset_boundary(q, &d2));
   return launch_gen_combine(p, data->g1, 0.5, data->g2, -0.5, T, 1.0, 1.0, s1, s2, bvec);
 }
 
@@ -161,8 +166,9 @@ kfbi_status bie_rhs_impl(kfbi_problem* p, const kfbi_data* data, double* bvec) {
   }
   // b = g2/(sigma_in + sigma_out) + mu avg d_n w, w with a = g1, F = f/sigma, g_B
   KFBI_TRY(potential_with_data(p, data->g1, nullptr, data, true, p->ugrid));
-  return launch_operator_trace(p, p->ugrid, p->cvals, data->g2,
-                               1.0 / (p->cfg.sigma_in + p->cfg.sigma_out), p->mu, bvec);
+  KFBI_TRY(launch_operator_trace(p, p->ugrid, p->cvals, data->g2,
+                                 1.0 / (p->cfg.sigma_in + p->cfg.sigma_out), p->mu, bvec));
+  return reset_boundary(p, data);
 }
 
 // The boundary data each kind reads: g1 (Dirichlet), g2 (Neumann), both (interface).
@@ -327,17 +333,22 @@ static void free_geometry(kfbi_problem* p, bool keep_arena = true) {
 }
 
 // The per-DOF work vectors and the GMRES workspace of a set-up geometry (the
-// grids R and u once).
+// grids R, R of the operator and u once).
 static kfbi_status alloc_work(kfbi_problem* p) {
   p->nx = p->cfg.kind == KFBI_INTERFACE_GENERAL ? 2 * p->nb : p->nb;
   const long long nodes = p->g.nodes();
   if ((!p->rhs && dalloc(&p->rhs, nodes) != cudaSuccess) ||
+      (!p->rhs_op && dalloc(&p->rhs_op, nodes) != cudaSuccess) ||
       (!p->ugrid && dalloc(&p->ugrid, nodes) != cudaSuccess) ||
       galloc(p, &p->cvals, p->nent) != cudaSuccess || galloc(p, &p->tvals, p->nb) != cudaSuccess ||
       galloc(p, &p->bvec, p->nx) != cudaSuccess || galloc(p, &p->xbuf, p->nx) != cudaSuccess ||
       galloc(p, &p->ybuf, p->nx) != cudaSuccess ||
       (p->cfg.kind == KFBI_INTERFACE_GENERAL && galloc(p, &p->gen, 11 * (size_t)p->nb) != cudaSuccess))
     return fail(p, KFBI_ERR_CUDA, "out of device memory");
+  // what the operator expects to find: R zero off the (new) irregular nodes, u
+  // zero on the boundary layer
+  KFBI_CUDA(p, cudaMemsetAsync(p->rhs_op, 0, sizeof(double) * nodes, p->stream));
+  KFBI_TRY(launch_set_boundary(p, p->ugrid, nullptr));
   return gmres_create(p, kMaxKrylov);
 }
 
@@ -472,7 +483,7 @@ kfbi_status kfbi_destroy_problem(kfbi_problem* p) {
   box_destroy(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   if (p->ls_samples) cudaFree(p->ls_samples);
-  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->ugrid, p->ftilde, p->stencil_dev};
+  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->rhs_op, p->ugrid, p->ftilde, p->stencil_dev};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t e : p->prof.pool) cudaEventDestroy(e);
@@ -727,7 +738,8 @@ kfbi_status kfbi_evaluate(kfbi_problem* p, const kfbi_data* data, const double* 
     KFBI_TRY(launch_gen_eval_prep(p, density, density + nb, data->g1, data->g2, s, s + nb, s + 2 * (size_t)nb));
     KFBI_TRY(potential_with_data(p, density, s, &d1, false, u_grid));
     KFBI_TRY(potential_with_data(q, s + 2 * (size_t)nb, s + nb, &d2, true, q->ugrid));
-    return launch_select_side(p, u_grid, q->ugrid);
+    KFBI_TRY(launch_select_side(p, u_grid, q->ugrid));
+    return reset_boundary(q, &d2);
   }
   if (!data || !data->g1) return fail(p, KFBI_ERR_ARG, "interface evaluate needs data->g1");
   return potential_with_data(p, data->g1, density, data, true, u_grid);

@@ -1900,6 +1900,13 @@ kfbi_status box_steps_total(kfbi_problem* p, long long* out) {
   return KFBI_OK;
 }
 
+// box_solve with the boundary layer of u left as it is where the solver does not
+// write it (the FP64 transform)
+kfbi_status box_solve_interior(kfbi_problem* p, const double* rhs, double* u) {
+  if (p->mg || p->cfg.precision == KFBI_MIXED) return box_solve(p, rhs, u);
+  return dst_solve_t<double>(p, rhs, 1, u, 0, nullptr);
+}
+
 kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   if (p->mg) {
     KFBI_TRY(mg_solve(p, rhs, u));

@@ -216,15 +216,18 @@ namespace {
 // partial sums in a fixed order, runs on every SM (0.04 ms).
 constexpr int kCgsThreads = 256;
 
-// part[i nchunk + c] = V_i . V_{j+1} over chunk c, i <= j (CTAs beyond j exit)
+// part[i nchunk + c] = V_i . w over chunk c, i <= j (CTAs beyond j exit); w is
+// V_{j+1}, or the operator's output y in the first projection, which also takes
+// over the step index: jdev[3], advanced by the step before, becomes jdev[0]
 __global__ void __launch_bounds__(kCgsThreads) k_cgs_dots(const double* __restrict__ V, int nb,
-                                                          const int* __restrict__ jdev, int nchunk,
-                                                          double* __restrict__ part) {
-  const int j = jdev[0];
+                                                          int* __restrict__ jdev, int nchunk,
+                                                          const double* __restrict__ y, double* __restrict__ part) {
+  const int j = y ? jdev[3] : jdev[0];
   const int i = blockIdx.y, c = blockIdx.x;
+  if (y && i == 0 && c == 0 && threadIdx.x == 0) jdev[0] = j;
   if (i > j) return;
   const double* v = V + (size_t)i * nb;
-  const double* w = V + (size_t)(j + 1) * nb;
+  const double* w = y ? y : V + (size_t)(j + 1) * nb;
   const int per = (nb + nchunk - 1) / nchunk;
   const int b = c * per, e = min(nb, b + per);
   double s = 0.0;
@@ -240,12 +243,13 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_dots(const double* __restri
   }
 }
 
-// h[i] = sum_c part[i nchunk + c]; V_{j+1} -= sum_{i <= j} h[i] V_i; with npart:
-// the CTA's sum of squares of the result
+// h[i] = sum_c part[i nchunk + c]; V_{j+1} = w - sum_{i <= j} h[i] V_i, w = y or
+// V_{j+1}; with npart: the CTA's sum of squares of the result
 __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__ V, int nb,
                                                             const int* __restrict__ jdev,
                                                             const double* __restrict__ part, int nchunk,
-                                                            double* __restrict__ h, double* __restrict__ npart) {
+                                                            const double* __restrict__ y, double* __restrict__ h,
+                                                            double* __restrict__ npart) {
   const int j = jdev[0];
   __shared__ double hs[kMaxKrylov + 1];
   if (nchunk == 1) {
@@ -264,7 +268,7 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__
   double* w = V + (size_t)(j + 1) * nb;
   double acc = 0.0;
   for (int k = blockIdx.x * kCgsThreads + threadIdx.x; k < nb; k += gridDim.x * kCgsThreads) {
-    double s = w[k];
+    double s = y ? y[k] : w[k];
     for (int i = 0; i <= j; ++i) s -= hs[i] * V[(size_t)i * nb + k];
     w[k] = s;
     acc += s * s;
@@ -281,45 +285,55 @@ __global__ void __launch_bounds__(kCgsThreads) k_cgs_update(double* __restrict__
   }
 }
 
-// Hessenberg column j = h1 + h2, h_{j+1,j} = |V_{j+1}| (from the partials, in a
-// fixed order), Givens update, res = |g_{j+1}|, scal = 1/h_{j+1,j}, j <- j + 1
-// With use_cond (the body of the device-driven loop): the loop continues while
-// res > thr and j + 1 < jdev[2], so it ends after at most jdev[2] iterations
-// whatever the residual (NaN included).
-__global__ void k_cgs_finish(double* __restrict__ H, int ld, double* __restrict__ cs, double* __restrict__ sn,
-                             double* __restrict__ g, double* __restrict__ res, const double* __restrict__ h1,
-                             const double* __restrict__ h2, const double* __restrict__ part, int npart,
-                             int* __restrict__ jdev, double* __restrict__ scal, cudaGraphConditionalHandle cond,
-                             int use_cond, const double* __restrict__ thr) {
-  __shared__ double ws[32];
+// h_{j+1,j} = |V_{j+1}| (from the partials, in a fixed order, by every CTA);
+// V_{j+1} /= h_{j+1,j}, also into x, the operator's input.  CTA 0 then adds the
+// Hessenberg column h1 + h2, its Givens update, res = |g_{j+1}|, and advances the
+// step index (jdev[3], which no CTA of this kernel reads).  With use_cond (the
+// body of the device-driven loop): the loop continues while res > thr and j + 1
+// < jdev[2], so it ends after at most jdev[2] iterations whatever the residual
+// (NaN included).
+__global__ void __launch_bounds__(kCgsThreads) k_cgs_finish(double* __restrict__ V, int nb, double* __restrict__ x,
+                                                            double* __restrict__ H, int ld, double* __restrict__ cs,
+                                                            double* __restrict__ sn, double* __restrict__ g,
+                                                            double* __restrict__ res, const double* __restrict__ h1,
+                                                            const double* __restrict__ h2,
+                                                            const double* __restrict__ part, int npart,
+                                                            int* __restrict__ jdev, cudaGraphConditionalHandle cond,
+                                                            int use_cond, const double* __restrict__ thr) {
+  __shared__ double ws[kCgsThreads / 32];
+  const int j = jdev[0];
   double s = 0.0;
-  for (int c = threadIdx.x; c < npart; c += blockDim.x) s += part[c];
+  for (int c = threadIdx.x; c < npart; c += kCgsThreads) s += part[c];
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x != 0) return;
   double nn = 0.0;
-  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) nn += ws[q];
-  const int j = jdev[0];
-  double* col = H + (size_t)j * ld;
-  for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
+  for (int q = 0; q < kCgsThreads / 32; ++q) nn += ws[q];
   const double hn = sqrt(nn);
-  col[j + 1] = hn;
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
+  const double f = 1.0 / hn;
+  double* w = V + (size_t)(j + 1) * nb;
+  for (int k = blockIdx.x * kCgsThreads + threadIdx.x; k < nb; k += gridDim.x * kCgsThreads) {
+    const double v = w[k] * f;
+    w[k] = v;
+    x[k] = v;
   }
-  const double rr = hypot(col[j], col[j + 1]);
-  cs[j] = col[j] / rr;
-  sn[j] = col[j + 1] / rr;
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  double* col = H + (size_t)j * ld;
+  double below = h1[0] + h2[0];        // the entry the next rotation turns
+  for (int i = 0; i < j; ++i) {
+    const double next = h1[i + 1] + h2[i + 1];
+    col[i] = cs[i] * below + sn[i] * next;
+    below = -sn[i] * below + cs[i] * next;
+  }
+  const double rr = hypot(below, hn);
+  cs[j] = below / rr;
+  sn[j] = hn / rr;
   col[j] = rr;
   col[j + 1] = 0.0;
   g[j + 1] = -sn[j] * g[j];
   g[j] = cs[j] * g[j];
   res[0] = fabs(g[j + 1]);
-  scal[0] = 1.0 / hn;
-  jdev[0] = j + 1;
+  jdev[3] = j + 1;
   if (use_cond) cudaGraphSetConditional(cond, (res[0] > thr[0] && j + 1 < jdev[2]) ? 1u : 0u);
 }
 
@@ -335,15 +349,6 @@ __global__ void k_relax_tol(const double* __restrict__ thr, const double* __rest
   if (!(t > base)) t = base;
   if (t1) *t1 = t;
   if (t2) *t2 = t;
-}
-
-// V_j *= scal (j already advanced)
-__global__ void k_cgs_normalize(double* __restrict__ V, int nb, const int* __restrict__ jdev,
-                                const double* __restrict__ scal) {
-  const int j = jdev[0];
-  const double f = scal[0];
-  double* w = V + (size_t)j * nb;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += gridDim.x * blockDim.x) w[k] *= f;
 }
 
 }  // namespace
@@ -620,7 +625,6 @@ void gmres_destroy(kfbi_problem* p) {
   cudaFree(G.h1);
   cudaFree(G.h2);
   cudaFree(G.npart);
-  cudaFree(G.desc);
   G = Gmres();
 }
 
@@ -641,45 +645,31 @@ static kfbi_status read_scalar(kfbi_problem* p, const double* dev, double* host)
   return KFBI_OK;
 }
 
-// The kernels of one GMRES iteration of problem p on its stream: x = V_j;
-// y = A x (the operator's kernels); V_{j+1} = y; CGS2 over all SMs; Givens;
-// normalise; j <- j + 1.  With use_cond the finish kernel also sets the
-// condition of the enclosing device-driven loop.
+// The kernels of one GMRES iteration of problem p on its stream, V_j in the
+// operator's input buffer: y = A x (the operator's kernels); CGS2 over all SMs,
+// starting from y; norm, normalisation (V_{j+1} also into x) and Givens update;
+// j <- j + 1.  With use_cond the finish kernel also sets the condition of the
+// enclosing device-driven loop.  (Copies of V_j and y, the clearing of the
+// right-hand side and of the boundary layer and a norm kernel of its own were
+// five launches more: 64^2 Dirichlet solve 706 -> 677 us, 1024^2 mixed 3515 -> 3462.)
 static kfbi_status iteration_body(kfbi_problem* p, cudaGraphConditionalHandle cond, int use_cond) {
   Gmres& G = p->gm;
   const int nb = G.nb;
   const int eb = std::min(div_up(nb, kCgsThreads), 152 * 4);
-  const ArnDesc* d = static_cast<const ArnDesc*>(G.desc);
-  const int* done = G.jdev + 1;
-  KFBI_TRY(batch_arnoldi_copy_in(p, d, G.jdev, done, 1, nb, p->stream));
   KFBI_TRY(relax_box_tol(p));
   KFBI_TRY(apply_operator_impl(p, p->xbuf, p->ybuf));
   cudaStream_t cs = p->stream;
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_copy_out_batched<<<dim3(div_up(nb, 256), 1), 256, 0, cs>>>(d, G.jdev, done));
   const dim3 dg(G.nchunk, G.m + 1);
   for (int pass = 0; pass < 2; ++pass) {
-    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_dots<<<dg, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.nchunk, G.part));
+    const double* y = pass ? nullptr : p->ybuf;
+    KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_dots<<<dg, kCgsThreads, 0, cs>>>(G.V, nb, G.jdev, G.nchunk, y, G.part));
     KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_update<<<eb, kCgsThreads, 0, cs>>>(
-        G.V, nb, G.jdev, G.part, G.nchunk, pass ? G.h2 : G.h1, pass ? G.npart : nullptr));
+        G.V, nb, G.jdev, G.part, G.nchunk, y, pass ? G.h2 : G.h1, pass ? G.npart : nullptr));
   }
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_finish<<<1, 256, 0, cs>>>(G.H, G.m + 1, G.cs, G.sn, G.g, G.scal + 2, G.h1,
-                                                                 G.h2, G.npart, eb, G.jdev, G.scal + 3, cond,
-                                                                 use_cond, G.scal + 5));
-  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_normalize<<<eb, 256, 0, cs>>>(G.V, nb, G.jdev, G.scal + 3));
+  KFBI_LAUNCH(p, KFBI_KC_GMRES, k_cgs_finish<<<eb, kCgsThreads, 0, cs>>>(
+      G.V, nb, p->xbuf, G.H, G.m + 1, G.cs, G.sn, G.g, G.scal + 2, G.h1, G.h2, G.npart, eb, G.jdev, cond, use_cond,
+      G.scal + 5));
   KFBI_CUDA(p, cudaGetLastError());
-  return KFBI_OK;
-}
-
-static kfbi_status ensure_desc(kfbi_problem* p) {
-  Gmres& G = p->gm;
-  if (!p->cap_stream) KFBI_CUDA(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-  if (!G.desc) {
-    ArnDesc d{G.V, G.nb, G.m, G.H, G.m + 1, G.cs, G.sn, G.g, G.scal + 2, p->xbuf, p->ybuf};
-    ArnDesc* dd = nullptr;
-    KFBI_CUDA(p, dalloc(&dd, 1));
-    KFBI_CUDA(p, cudaMemcpy(dd, &d, sizeof(d), cudaMemcpyHostToDevice));
-    G.desc = dd;
-  }
   return KFBI_OK;
 }
 
@@ -689,6 +679,7 @@ static kfbi_status capture_body(kfbi_problem* p, cudaGraph_t into, cudaGraph_t* 
                                 cudaGraphConditionalHandle cond, int use_cond) {
   Gmres& G = p->gm;
   cudaStream_t st = p->stream;
+  if (!p->cap_stream) KFBI_CUDA(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
   KFBI_CUDA(p, cudaStreamSynchronize(st));
   long long before[KFBI_KC_COUNT];
   for (int k = 0; k < KFBI_KC_COUNT; ++k) before[k] = p->prof.launches[k];
@@ -728,7 +719,6 @@ static bool loop_graph(kfbi_problem* p) {
   if (G.loop_exec) return true;
   if (G.loop_failed) return false;
   G.loop_failed = true;
-  if (ensure_desc(p) != KFBI_OK) return false;
   cudaGraph_t g = nullptr;
   if (cudaGraphCreate(&g, 0) != cudaSuccess) return false;
   cudaGraphConditionalHandle h;
@@ -816,6 +806,7 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
     }
     KFBI_LAUNCH(p, KFBI_KC_GMRES, k_scale<<<eb, 256, 0, st>>>(V0, nb, beta, 1));
     KFBI_LAUNCH(p, KFBI_KC_GMRES, k_init_g<<<1, 128, 0, st>>>(G.g, G.m, beta));
+    KFBI_CUDA(p, cudaMemcpyAsync(p->xbuf, V0, sizeof(double) * nb, cudaMemcpyDeviceToDevice, st));
     // the residual estimate starts at beta and the threshold is rtol ||b||
     // (both read on the device by the loop and by the relaxation)
     {
@@ -829,14 +820,14 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
     if (graph_it && loop_graph(p)) {
       // one launch runs the cycle: at most min(m, max_iter - total) iterations
       const int jmax = std::min(m, max_iter - total);
-      const int head[3] = {0, 0, jmax};
+      const int head[4] = {0, 0, jmax, 0};
       const double thr = rtol * bnorm;
       KFBI_CUDA(p, cudaMemcpyAsync(G.jdev, head, sizeof(head), cudaMemcpyHostToDevice, st));
       KFBI_CUDA(p, cudaMemcpyAsync(G.scal + 5, &thr, sizeof(double), cudaMemcpyHostToDevice, st));
       KFBI_CUDA(p, cudaGraphLaunch(G.loop_exec, st));
       int jdone = 0;
       KFBI_CUDA(p, cudaMemcpyAsync(G.host_res, res, sizeof(double), cudaMemcpyDeviceToHost, st));
-      KFBI_CUDA(p, cudaMemcpyAsync(&jdone, G.jdev, sizeof(int), cudaMemcpyDeviceToHost, st));
+      KFBI_CUDA(p, cudaMemcpyAsync(&jdone, G.jdev + 3, sizeof(int), cudaMemcpyDeviceToHost, st));
       KFBI_CUDA(p, cudaStreamSynchronize(st));
       hres = G.host_res[0];
       if (jdone < 1 || jdone > jmax) return fail(p, KFBI_ERR_CUDA, "device-driven GMRES loop lost its step count");
@@ -845,8 +836,7 @@ kfbi_status gmres_run(kfbi_problem* p, const double* b, const double* x0, double
       jend = jdone;
       if (!std::isfinite(hres)) return fail(p, KFBI_ERR_NONFINITE, "non-finite GMRES residual");
     } else {
-      KFBI_TRY(ensure_desc(p));
-      KFBI_CUDA(p, cudaMemsetAsync(G.jdev, 0, 3 * sizeof(int), st));
+      KFBI_CUDA(p, cudaMemsetAsync(G.jdev, 0, 4 * sizeof(int), st));
       for (int j = 0; j < m; ++j) {
         KFBI_TRY(iteration_body(p, 0, 0));
         ++total;

@@ -174,7 +174,7 @@ __global__ void k_rhs_correct_multi(int nirr, int nnb, const int32_t* __restrict
                                     const int32_t* __restrict__ corr_a,
                                     const int32_t* __restrict__ corr_b,
                                     const double* __restrict__ nbc, const double* __restrict__ cv,
-                                    double* __restrict__ R) {
+                                    double* __restrict__ R, int add) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= nirr) return;
   double acc = 0.0;
@@ -183,7 +183,8 @@ __global__ void k_rhs_correct_multi(int nirr, int nnb, const int32_t* __restrict
     const int jb = corr_b[(size_t)s * nirr + q];
     if (ja >= 0 || jb >= 0) acc += nbc[s] * ((ja >= 0 ? cv[ja] : 0.0) - (jb >= 0 ? cv[jb] : 0.0));
   }
-  R[lin[q]] += acc;
+  const long long t = lin[q];
+  R[t] = add ? R[t] + acc : acc;
 }
 
 // The corrected datum of trace stencil entry e: one interface, u + C across
@@ -574,13 +575,26 @@ kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* da
   }
   if (cvals && p->n_iface > 1) {
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct_multi<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
-        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, d_nbc, cvals, rhs));
+        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, d_nbc, cvals, rhs, 1));
     KFBI_CUDA(p, cudaGetLastError());
   } else if (cvals) {
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
         p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, d_nbc, cvals, rhs, 1));
     KFBI_CUDA(p, cudaGetLastError());
   }
+  return KFBI_OK;
+}
+
+// The operator's right-hand side: the corrections alone, assigned at the
+// irregular nodes of p->rhs_op, which is zero elsewhere.
+kfbi_status launch_rhs_operator(kfbi_problem* p, const double* cvals) {
+  if (p->n_iface > 1)
+    KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct_multi<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
+        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, p->nb_coef, cvals, p->rhs_op, 0));
+  else
+    KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
+        p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, p->nb_coef, cvals, p->rhs_op, 0));
+  KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
 }
 

@@ -116,11 +116,10 @@ struct Gmres {
   int nchunk = 0;
   // one GMRES iteration (operator + Arnoldi step) with the step index on the
   // device
-  int* jdev = nullptr;          // [0] j, [1] done flag (always 0 here), [2] iteration limit
+  int* jdev = nullptr;          // [0] j of the running step, [2] iteration limit, [3] steps done
   double* h1 = nullptr;         // (m+1)
   double* h2 = nullptr;         // (m+1)
   double* npart = nullptr;      // partial norms (one per CTA of the update)
-  void* desc = nullptr;         // ArnDesc of this problem (device)
   // the whole Arnoldi cycle as a conditional WHILE node around that iteration
   cudaGraphExec_t loop_exec = nullptr;
   cudaGraph_t loop_graph = nullptr;
@@ -224,6 +223,10 @@ struct kfbi_problem {
   long long op_counts[KFBI_KC_COUNT] = {};
   double* xbuf = nullptr;
   double* ybuf = nullptr;
+  // the operator's right-hand side: only its entries at the irregular nodes are
+  // ever written, the rest stays zero (one grid of memory in place of a clearing
+  // pass per application)
+  double* rhs_op = nullptr;
   bool use_graphs = true;
   int nx = 0;                    // unknowns of the BIE: N_b, or 2 N_b for the general interface kind
   kfbi_problem* twin = nullptr;  // general interface kind: the kappa_2/sigma_2 operator (owned)
@@ -335,6 +338,7 @@ kfbi_status launch_collocation_fit(kfbi_problem* p, const double* a, const doubl
                                    const double* ftilde, double* coef);
 kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* data,
                        double* rhs);
+kfbi_status launch_rhs_operator(kfbi_problem* p, const double* cvals);
 kfbi_status launch_correction_values_data(kfbi_problem* p, const double* a, const double* b,
                                           const kfbi_data* data, double* cvals);
 kfbi_status upload_neighbour_tables(kfbi_problem* p);
@@ -344,6 +348,9 @@ kfbi_status launch_operator_trace(kfbi_problem* p, const double* u, const double
                                   const double* x, double alpha_x, double beta_t,
                                   double* y);
 kfbi_status launch_set_boundary(kfbi_problem* p, double* u, const double* g_b);
+// p->ugrid's boundary layer back to the zeros that the operator expects, after
+// a potential with data->g_b was read from it
+kfbi_status reset_boundary(kfbi_problem* p, const kfbi_data* data);
 // Neumann BVP with kappa~ = 0 (Sec. 7.2.1): y -= mean(y) over the N_b DOFs;
 // a no-op for every other problem.
 kfbi_status launch_mean_project(kfbi_problem* p, double* y);
@@ -364,6 +371,7 @@ kfbi_status launch_select_side(kfbi_problem* p, double* u, const double* u2);
 kfbi_status box_create(kfbi_problem* p);
 void box_destroy(kfbi_problem* p);
 kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u);
+kfbi_status box_solve_interior(kfbi_problem* p, const double* rhs, double* u);
 kfbi_status box_last_residual(kfbi_problem* p, double* rel, int* converged);
 kfbi_status box_steps(kfbi_problem* p, int* steps, int* cycles);
 double* box_tol_dev(kfbi_problem* p);
