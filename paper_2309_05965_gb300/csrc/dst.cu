@@ -710,7 +710,10 @@ struct Reg {
   static constexpr int T = G >= 16 ? 9 * G / 16 : 9;   // FFT threads per pair: 16 points (G < 16: a sequence)
   // one pair per CTA (2D): as many threads as the stores need
   static constexpr int THREADS = P == 1 && G >= 32 ? G : (P * T + 31) / 32 * 32;
-  static constexpr int MINB = THREADS >= 128 && THREADS <= 160 ? 4 : 1;
+  // CTAs per SM by the register cap: latency-bound passes, 256^3 box solve 1635 ->
+  // 1592 us with five CTAs of 128..160 threads instead of four, 2048^2 469 -> 464
+  // with three of 256 instead of two
+  static constexpr int MINB = THREADS >= 128 && THREADS <= 160 ? 5 : THREADS == 256 ? 3 : 1;
   static constexpr int GP = (G + G / 16) | 1;          // odd pitches: no bank conflicts across q or pairs
   static constexpr int PP = 9 * GP;
   static constexpr size_t SMEM = sizeof(Cx<float>) * (size_t)P * PP;
@@ -1518,9 +1521,8 @@ void launch_pass32(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cud
 }
 
 // The FP64 pass on the tensor cores (dst_mma.cuh), N = 64..1024; below and
-// above (2D 2048: the dense products would cost 1.2 ms a solve, the FFT 1.9 ms,
-// but its lines do not fit beside their digits) the FFT kernel stays.
-// Measured, FFT -> products, FP64 box solve: 256^3 6709 -> 2127 us, 128^3 845 ->
+// above (2D 2048, whose lines do not fit beside their digits) the FFT kernel stays.
+// Measured, FFT -> products, FP64 box solve: 256^3 6709 -> 2116 us, 128^3 845 ->
 // 234, 64^3 124 -> 50, 1024^2 414 -> 412, 512^2 116 -> 85, 256^2 52 -> 35, 64^2
 // 33 -> 27; relative error against a quad-precision solve 4e-16..9e-16 -> 1e-16..3e-16.
 template <int LOGN, int W>
@@ -1547,7 +1549,7 @@ void launch_pass_mma(kfbi_problem* p, const PassArgs& A, int na, cudaStream_t st
   int split = 1;
   while (2 * split * ctas <= 152 && (n >> 4) / (2 * split) >= 4) split *= 2;
   // many line groups: four CTAs of four warps per SM overlap their phases
-  // (256^3: 2127 us; two of eight 2190)
+  // (256^3: 2116 us; five of them 2283, two of eight warps with 16 lines 2317)
   const bool many = ctas >= 4 * 152;
   switch (n) {
     case 64: launch_mma<6, 4>(p, A, na, split, st); break;
