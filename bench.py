@@ -1003,7 +1003,7 @@ def _inside(G, kfbi):
 # one ncu capture of the current kernels (profiles/k_dst32_k_res_fix2_flower1024.md;
 # cold cache: ncu flushes L2 before each replay, in the timed loop the grids
 # stay in L2); None once the kernels change
-NCU_DST_BYTES_PER_LAUNCH_1024 = (4.279e6 + 4.285e6 + 12.667e6) / 3
+NCU_DST_BYTES_PER_LAUNCH_1024 = (4.247e6 + 4.245e6 + 12.635e6) / 3
 
 
 def roofline(args, G, prof, prec, box_steps=None):
