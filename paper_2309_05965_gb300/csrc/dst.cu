@@ -1115,7 +1115,8 @@ __device__ __forceinline__ void fix_scale_store(const FixScale& s, double kc, do
 // (u0 is 0 on the boundary layer).  Every CTA derives the scale itself (a few
 // integer operations on the exponent; no launch of its own), the first writes
 // it for the later kernels.  A CTA takes kFixRows rows of 128 columns, all
-// their loads in flight together.
+// their loads in flight together.  The items lie on gridDim.x: in 3D the row
+// groups, up to 1025^2 / 8 = 131,329, are too many for gridDim.y (65,535).
 constexpr int kFixRows = 8;
 __global__ void __launch_bounds__(128) k_fix0(Grid g, int rows, const float* __restrict__ u0,
                                               const double* __restrict__ R,
@@ -1124,8 +1125,9 @@ __global__ void __launch_bounds__(128) k_fix0(Grid g, int rows, const float* __r
                                               float* __restrict__ fixf, long long* __restrict__ ufix,
                                               long long* __restrict__ rfix, double* __restrict__ u) {
   const int n = g.n, n1 = n + 1;
-  const int j = blockIdx.x * 128 + threadIdx.x;
-  const int r0 = blockIdx.y * kFixRows;
+  const int ncb = (n1 + 127) / 128;
+  const int j = (int)(blockIdx.x % ncb) * 128 + threadIdx.x;
+  const int r0 = (int)(blockIdx.x / ncb) * kFixRows;
   const bool in_j = j >= 1 && j < n;
   float uv[kFixRows];
   double rv[kFixRows];
@@ -1136,7 +1138,7 @@ __global__ void __launch_bounds__(128) k_fix0(Grid g, int rows, const float* __r
     rv[k] = ok && in_j ? R[(r0 + k) * n1 + j] : 0.0;
   }
   const FixScale s = fix_scale_of(umax[0], multh2, inv_multh2);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) fix_scale_store(s, kc, fixd, fixf);
+  if (blockIdx.x == 0 && threadIdx.x == 0) fix_scale_store(s, kc, fixd, fixf);
   if (j > n) return;
 #pragma unroll
   for (int k = 0; k < kFixRows; ++k) {
@@ -1156,7 +1158,7 @@ void launch_fix0(kfbi_problem* p, const Grid& g, const float* u0, const double* 
                  double multh2, double kc, double* fixd, float* fixf, long long* ufix, long long* rfix, double* u,
                  cudaStream_t st) {
   const int rows = (int)(g.nodes() / (g.n + 1));
-  const dim3 grid((unsigned)div_up(g.n + 1, 128), (unsigned)div_up(rows, kFixRows));
+  const int grid = div_up(g.n + 1, 128) * div_up(rows, kFixRows);
   KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_fix0<<<grid, 128, 0, st>>>(g, rows, u0, R, umax, multh2, 1.0 / multh2, kc,
                                                                 fixd, fixf, ufix, rfix, u));
 }
