@@ -1027,6 +1027,7 @@ struct StepCheck {
   int* conv;
   double margin;
   int step;        // the step to check
+  bool last;       // a step follows that is the last: its pass writes u at the interior nodes only
 };
 
 // whether the refinement is over at this check (or was before)
@@ -1112,7 +1113,7 @@ __device__ __forceinline__ void fix_scale_store(const FixScale& s, double kc, do
 
 // The fixed-point scale from max|u0|, u_fix = round(u0 2^F / (mult h^2)),
 // R_fix = round(R 2^F); with u, also the FP64 solution of the fixed-point u_fix
-// (u0 is 0 on the boundary layer).  Every CTA derives the scale itself (a few
+// and its zero boundary layer.  Every CTA derives the scale itself (a few
 // integer operations on the exponent; no launch of its own), the first writes
 // it for the later kernels.  A CTA takes kFixRows rows of 128 columns, all
 // their loads in flight together.  The items lie on gridDim.x: in 3D the row
@@ -1149,7 +1150,7 @@ __global__ void __launch_bounds__(128) k_fix0(Grid g, int rows, const float* __r
     const int t = r * n1 + j;
     const long long uf = f2ll((uv[k] * s.f[0]) * s.f[1]);
     ufix[t] = uf;
-    if (u) u[t] = ll2d(uf) * s.isc;
+    if (u) u[t] = interior ? ll2d(uf) * s.isc : 0.0;
     rfix[t] = interior ? d2ll_pow2(rv[k], s.F) : 0ll;
   }
 }
@@ -1263,8 +1264,10 @@ __device__ __forceinline__ long long kappa_int(const KappaFix& f, long long m) {
 // window of centre values and horizontal pair sums (three int64 loads per
 // node instead of nine; integer sums are exact, so the grouping of the
 // stencil sums does not change the result).  Grid: x over the columns 0..N, y over
-// row chunks of 0..N; with uout and the convergence flag set, it writes the
-// FP64 solution at every node instead.
+// row chunks of 0..N.  When the refinement is over it writes the FP64 solution
+// instead, at every node (0 on the boundary layer, whatever the scale: 0 times the
+// NaN scale of non-finite data would not be); before the last step, whose pass
+// writes the interior nodes, the boundary layer.
 constexpr int kResRows = 4;
 __global__ void k_res_fix2(Grid g, FixStencil W, const long long* __restrict__ R, const long long* __restrict__ u,
                            const double* __restrict__ fixd, const float* __restrict__ fixf,
@@ -1275,9 +1278,13 @@ __global__ void k_res_fix2(Grid g, FixStencil W, const long long* __restrict__ R
   const int i0 = blockIdx.y * kResRows, i1 = min(n1, i0 + kResRows);
   if (chk.nrm ? step_stop(chk, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) : (skip && *skip)) {
     if (uout)
-      for (int i = i0; i < i1; ++i) uout[i * n1 + j] = ll2d(u[i * n1 + j]) * fixd[1];
+      for (int i = i0; i < i1; ++i)
+        uout[i * n1 + j] = j > 0 && j < n && i > 0 && i < n ? ll2d(u[i * n1 + j]) * fixd[1] : 0.0;
     return;
   }
+  if (chk.last)
+    for (int i = i0; i < i1; ++i)
+      if (j == 0 || j == n || i == 0 || i == n) uout[i * n1 + j] = 0.0;
   if (j < 1 || j >= n) return;   // boundary columns of r are never read
   const int a = max(i0, 1), b = min(i1, n);
   if (a >= b) return;
@@ -1313,8 +1320,7 @@ __global__ void k_res_fix2(Grid g, FixStencil W, const long long* __restrict__ R
 // sums are e = S1 + C(z-1) + C(z+1), k2 = S2 + S1(z-1) + S1(z+1),
 // k3 = S2(z-1) + S2(z+1).  The next slice of u and R is loaded before the
 // current one is computed.  Integer sums are exact, so the grouping does not
-// change the result (checked bit for bit against the one-node 27-point form).  The grid covers every node 0..N per axis: interior nodes get
-// the residual; with uout and the convergence flag set, every node gets u.
+// change the result (checked bit for bit against the one-node 27-point form).  The grid covers every node 0..N per axis; u as in k_res_fix2.
 constexpr int kR3 = 2, kR3X = 32, kR3Y = 4, kR3Threads = kR3X * kR3Y;
 __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W, const long long* __restrict__ R,
                                                             const long long* __restrict__ u,
@@ -1328,6 +1334,7 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
   if (x > n || yb > n) return;
   const int z0 = blockIdx.z * kz, z1 = min(n1, z0 + kz);
   const bool keeper = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0;
+  auto layer = [&](int y, int z) { return x == 0 || x == n || y == 0 || y == n || z == 0 || z == n; };
   if (chk.nrm ? step_stop(chk, keeper) : (skip && *skip)) {
     if (uout) {
       const double isc = fixd[1];
@@ -1336,11 +1343,16 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
         for (int r = 0; r < kR3; ++r)
           if (yb + r <= n) {
             const int t = z * plane + (yb + r) * n1 + x;
-            uout[t] = ll2d(u[t]) * isc;
+            uout[t] = layer(yb + r, z) ? 0.0 : ll2d(u[t]) * isc;
           }
     }
     return;
   }
+  if (chk.last)
+    for (int z = z0; z < z1; ++z)
+#pragma unroll
+      for (int r = 0; r < kR3; ++r)
+        if (yb + r <= n && layer(yb + r, z)) uout[z * plane + (yb + r) * n1 + x] = 0.0;
   if (x < 1 || x >= n) return;   // boundary nodes of r are never read
   const int za = max(z0, 1), zb = min(z1, n);
   if (za >= zb) return;
@@ -1422,7 +1434,7 @@ __global__ void __launch_bounds__(kR3Threads, 5) k_res_fix3(Grid g, FixStencil W
 // launch of the fixed-point residual for the grid's dimension
 void launch_res_fix(kfbi_problem* p, const Grid& g, const FixStencil& W, const long long* R, const long long* u,
                     const double* fixd, const float* fixf, float* r32, const int* skip, double* uout,
-                    cudaStream_t st, const StepCheck& chk = StepCheck{nullptr, nullptr, nullptr, 0.0, 0}) {
+                    cudaStream_t st, const StepCheck& chk = StepCheck{nullptr, nullptr, nullptr, 0.0, 0, false}) {
   if (g.d == 2) {
     const dim3 grid((unsigned)div_up(g.n + 1, 128), (unsigned)div_up(g.n + 1, kResRows), 1u);
     KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_res_fix2<<<grid, 128, 0, st>>>(g, W, R, u, fixd, fixf, r32, skip, uout,
@@ -1947,7 +1959,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   launch_fix0(p, g, B->work32, rhs, slot + 1, B->multh2, B->kc, B->fixd, B->fixf, B->ufix, B->rfix,
               B->refine_steps > 1 ? nullptr : u, st);
   if (B->refine_steps == 1)
-    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, 0}));
+    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, 0, false}));
   float* r32 = reinterpret_cast<float*>(B->res);
   PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, nullptr);
   {
@@ -1962,7 +1974,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   const FixStencil W{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB};
   for (int it = 1; it < B->refine_steps; ++it) {
     launch_res_fix(p, g, W, B->rfix, B->ufix, B->fixd, B->fixf, r32, B->conv, u, st,
-                   StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, it - 1});
+                   StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, it - 1, it + 1 == B->refine_steps});
     PassArgs& last = PK.args[PK.npass - 1];
     last.corr_max = slot + 2 * it;
     last.uout = it + 1 < B->refine_steps ? nullptr : u;   // the last step also writes the FP64 solution
@@ -2337,7 +2349,7 @@ __global__ void k_check_batched(const BoxDesc* __restrict__ D, int ninst, int st
 // MODE 1: exact residual -> r32 (skips converged instances), in 2D marching
 // over the rows with k_res_fix2's three-row window;
 // MODE 2: u = u_fix mult h^2 2^-F of the instances that converged before the last
-// step; of the others, whose last pass writes u at the interior nodes, the
+// step (0 on the boundary layer); of the others, whose last pass writes u at the interior nodes, the
 // boundary layer (0); nothing of those in `done`.  MODE 3: u of every instance.
 template <int MODE>
 __global__ void __launch_bounds__(128) k_rows_batched(const BoxDesc* __restrict__ D, const int* __restrict__ rstart,
@@ -2383,12 +2395,13 @@ __global__ void __launch_bounds__(128) k_rows_batched(const BoxDesc* __restrict_
       const double isc = B.fixd[1];
       const long long* __restrict__ uf = B.ufix;
       double* __restrict__ u = B.u;
+      auto interior = [&](int r) {
+        const int i1 = d2 ? r : r % n1, i0 = d2 ? 1 : r / n1;
+        return in_j && i1 >= 1 && i1 < n && i0 >= 1 && i0 < n;
+      };
       if (MODE == 2 && !conv) {
-        for (int k = 0; k < nr; ++k) {
-          const int r = r0 + k;
-          const int i1 = d2 ? r : r % n1, i0 = d2 ? 1 : r / n1;
-          if (!(in_j && i1 >= 1 && i1 < n && i0 >= 1 && i0 < n)) u[r * n1 + j] = 0.0;
-        }
+        for (int k = 0; k < nr; ++k)
+          if (!interior(r0 + k)) u[(r0 + k) * n1 + j] = 0.0;
         continue;
       }
       long long v[kFixRows];
@@ -2396,7 +2409,7 @@ __global__ void __launch_bounds__(128) k_rows_batched(const BoxDesc* __restrict_
       for (int k = 0; k < kFixRows; ++k) v[k] = k < nr ? uf[(r0 + k) * n1 + j] : 0ll;
 #pragma unroll
       for (int k = 0; k < kFixRows; ++k)
-        if (k < nr) u[(r0 + k) * n1 + j] = ll2d(v[k]) * isc;
+        if (k < nr) u[(r0 + k) * n1 + j] = interior(r0 + k) ? ll2d(v[k]) * isc : 0.0;
     } else {
       if (!in_j) continue;
       const FixStencil W = B.W;
