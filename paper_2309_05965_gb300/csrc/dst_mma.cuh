@@ -28,7 +28,7 @@ namespace {
 constexpr int kMmaMinN = 64, kMmaMaxN = 1024;   // box sizes the kernel takes
 
 // (T 2^32 + L) 2^e rounded half up to FP64, |T| < 2^46, |L| < 2^50, by
-// assembling the bits; underflow gives 0, overflow an infinity
+// assembling the bits; overflow gives an infinity
 __device__ __forceinline__ double sum_value(long long T, long long L, int e) {
   unsigned l, h0, h1, l0, l1;
   split64(L, l, l1);
@@ -48,6 +48,11 @@ __device__ __forceinline__ double sum_value(long long T, long long L, int e) {
   l1 = __funnelshift_l(w1, w2, lz);                    // bit 31 of l1 set
   l0 = __funnelshift_l(w0, w1, lz);
   int E = 1023 + (one ? 63 : 95) - lz + e;
+  if (E <= 0) {                                        // subnormal: 12 - E bits go; a carry makes 2^-1022
+    const int s = 11 - E;
+    const unsigned long long m = s > 63 ? 0ull : (unsigned long long)join64(l0, l1) >> s;
+    return __longlong_as_double((long long)(((m + 1ull) >> 1) | ((unsigned long long)sign << 32)));
+  }
   unsigned cy;
   asm("add.cc.u32 %0, %0, 1024;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, 0, 0;" : "+r"(l0), "+r"(l1), "=r"(cy));
   if (cy) {                                            // rounded up to a power of two
@@ -55,21 +60,21 @@ __device__ __forceinline__ double sum_value(long long T, long long L, int e) {
     l0 = 0u;
     E += 1;
   }
-  if (E <= 0) return 0.0;
   if (E >= 2047) return __hiloint2double((int)(sign | 0x7ff00000u), 0);
   return __hiloint2double((int)(sign | ((unsigned)E << 20) | ((l1 >> 11) & 0xfffffu)),
                           (int)__funnelshift_r(l0, l1, 11));
 }
 
-// x (of a line whose largest exponent field is e) as a 60-bit integer,
-// x 2^(1082 - e) rounded (truncation towards zero would bias the low modes)
+// x (of a line whose largest exponent field is e, at least 1) as a 60-bit integer,
+// x 2^(1082 - e) rounded (truncation towards zero would bias the low modes);
+// subnormals have the exponent of field 1 and no leading bit
 __device__ __forceinline__ long long line_int(double x, int e) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int ex = (int)((hi >> 20) & 0x7ffu);
-  const int s = e - ex;
-  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  const int s = e - max(ex, 1);
+  const unsigned mh = (hi & 0xfffffu) | (ex == 0 ? 0u : 0x100000u);
   const unsigned long long m = (unsigned long long)join64(lo << 8, __funnelshift_l(lo, mh, 8));
-  const long long v = (ex == 0 || s > 62) ? 0ll : (long long)(((m >> s) + 1ull) >> 1);
+  const long long v = s > 62 ? 0ll : (long long)(((m >> s) + 1ull) >> 1);
   return (int)hi < 0 ? -v : v;
 }
 
@@ -214,7 +219,7 @@ __device__ __forceinline__ void mma_coord(bool contig, int i, int& q, int& j) {
 }
 
 // The lines' values x (as mma_coord deals them) as 60-bit integers in raw,
-// their exponents in sexp (zero on entry), then the foldings as digit pairs.
+// their exponents in sexp (1 on entry), then the foldings as digit pairs.
 template <int LOGN, int W>
 __device__ __forceinline__ void mma_fold(double (&x)[Mma<LOGN, W>::VALS], bool contig, double* raw, uint4* pk,
                                          int* sexp) {
@@ -227,7 +232,7 @@ __device__ __forceinline__ void mma_fold(double (&x)[Mma<LOGN, W>::VALS], bool c
 #pragma unroll
       for (int i = 0; i < PER; ++i) mx = max(mx, (unsigned)__double2hiint(x[l * PER + i]) & 0x7fffffffu);
       mx = __reduce_max_sync(0xffffffffu, mx);
-      if ((threadIdx.x & 31) == 0) sexp[(threadIdx.x >> 5) + W * l] = (int)(mx >> 20);
+      if ((threadIdx.x & 31) == 0) sexp[(threadIdx.x >> 5) + W * l] = max((int)(mx >> 20), 1);
     }
     __syncwarp();                                      // a warp reads its own lines' exponents
   } else {
@@ -407,7 +412,7 @@ __global__ void __launch_bounds__(32 * W, LOGN > 9 ? 1 : W == 8 ? 2 : 4) k_dst_m
   const int a = blockIdx.y + 1, b0 = 1 + NL * blockIdx.x;
   const int sb = (int)A.sb, es = (int)A.es, off0 = a * (int)A.sa + b0 * sb;   // 32-bit: at most 1025^3 nodes
   const bool contig = es == 1;
-  if (threadIdx.x < NL) sexp[threadIdx.x] = 0;
+  if (threadIdx.x < NL) sexp[threadIdx.x] = 1;
   double x[VALS];
   {
     const double* src = static_cast<const double*>(A.src) + off0;
