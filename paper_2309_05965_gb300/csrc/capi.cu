@@ -24,7 +24,7 @@ static kfbi_status potential_traces(kfbi_problem* q, const double* a, const doub
   const int nb = q->nb;
   KFBI_TRY(launch_correction_values(q, a, b, nullptr, q->cvals));
   KFBI_TRY(launch_rhs_operator(q, q->cvals));
-  KFBI_TRY(box_solve_interior(q, q->rhs_op, q->ugrid));
+  KFBI_TRY(box_solve_interior(q, q->rhs, q->ugrid));
   return launch_traces(q, q->ugrid, q->cvals, T, T + nb, T + 2 * nb, T + 3 * nb);
 }
 
@@ -54,7 +54,7 @@ kfbi_status apply_operator_impl(kfbi_problem* p, const double* x, double* y) {
   // Step 3.2
   KFBI_TRY(launch_rhs_operator(p, p->cvals));
   // Step 3.3
-  KFBI_TRY(box_solve_interior(p, p->rhs_op, p->ugrid));
+  KFBI_TRY(box_solve_interior(p, p->rhs, p->ugrid));
   // Step 3.4 + BIE: Dirichlet y = x/2 + avg value; mu-form y = x/2 - mu avg d_n;
   // Neumann y = x/2 + avg d_n (= x/2 - K'x), projected when kappa~ = 0
   KFBI_TRY(launch_operator_trace(p, p->ugrid, p->cvals, x, 0.5, dir || neu ? 1.0 : -p->mu, y));
@@ -106,8 +106,11 @@ static kfbi_status potential_with_data(kfbi_problem* p, const double* a, const d
   if (data) dd = *data;
   if (!use_gb) dd.g_b = nullptr;
   KFBI_TRY(launch_correction_values_data(p, a, b, &dd, p->cvals));
-  KFBI_TRY(launch_rhs(p, p->cvals, &dd, p->rhs));
-  KFBI_TRY(box_solve(p, p->rhs, u));
+  kfbi_status s = launch_rhs(p, p->cvals, &dd, p->rhs);
+  if (s == KFBI_OK) s = box_solve(p, p->rhs, u);
+  const kfbi_status r = reset_rhs(p, &dd);
+  if (s != KFBI_OK) return s;
+  KFBI_TRY(r);
   return launch_set_boundary(p, u, use_gb ? dd.g_b : nullptr);
 }
 
@@ -333,12 +336,11 @@ static void free_geometry(kfbi_problem* p, bool keep_arena = true) {
 }
 
 // The per-DOF work vectors and the GMRES workspace of a set-up geometry (the
-// grids R, R of the operator and u once).
+// grids R and u once).
 static kfbi_status alloc_work(kfbi_problem* p) {
   p->nx = p->cfg.kind == KFBI_INTERFACE_GENERAL ? 2 * p->nb : p->nb;
   const long long nodes = p->g.nodes();
   if ((!p->rhs && dalloc(&p->rhs, nodes) != cudaSuccess) ||
-      (!p->rhs_op && dalloc(&p->rhs_op, nodes) != cudaSuccess) ||
       (!p->ugrid && dalloc(&p->ugrid, nodes) != cudaSuccess) ||
       galloc(p, &p->cvals, p->nent) != cudaSuccess || galloc(p, &p->tvals, p->nb) != cudaSuccess ||
       galloc(p, &p->bvec, p->nx) != cudaSuccess || galloc(p, &p->xbuf, p->nx) != cudaSuccess ||
@@ -347,7 +349,7 @@ static kfbi_status alloc_work(kfbi_problem* p) {
     return fail(p, KFBI_ERR_CUDA, "out of device memory");
   // what the operator expects to find: R zero off the (new) irregular nodes, u
   // zero on the boundary layer
-  KFBI_CUDA(p, cudaMemsetAsync(p->rhs_op, 0, sizeof(double) * nodes, p->stream));
+  KFBI_CUDA(p, cudaMemsetAsync(p->rhs, 0, sizeof(double) * nodes, p->stream));
   KFBI_TRY(launch_set_boundary(p, p->ugrid, nullptr));
   return gmres_create(p, kMaxKrylov);
 }
@@ -483,7 +485,7 @@ kfbi_status kfbi_destroy_problem(kfbi_problem* p) {
   box_destroy(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   if (p->ls_samples) cudaFree(p->ls_samples);
-  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->rhs_op, p->ugrid, p->ftilde, p->stencil_dev};
+  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->ugrid, p->ftilde, p->stencil_dev};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t e : p->prof.pool) cudaEventDestroy(e);

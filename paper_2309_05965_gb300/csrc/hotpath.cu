@@ -557,14 +557,17 @@ static void neighbour_table(kfbi_problem* p, std::vector<double>* coef, std::vec
       }
 }
 
+// Whether the data reach nodes off the interface (sources, outer values).
+static bool fills_grid(const kfbi_data* data) {
+  return data && (data->f_in || data->f_out || data->lapf_in || data->lapf_out || data->g_b);
+}
+
 kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* data,
                        double* rhs) {
   const Grid g = p->g;
   const double* d_nbc = p->nb_coef;
   const int8_t* d_off = p->nb_off;
-  const bool src = data && (data->f_in || data->f_out || data->lapf_in || data->lapf_out);
-  const bool gb = data && data->g_b;
-  if (src || gb) {
+  if (fills_grid(data)) {
     const double* fi = data->f_in;
     const double* fo = interior_bvp(p) ? nullptr : data->f_out;
     const double* li = data->lapf_in;
@@ -590,15 +593,22 @@ kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* da
 }
 
 // The operator's right-hand side: the corrections alone, assigned at the
-// irregular nodes of p->rhs_op, which is zero elsewhere.
+// irregular nodes of p->rhs, which is zero elsewhere.  (A clearing pass per
+// application would be a grid of writes; data clear up behind themselves instead,
+// on the stream, so that replayed graphs find the zeros too.)
 kfbi_status launch_rhs_operator(kfbi_problem* p, const double* cvals) {
   if (p->n_iface > 1)
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct_multi<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
-        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, p->nb_coef, cvals, p->rhs_op, 0));
+        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, p->nb_coef, cvals, p->rhs, 0));
   else
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
-        p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, p->nb_coef, cvals, p->rhs_op, 0));
+        p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, p->nb_coef, cvals, p->rhs, 0));
   KFBI_CUDA(p, cudaGetLastError());
+  return KFBI_OK;
+}
+
+kfbi_status reset_rhs(kfbi_problem* p, const kfbi_data* data) {
+  if (fills_grid(data)) KFBI_CUDA(p, cudaMemsetAsync(p->rhs, 0, sizeof(double) * p->g.nodes(), p->stream));
   return KFBI_OK;
 }
 

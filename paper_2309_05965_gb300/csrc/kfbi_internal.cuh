@@ -207,7 +207,7 @@ struct kfbi_problem {
   // box solver + work
   kfbi::BoxSolver* box = nullptr;
   double* cvals = nullptr;       // [n_ent]
-  double* rhs = nullptr;         // grid
+  double* rhs = nullptr;         // grid, between calls zero off the irregular nodes (reset_rhs)
   double* ugrid = nullptr;       // grid
   double* tvals = nullptr;       // [N_b]
   double* ftilde = nullptr;      // grid scratch
@@ -223,10 +223,6 @@ struct kfbi_problem {
   long long op_counts[KFBI_KC_COUNT] = {};
   double* xbuf = nullptr;
   double* ybuf = nullptr;
-  // the operator's right-hand side: only its entries at the irregular nodes are
-  // ever written, the rest stays zero (one grid of memory in place of a clearing
-  // pass per application)
-  double* rhs_op = nullptr;
   bool use_graphs = true;
   int nx = 0;                    // unknowns of the BIE: N_b, or 2 N_b for the general interface kind
   kfbi_problem* twin = nullptr;  // general interface kind: the kappa_2/sigma_2 operator (owned)
@@ -339,6 +335,9 @@ kfbi_status launch_collocation_fit(kfbi_problem* p, const double* a, const doubl
 kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* data,
                        double* rhs);
 kfbi_status launch_rhs_operator(kfbi_problem* p, const double* cvals);
+// p->rhs back to zero off the irregular nodes, as the operator expects it, after
+// launch_rhs put data with sources or outer values there
+kfbi_status reset_rhs(kfbi_problem* p, const kfbi_data* data);
 kfbi_status launch_correction_values_data(kfbi_problem* p, const double* a, const double* b,
                                           const kfbi_data* data, double* cvals);
 kfbi_status upload_neighbour_tables(kfbi_problem* p);
