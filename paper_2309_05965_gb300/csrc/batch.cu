@@ -437,10 +437,15 @@ kfbi_status kfbi_evaluate_batch(kfbi_batch* b, const kfbi_data* data, const doub
     if (mu) bb[k] = densities[k];
   }
   KFBI_TRY(batch_potentials(b, a.data(), mu ? bb.data() : nullptr, data, mu));
+  // every layer before any output: outputs may be the buffers of the outer values
+  if (mu)
+    for (int k = 0; k < n; ++k)
+      if (data[k].g_b) KFBI_TRY(launch_set_boundary(b->ps[k], b->ps[k]->ugrid, data[k].g_b));
   for (int k = 0; k < n; ++k) {
-    KFBI_CUDA(p0, cudaMemcpyAsync(u_grids[k], b->ps[k]->ugrid, sizeof(double) * b->ps[k]->g.nodes(),
-                                  cudaMemcpyDeviceToDevice, b->stream));
-    if (mu && data[k].g_b) KFBI_TRY(launch_set_boundary(b->ps[k], u_grids[k], data[k].g_b));
+    kfbi_problem* p = b->ps[k];
+    KFBI_CUDA(p0, cudaMemcpyAsync(u_grids[k], p->ugrid, sizeof(double) * p->g.nodes(), cudaMemcpyDeviceToDevice,
+                                  b->stream));
+    if (mu) KFBI_TRY(reset_boundary(p, &data[k]));
   }
   return KFBI_OK;
 }
