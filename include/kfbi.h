@@ -142,9 +142,11 @@ typedef struct {
                              before application j inside kfbi_gmres_solve the
                              refinement stops at max(box_rtol, omega rtol ||b|| /
                              ||r_j||) (relaxation as the residual falls, after
-                             Simoncini & Szyld 2003; half of omega for the
-                             interface kinds); right-hand side, starts,
-                             restarts and evaluation stay at box_rtol           */
+                             Simoncini & Szyld 2003; KFBI_INTERFACE_MU takes
+                             half of omega, and stops before the first
+                             refinement by a margin that grows with the
+                             contrast); right-hand side, starts, restarts
+                             and evaluation stay at box_rtol                    */
 } kfbi_config;
 
 /* Problem data (Sec. 2).  f_* are the physical right-hand sides f of eqs.

@@ -71,7 +71,6 @@ struct BoxSolver {
   double* tol_dev = nullptr;  // the refinement tolerance the checks read (relaxed inside GMRES)
   int* conv = nullptr;        // device flag
   int refine_steps = 4;
-  double margin = 10.0;       // first_margin of the problem
   double tol = 1e-13;
   // exact residual of the mixed path in fixed point: mult h^2 A_h = S - kappa h^2 K
   // with S integer weights w[c] by the number c of nonzero offsets and
@@ -1701,12 +1700,13 @@ kfbi_status mg_solve(kfbi_problem* p, const double* rhs, double* u);
 kfbi_status mg_last_residual(kfbi_problem* p, double* rel, int* converged);
 
 // Margin between the error estimate of an unrefined FP32 solve and the relaxed
-// tolerance it may stop at: 10, times the contrast of an interface problem, whose
+// tolerance it may stop at: 10, times the contrast of a mu-form problem, whose
 // operator nearly annihilates the constants (by the contrast): the mean of the
 // rounding errors, of which the estimate (a maximum norm) says nothing, reaches the
-// solution larger by that.  See relax_omega for figures.
+// solution larger by that.  See relax_omega for figures.  (The second side operator
+// of a general problem is set up as a mu-form one, but belongs to its parent's rule.)
 static double first_margin(const kfbi_problem* p) {
-  if (p->cfg.kind != KFBI_INTERFACE_MU && p->cfg.kind != KFBI_INTERFACE_GENERAL) return 10.0;
+  if (p->parent || p->cfg.kind != KFBI_INTERFACE_MU) return 10.0;
   const double a = std::fabs(p->cfg.sigma_in), b = std::fabs(p->cfg.sigma_out);
   return 10.0 * std::max(a / b, b / a);
 }
@@ -1822,7 +1822,6 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, dalloc(&B->conv, 1));
   KFBI_CUDA(p, dalloc(&B->tol_dev, 1));
   B->tol = p->cfg.box_rtol > 0 ? p->cfg.box_rtol : 1e-13;
-  B->margin = first_margin(p);
   KFBI_CUDA(p, cudaMemcpy(B->tol_dev, &B->tol, sizeof(double), cudaMemcpyHostToDevice));
   B->refine_steps = p->cfg.box_max_iters > 0 ? std::min(p->cfg.box_max_iters, kMaxSteps) : 5;
   int dev = 0, optin = 0;
@@ -1945,6 +1944,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   // the host-side diagnostics (box_last_residual).
   cudaStream_t st = p->stream;
   unsigned long long* slot = B->nrm + 9;   // step s: slot + 2 s
+  const double margin = first_margin(p);
   {
     PassPlan P0 = plan_passes<float>(p, rhs, 1, u, 0, nullptr, slot);
     P0.args[0].zero_nrm = B->nrm;
@@ -1959,7 +1959,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   launch_fix0(p, g, B->work32, rhs, slot + 1, B->multh2, B->kc, B->fixd, B->fixf, B->ufix, B->rfix,
               B->refine_steps > 1 ? nullptr : u, st);
   if (B->refine_steps == 1)
-    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, 0, false}));
+    KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, margin, 0, false}));
   float* r32 = reinterpret_cast<float*>(B->res);
   PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, nullptr);
   {
@@ -1974,7 +1974,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   const FixStencil W{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB};
   for (int it = 1; it < B->refine_steps; ++it) {
     launch_res_fix(p, g, W, B->rfix, B->ufix, B->fixd, B->fixf, r32, B->conv, u, st,
-                   StepCheck{B->nrm, B->tol_dev, B->conv, B->margin, it - 1, it + 1 == B->refine_steps});
+                   StepCheck{B->nrm, B->tol_dev, B->conv, margin, it - 1, it + 1 == B->refine_steps});
     PassArgs& last = PK.args[PK.npass - 1];
     last.corr_max = slot + 2 * it;
     last.uout = it + 1 < B->refine_steps ? nullptr : u;   // the last step also writes the FP64 solution
@@ -2530,7 +2530,7 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
     const int n1 = p->g.n + 1;
     rstart[i + 1] = rstart[i] + div_up(n1, 128) * div_up(d == 2 ? n1 : n1 * n1, kFixRows);
     box[i] = BoxDesc{p->g, FixStencil{B->w[0], B->w[1], B->w[2], B->w[3], B->kA, B->kB}, B->multh2, B->kc, B->tol,
-                     B->margin, rhs[i], p->ugrid, B->work32, B->ufix, B->rfix, r32, B->fixd, B->fixf, B->nrm, B->conv,
+                     first_margin(p), rhs[i], p->ugrid, B->work32, B->ufix, B->rfix, r32, B->fixd, B->fixf, B->nrm, B->conv,
                      tol_dev ? tol_dev + i : nullptr};
   }
   bb->steps = 0;

@@ -353,18 +353,24 @@ __global__ void k_relax_tol(const double* __restrict__ thr, const double* __rest
 
 }  // namespace
 
-// The omega of the relaxed tolerance: half of cfg.relax for the interface kinds.
-// Flower 1024^2, contrast 1000, rtol 1e-8, where unrelaxed solves give an error of
-// 5.176e-9 in 28 refinement steps, by the margin of a first solve's stop
-// (first_margin) and this omega:
-//   omega               0.02   0.03   0.05   0.07   0.1
-//   margin 10           5.40   6.90   6.90   4.93   6.36   18..14 steps
-//   margin 10 contrast  5.176  5.169  5.153  5.059  6.54   22..17 steps
-// With a margin of 10 the rounding of the FP32 transforms decides; from 0.07 on the
-// relaxation itself does.
+// The omega of the relaxed tolerance: cfg.relax, half of it for the mu-form, whose
+// operator nearly annihilates the constants (by the contrast), so that what a solve
+// leaves out reaches the solution larger by the contrast.  Error against that of
+// unrelaxed solves / refinement steps, flowers, rtol 1e-8, by the margin of a first
+// solve's stop (first_margin) and omega / cfg.relax, at cfg.relax 0.03, 0.05, 0.1:
+//   grid, contrast     margin 10, whole                 margin 10 contrast, whole      the same, half
+//   1024^2, 10         1.00/13  0.95/11  0.95/11        1.00/14  1.00/13  1.00/13      1.00/14  1.00/14  1.00/13
+//   1024^2, 100        0.99/16  1.03/15  1.03/15        1.00/18  1.00/17  1.00/16      1.00/18  1.00/18  1.00/17
+//   1024^2, 1000       1.02/17  1.02/17  1.34/14        1.00/21  0.99/20  1.23/17      1.00/22  1.00/21  0.99/20
+//   512^2, 1000        0.87/17  0.87/17  0.95/14        1.00/21  1.00/21  1.03/18      1.00/23  1.00/22  1.00/21
+//   1024^2, 10000      0.97/14  0.97/14  7.7e4/9        0.67/20  0.67/20  0.67/19      0.28/21  0.67/20  0.67/20
+// The margin alone decides at 10000 (a margin of 10 fails); what is left at 1000 and
+// 0.1 is the relaxation itself, which also never stopping at a first solve leaves
+// (1.23/19).  The general kind shows neither: flower 512^2, margin 10, whole omega,
+// contrast 4 1.00/24  1.00/22  1.00/20, contrast 25 0.93/28  0.93/28  0.95/26 (by
+// the mu-form's rule 1.00/27..24 and 0.95/37..0.87/33; unrelaxed 48 and 84 steps).
 double relax_omega(const kfbi_problem* p) {
-  const bool interface = p->cfg.kind == KFBI_INTERFACE_MU || p->cfg.kind == KFBI_INTERFACE_GENERAL;
-  return interface ? 0.5 * p->cfg.relax : p->cfg.relax;
+  return p->cfg.kind == KFBI_INTERFACE_MU ? 0.5 * p->cfg.relax : p->cfg.relax;
 }
 
 // The relaxed refinement tolerance before an operator application inside
