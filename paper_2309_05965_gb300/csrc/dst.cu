@@ -13,7 +13,7 @@
 // of one axis, each CTA P line pairs in shared memory, natural order in and
 // out (self-sorting Stockham FFTs):
 //   * FP64 path, N = 64..1024 (k_dst_mma, dst_mma.cuh): exact fixed-point
-//     matrix products on the tensor cores; other N (k_dst_pass<double>):
+//     matrix products on the tensor cores; other N (k_dst_pass):
 //     radix-4 stages (and one radix-2 stage) over the shared buffer, bound by
 //     GB300's FP64 pipe;
 //   * FP32 path (k_dst32<LOGL, P, STR>): register DFTs of radix 16, a thread
@@ -54,9 +54,7 @@ constexpr int kNrm = 9 + 2 * kMaxSteps;  // entries of BoxSolver::nrm
 struct BoxSolver {
   int L = 0, logL = 0;
   double* tw64 = nullptr;     // L/2 twiddles exp(-2 pi i t / L)
-  float* tw32 = nullptr;
   float* twst = nullptr;      // FP32 stage twiddle tables (stage_twiddles)
-  double* cosv = nullptr;     // cos(k pi / N), k = 0..N
   double* s64 = nullptr;      // sin^2(k pi / 2N), k = 0..N
   float* s32 = nullptr;
   double* scale64 = nullptr;  // FP64 path: (2/N)^d / lambda on the mode grid (N-1)^d
@@ -89,36 +87,28 @@ namespace {
 struct PassArgs {
   const void* src;
   void* dst;
-  int src64, dst64, accumulate;
+  int src64;                // FP32 path: src is FP64 (the first pass)
   long long sa, sb, es;     // line strides: line(a, b) at a*sa + b*sb, element j at +j*es
   int n;                    // N
   int logL;
   const void* tw;
   const void* frag;         // FP64 path: sine-matrix digits (null: the FFT kernel)
   // spectral scaling (fused pass only)
-  const double* cosv;
   const float* s32;           // sin^2(k pi/2N) for the FP32 path
   const double* scale64;      // precomputed scale for the FP64 path (mode grid, C order)
-  double ih2, kt, gscale;   // gscale = (2/N)^d
+  double kt, gscale;        // kappa h^2, (2/N)^d h^2
   int d, order;
   int fused;
-  int amode;                // 1 if the a index is a mode index of the scaling (3D)
   const int* skip;          // convergence flag (skip when *skip != 0), may be null
   unsigned long long* corr_max;   // last pass: max |correction|, max |u + correction|
-  float* delta_out;               // accumulate pass: also keep the FP32 correction (in place)
   long long* dstfix;              // last pass of a refinement step: u_fix += round(delta 2^F)
   const void* twst;               // FP32 path: stage twiddle tables (stage_twiddles)
-  const float* fixf;              // [0..1] 2^Fa, 2^Fb; [2..3] 2^-Fa, 2^-Fb (k_fix_scale)
+  const float* fixf;              // [0..1] 2^Fa, 2^Fb; [2..3] 2^-Fa, 2^-Fb (fix_scale_of)
   const double* fixd;             // [1] mult h^2 2^-F (with uout)
   double* uout;                   // with dstfix: also u = u_fix mult h^2 2^-F in FP64
   unsigned long long* zero_nrm;   // first pass of a mixed solve: CTA 0 clears nrm (but [7], [8]) and
   int* zero_conv;                 // the convergence flag before anything reads them
 };
-
-template <typename T>
-__device__ __forceinline__ T ld(const void* p, int is64, long long i) {
-  return is64 ? (T)static_cast<const double*>(p)[i] : (T)static_cast<const float*>(p)[i];
-}
 
 // lambda h^2 with s_k = sin^2(k pi / 2N) (c_k = 1 - 2 s_k), free of the
 // cancellation of the cosine form for low modes:
@@ -182,8 +172,8 @@ __device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
 // memory, natural order in and out, radix-4 stages and one radix-2 stage when
 // k is odd.  x and y are ping-pong buffers; returns the buffer holding the
 // result.  tw[t] = exp(-2 pi i t / L), t in [0, L).
-template <typename T, int P>
-__device__ Cx<T>* fft_stockham(Cx<T>* x, Cx<T>* y, int L, const Cx<T>* __restrict__ tw) {
+template <int P>
+__device__ Cx<double>* fft_stockham(Cx<double>* x, Cx<double>* y, int L, const Cx<double>* __restrict__ tw) {
   int n = L, s = 1, ls = 0;
   const int lq4 = __ffs(L) - 3;     // log2(L / 4)
   while (n >= 4) {
@@ -195,23 +185,23 @@ __device__ Cx<T>* fft_stockham(Cx<T>* x, Cx<T>* y, int L, const Cx<T>* __restric
       const int b = t & (q4 - 1);
       const int q = b & (s - 1);
       const int p = b >> ls;
-      const Cx<T>* xx = x + pr * L;
-      Cx<T>* yy = y + pr * L;
-      const Cx<T> a = xx[q + s * p];
-      const Cx<T> bb = xx[q + s * (p + m)];
-      const Cx<T> c = xx[q + s * (p + 2 * m)];
-      const Cx<T> d = xx[q + s * (p + 3 * m)];
-      const Cx<T> apc = {a.x + c.x, a.y + c.y}, amc = {a.x - c.x, a.y - c.y};
-      const Cx<T> bpd = {bb.x + d.x, bb.y + d.y};
-      const Cx<T> jbmd = {bb.y - d.y, d.x - bb.x};   // -i (b - d)
+      const Cx<double>* xx = x + pr * L;
+      Cx<double>* yy = y + pr * L;
+      const Cx<double> a = xx[q + s * p];
+      const Cx<double> bb = xx[q + s * (p + m)];
+      const Cx<double> c = xx[q + s * (p + 2 * m)];
+      const Cx<double> d = xx[q + s * (p + 3 * m)];
+      const Cx<double> apc = {a.x + c.x, a.y + c.y}, amc = {a.x - c.x, a.y - c.y};
+      const Cx<double> bpd = {bb.x + d.x, bb.y + d.y};
+      const Cx<double> jbmd = {bb.y - d.y, d.x - bb.x};   // -i (b - d)
       const int o = q + s * 4 * p;
       yy[o] = {apc.x + bpd.x, apc.y + bpd.y};
-      yy[o + s] = cmul(Cx<T>{amc.x + jbmd.x, amc.y + jbmd.y}, tw[p * tstep]);
-      yy[o + 2 * s] = cmul(Cx<T>{apc.x - bpd.x, apc.y - bpd.y}, tw[2 * p * tstep]);
-      yy[o + 3 * s] = cmul(Cx<T>{amc.x - jbmd.x, amc.y - jbmd.y}, tw[3 * p * tstep]);
+      yy[o + s] = cmul(Cx<double>{amc.x + jbmd.x, amc.y + jbmd.y}, tw[p * tstep]);
+      yy[o + 2 * s] = cmul(Cx<double>{apc.x - bpd.x, apc.y - bpd.y}, tw[2 * p * tstep]);
+      yy[o + 3 * s] = cmul(Cx<double>{amc.x - jbmd.x, amc.y - jbmd.y}, tw[3 * p * tstep]);
     }
     __syncthreads();
-    Cx<T>* tmp = x;
+    Cx<double>* tmp = x;
     x = y;
     y = tmp;
     n = m;
@@ -223,9 +213,9 @@ __device__ Cx<T>* fft_stockham(Cx<T>* x, Cx<T>* y, int L, const Cx<T>* __restric
     for (int t = threadIdx.x; t < q2 * P; t += blockDim.x) {
       const int pr = t >> (lq4 + 1);
       const int q = t & (q2 - 1);    // p = 0, m = 1: no twiddle
-      const Cx<T>* xx = x + pr * L;
-      Cx<T>* yy = y + pr * L;
-      const Cx<T> a = xx[q], b = xx[q + s];
+      const Cx<double>* xx = x + pr * L;
+      Cx<double>* yy = y + pr * L;
+      const Cx<double> a = xx[q], b = xx[q + s];
       yy[q] = {a.x + b.x, a.y + b.y};
       yy[q + s] = {a.x - b.x, a.y - b.y};
     }
@@ -237,12 +227,12 @@ __device__ Cx<T>* fft_stockham(Cx<T>* x, Cx<T>* y, int L, const Cx<T>* __restric
 
 // One DST-I pass over P line pairs (see file comment): line pairs starting at
 // b0 = 1 + 2 P bx of the line family a = by + 1.
-template <typename T, int P>
+template <int P>
 __device__ __forceinline__ void dst_pass_device(const PassArgs& A, int bx, int by,
                                                 unsigned char* smraw) {
-  Cx<T>* z = reinterpret_cast<Cx<T>*>(smraw);
-  Cx<T>* zb = z + (size_t)P * 2 * A.n;      // ping-pong buffer
-  const Cx<T>* tw = static_cast<const Cx<T>*>(A.tw);
+  Cx<double>* z = reinterpret_cast<Cx<double>*>(smraw);
+  Cx<double>* zb = z + (size_t)P * 2 * A.n;      // ping-pong buffer
+  const Cx<double>* tw = static_cast<const Cx<double>*>(A.tw);
   const int n = A.n;
   const int L = 2 * n;
   const int nm1 = n - 1;
@@ -262,9 +252,9 @@ __device__ __forceinline__ void dst_pass_device(const PassArgs& A, int bx, int b
       j = 1 + t / (2 * P);
     }
     const int b = b0 + q;
-    T v = (T)0;
-    if (b <= nm1) v = ld<T>(A.src, A.src64, abase + (long long)b * A.sb + (long long)j * A.es);
-    Cx<T>* zz = z + (q >> 1) * L;
+    double v = 0.0;
+    if (b <= nm1) v = static_cast<const double*>(A.src)[abase + (long long)b * A.sb + (long long)j * A.es];
+    Cx<double>* zz = z + (q >> 1) * L;
     if (q & 1) {
       zz[j].y = v;
       zz[L - j].y = -v;
@@ -274,12 +264,12 @@ __device__ __forceinline__ void dst_pass_device(const PassArgs& A, int bx, int b
     }
   }
   for (int t = threadIdx.x; t < P; t += blockDim.x) {
-    z[t * L] = {(T)0, (T)0};
-    z[t * L + n] = {(T)0, (T)0};
+    z[t * L] = {0.0, 0.0};
+    z[t * L + n] = {0.0, 0.0};
   }
   __syncthreads();
-  z = fft_stockham<T, P>(z, zb, L, tw);
-  zb = (z == reinterpret_cast<Cx<T>*>(smraw)) ? z + (size_t)P * L : reinterpret_cast<Cx<T>*>(smraw);
+  z = fft_stockham<P>(z, zb, L, tw);
+  zb = (z == reinterpret_cast<Cx<double>*>(smraw)) ? z + (size_t)P * L : reinterpret_cast<Cx<double>*>(smraw);
   if (A.fused) {
     // spectral division in place (natural order; Z_{L-k} = -Z_k makes the
     // rescaled sequence the odd extension of the next input), then the same FFT
@@ -287,43 +277,25 @@ __device__ __forceinline__ void dst_pass_device(const PassArgs& A, int bx, int b
       const int pr = t >> A.logL;
       const int pos = t & (L - 1);
       const int k = pos;
-      Cx<T>* zz = z + pr * L;
+      Cx<double>* zz = z + pr * L;
       if (k == 0 || k == n) {
-        zz[pos] = {(T)0, (T)0};
+        zz[pos] = {0.0, 0.0};
         continue;
       }
       const int km = k < n ? k : L - k;     // the mode of k and of L - k
       const int bA = b0 + 2 * pr, bB = min(bA + 1, nm1);
-      T scA, scB;
-      if (sizeof(T) == 8) {
-        // FP64: precomputed (2/N)^d h^2 / (lambda h^2), table index (km, a, b)
-        const long long m1 = nm1;
-        long long base = (A.d == 2) ? (long long)(km - 1) * m1
-                                    : ((long long)(km - 1) * m1 + (a - 1)) * m1;
-        scA = (T)A.scale64[base + bA - 1];
-        scB = (T)A.scale64[base + bB - 1];
-      } else {
-        const float kh2 = (float)A.kt;   // kappa h^2 (precomputed on the host)
-        const float g = (float)A.gscale;
-        const float sk = A.s32[km];
-        const float sa = A.d == 3 ? A.s32[a] : 0.f;
-        if (A.d == 2) {
-          scA = (T)(g / lam_h2<float>(2, A.order, kh2, sk, A.s32[bA], 0.f));
-          scB = (T)(g / lam_h2<float>(2, A.order, kh2, sk, A.s32[bB], 0.f));
-        } else {
-          scA = (T)(g / lam_h2<float>(3, A.order, kh2, sk, sa, A.s32[bA]));
-          scB = (T)(g / lam_h2<float>(3, A.order, kh2, sk, sa, A.s32[bB]));
-        }
-      }
-      Cx<T> Z = zz[pos];
+      // precomputed (2/N)^d h^2 / (lambda h^2), table index (km, a, b)
+      const long long m1 = nm1;
+      const long long base = (A.d == 2) ? (long long)(km - 1) * m1 : ((long long)(km - 1) * m1 + (a - 1)) * m1;
+      const double scA = A.scale64[base + bA - 1], scB = A.scale64[base + bB - 1];
+      Cx<double> Z = zz[pos];
       // A_k = -Im(Z)/2 (line bA), B_k = Re(Z)/2 (line bB); repack x = sA A + i sB B
-      zz[pos] = {scA * ((T)-0.5 * Z.y), scB * ((T)0.5 * Z.x)};
+      zz[pos] = {scA * (-0.5 * Z.y), scB * (0.5 * Z.x)};
     }
     __syncthreads();
-    z = fft_stockham<T, P>(z, zb, L, tw);
+    z = fft_stockham<P>(z, zb, L, tw);
   }
   // extract S_k = -Im(Z_k)/2 (first line) and Re(Z_k)/2 (second line) and store
-  float dmx = 0.f, umx = 0.f;
   for (int t = threadIdx.x; t < nval; t += blockDim.x) {
     int j, q;
     if (contig) {
@@ -335,41 +307,16 @@ __device__ __forceinline__ void dst_pass_device(const PassArgs& A, int bx, int b
     }
     const int b = b0 + q;
     if (b > nm1) continue;
-    const Cx<T>* zz = z + (q >> 1) * L;
-    Cx<T> Z = zz[j];
-    T v = (q & 1) ? (T)0.5 * Z.x : (T)-0.5 * Z.y;
-    long long off = abase + (long long)b * A.sb + (long long)j * A.es;
-    if (A.dst64) {
-      double* o = static_cast<double*>(A.dst);
-      double nv = A.accumulate ? o[off] + (double)v : (double)v;
-      o[off] = nv;
-      if (A.delta_out) A.delta_out[off] = (float)v;
-      if (A.corr_max) {
-        dmx = fmax_nan(dmx, fabsf((float)v));
-        umx = fmax_nan(umx, fabsf((float)nv));
-      }
-    } else {
-      static_cast<float*>(A.dst)[off] = (float)v;
-    }
-  }
-  if (A.corr_max) {
-    for (int o = 16; o > 0; o >>= 1) {
-      dmx = fmax_nan(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
-      umx = fmax_nan(umx, __shfl_xor_sync(0xffffffffu, umx, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      // non-negative doubles order like their bit patterns
-      if (!(dmx <= 0.f)) atomicMax(A.corr_max, (unsigned long long)__double_as_longlong((double)dmx));
-      if (!(umx <= 0.f)) atomicMax(A.corr_max + 1, (unsigned long long)__double_as_longlong((double)umx));
-    }
+    const Cx<double>* zz = z + (q >> 1) * L;
+    Cx<double> Z = zz[j];
+    static_cast<double*>(A.dst)[abase + (long long)b * A.sb + (long long)j * A.es] = (q & 1) ? 0.5 * Z.x : -0.5 * Z.y;
   }
 }
 
-template <typename T, int P>
+template <int P>
 __global__ void __launch_bounds__(256) k_dst_pass(PassArgs A) {
-  if (A.skip && *A.skip) return;
   extern __shared__ unsigned char smraw[];
-  dst_pass_device<T, P>(A, blockIdx.x, blockIdx.y, smraw);
+  dst_pass_device<P>(A, blockIdx.x, blockIdx.y, smraw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1494,11 +1441,11 @@ __global__ void k_absmax32(long long tot, const float* __restrict__ x, unsigned 
   if ((threadIdx.x & 31) == 0 && !(m <= 0.f)) atomicMax(out, (unsigned long long)__double_as_longlong((double)m));
 }
 
-template <typename T, int P>
+template <int P>
 void launch_pass_p(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st) {
   dim3 grid((unsigned)((npairs_b + P - 1) / P), (unsigned)na);
-  size_t smem = sizeof(Cx<T>) * (size_t)(2 * A.n) * P * 2;
-  KFBI_LAUNCH(p, KFBI_KC_DST, k_dst_pass<T, P><<<grid, 256, smem, st>>>(A));
+  size_t smem = sizeof(Cx<double>) * (size_t)(2 * A.n) * P * 2;
+  KFBI_LAUNCH(p, KFBI_KC_DST, k_dst_pass<P><<<grid, 256, smem, st>>>(A));
 }
 
 template <int LOGL, int P, bool STR>
@@ -1573,36 +1520,30 @@ void launch_pass_mma(kfbi_problem* p, const PassArgs& A, int na, cudaStream_t st
   }
 }
 
-// pairs per CTA: enough butterflies for 256 threads (P L / 4 >= 256), at least
-// `pmin` (strided passes read 2 P adjacent lines per row)
-template <typename T>
-void launch_pass(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st, int pmin) {
-  if (sizeof(T) == 4) {
-    launch_pass32(p, A, npairs_b, na, st);
-    return;
-  }
+// FP64 pass; pairs per CTA of the FFT kernel: enough butterflies for 256 threads
+// (P L / 4 >= 256), at least `pmin` (strided passes read 2 P adjacent lines per row)
+void launch_pass64(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cudaStream_t st, int pmin) {
   if (A.frag) {
     launch_pass_mma(p, A, na, st);
     return;
   }
   const int L = 2 * A.n;
   int P = std::max(pmin, 1024 / L);
-  if (sizeof(T) == 8 && L >= 2048) P = std::min(P, 1);
+  if (L >= 2048) P = std::min(P, 1);
   // small grids: fewer pairs per CTA until the pass has two CTAs per SM (a
   // 64^2 grid otherwise runs on 4 CTAs, each bound by one SM's FP64 rate)
   while (P > pmin && (long long)((npairs_b + P - 1) / P) * na < 2 * 152) P /= 2;
-  if (P >= 8) launch_pass_p<T, 8>(p, A, npairs_b, na, st);
-  else if (P >= 4) launch_pass_p<T, 4>(p, A, npairs_b, na, st);
-  else if (P >= 2) launch_pass_p<T, 2>(p, A, npairs_b, na, st);
-  else launch_pass_p<T, 1>(p, A, npairs_b, na, st);
+  if (P >= 8) launch_pass_p<8>(p, A, npairs_b, na, st);
+  else if (P >= 4) launch_pass_p<4>(p, A, npairs_b, na, st);
+  else if (P >= 2) launch_pass_p<2>(p, A, npairs_b, na, st);
+  else launch_pass_p<1>(p, A, npairs_b, na, st);
 }
 
 // The dynamic shared-memory limit is a per-kernel, process-wide attribute:
 // raise it once to the device maximum (problems of different N share it).
-template <typename T, int P>
+template <int P>
 cudaError_t set_smem(int max_optin) {
-  return cudaFuncSetAttribute(k_dst_pass<T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              max_optin);
+  return cudaFuncSetAttribute(k_dst_pass<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin);
 }
 
 template <int LOGN, int W>
@@ -1611,10 +1552,11 @@ cudaError_t set_smem_mma() {
                               (int)Mma<LOGN, W>::SMEM);
 }
 
-// The passes of one DST solve of `src` (grid, FP64 or FP32) into `dst` (grid,
-// FP64), overwriting or accumulating, with a work buffer of type T: the
-// argument block of each pass, the pairs-per-CTA floor (strided passes read
-// 2 P adjacent lines) and the number of line families.
+// The passes of one DST solve of `src` (FP64 grid; FP32 path: or FP32) into
+// `dst` (FP64; FP32 path: what the caller sets for the last pass), with a work
+// grid of type T: the argument block of each pass, the FFT kernel's
+// pairs-per-CTA floor (strided passes read 2 P adjacent lines) and the number of
+// line families.
 struct PassPlan {
   PassArgs args[5];
   int pmin[5];
@@ -1622,44 +1564,35 @@ struct PassPlan {
 };
 
 template <typename T>
-PassPlan plan_passes(kfbi_problem* p, const void* src, int src64, double* dst, int accumulate,
-                     const int* skip, unsigned long long* corr_max) {
+PassPlan plan_passes(kfbi_problem* p, const void* src, int src64, void* dst, const int* skip) {
+  constexpr bool f64 = std::is_same<T, double>::value;
   BoxSolver* B = p->box;
   const Grid g = p->g;
   const int n = g.n, n1 = n + 1;
-  T* work = std::is_same<T, double>::value ? reinterpret_cast<T*>(B->work64)
-                                            : reinterpret_cast<T*>(B->work32);
-  const void* tw = std::is_same<T, double>::value ? (const void*)B->tw64 : (const void*)B->tw32;
+  void* work = f64 ? (void*)B->work64 : (void*)B->work32;
   PassArgs A;
   memset(&A, 0, sizeof(A));
   A.n = n;
   A.logL = B->logL;
-  A.tw = tw;
+  A.tw = B->tw64;
   A.twst = B->twst;
-  A.cosv = B->cosv;
   A.s32 = B->s32;
   A.scale64 = B->scale64;
-  A.frag = std::is_same<T, double>::value ? B->frag : nullptr;
-  A.ih2 = 1.0 / (g.h * g.h);
+  A.frag = f64 ? B->frag : nullptr;
   A.kt = p->kt * g.h * g.h;   // kappa h^2
   A.d = g.d;
   A.order = p->cfg.order;
   A.skip = skip;
   A.gscale = (g.d == 2 ? (2.0 / n) * (2.0 / n) : (2.0 / n) * (2.0 / n) * (2.0 / n)) * g.h * g.h;
-  const int is64 = std::is_same<T, double>::value ? 1 : 0;
   PassPlan P;
   P.npairs = n / 2;   // ceil((N-1)/2) for even N
   P.na = g.d == 2 ? 1 : n - 1;
-  auto add = [&](const void* s, int s64, void* d, int d64, int acc, long long sa, long long sb,
-                 long long es, int fused, int pmin) {
+  auto add = [&](const void* s, int s64, void* d, long long sa, long long sb, long long es, int fused, int pmin) {
     PassArgs& Q = P.args[P.npass];
     Q = A;
     Q.src = s;
     Q.src64 = s64;
     Q.dst = d;
-    Q.dst64 = d64;
-    Q.accumulate = acc;
-    Q.corr_max = (d64 && acc) ? corr_max : nullptr;
     Q.sa = sa;
     Q.sb = sb;
     Q.es = es;
@@ -1668,26 +1601,24 @@ PassPlan plan_passes(kfbi_problem* p, const void* src, int src64, double* dst, i
     ++P.npass;
   };
   if (g.d == 2) {
-    add(src, src64, work, is64, 0, 0, n1, 1, 0, 1);          // axis 1, lines b = i0
-    add(work, is64, work, is64, 0, 0, 1, n1, 1, 2);          // axis 0 fused, lines b = i1
-    add(work, is64, dst, 1, accumulate, 0, n1, 1, 0, 1);     // axis 1
+    add(src, src64, work, 0, n1, 1, 0, 1);          // axis 1, lines b = i0
+    add(work, f64, work, 0, 1, n1, 1, 2);           // axis 0 fused, lines b = i1
+    add(work, f64, dst, 0, n1, 1, 0, 1);            // axis 1
   } else {
     const long long s0 = (long long)n1 * n1;
-    add(src, src64, work, is64, 0, s0, n1, 1, 0, 1);         // axis 2, lines (i0, i1)
-    add(work, is64, work, is64, 0, s0, 1, n1, 0, 2);         // axis 1, lines (i0, i2)
-    add(work, is64, work, is64, 0, n1, 1, s0, 1, 2);         // axis 0 fused, lines (i1, i2)
-    add(work, is64, work, is64, 0, s0, 1, n1, 0, 2);         // axis 1
-    add(work, is64, dst, 1, accumulate, s0, n1, 1, 0, 1);    // axis 2
+    add(src, src64, work, s0, n1, 1, 0, 1);         // axis 2, lines (i0, i1)
+    add(work, f64, work, s0, 1, n1, 0, 2);          // axis 1, lines (i0, i2)
+    add(work, f64, work, n1, 1, s0, 1, 2);          // axis 0 fused, lines (i1, i2)
+    add(work, f64, work, s0, 1, n1, 0, 2);          // axis 1
+    add(work, f64, dst, s0, n1, 1, 0, 1);           // axis 2
   }
   return P;
 }
 
-template <typename T>
-kfbi_status dst_solve_t(kfbi_problem* p, const void* src, int src64, double* dst, int accumulate,
-                        const int* skip, unsigned long long* corr_max = nullptr) {
-  PassPlan P = plan_passes<T>(p, src, src64, dst, accumulate, skip, corr_max);
-  for (int k = 0; k < P.npass; ++k)
-    launch_pass<T>(p, P.args[k], P.npairs, P.na, p->stream, P.pmin[k]);
+// FP64 path: u = A_h^{-1} rhs at the interior nodes
+kfbi_status dst_solve64(kfbi_problem* p, const double* rhs, double* u) {
+  const PassPlan P = plan_passes<double>(p, rhs, 1, u, nullptr);
+  for (int k = 0; k < P.npass; ++k) launch_pass64(p, P.args[k], P.npairs, P.na, p->stream, P.pmin[k]);
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
 }
@@ -1724,16 +1655,11 @@ kfbi_status box_create(kfbi_problem* p) {
   B->logL = 0;
   while ((1 << B->logL) < B->L) ++B->logL;
   std::vector<double> tw(2 * B->L);    // interleaved re, im over the full circle
-  std::vector<float> tw32(2 * B->L);
   for (int t = 0; t < B->L; ++t) {
     double ang = -2.0 * M_PI * (double)t / (double)B->L;
     tw[2 * t] = std::cos(ang);
     tw[2 * t + 1] = std::sin(ang);
-    tw32[2 * t] = (float)tw[2 * t];
-    tw32[2 * t + 1] = (float)tw[2 * t + 1];
   }
-  std::vector<double> cs(n + 1);
-  for (int k = 0; k <= n; ++k) cs[k] = std::cos((double)k * M_PI / (double)n);
   std::vector<double> sv(n + 1);
   std::vector<float> sv32(n + 1);
   for (int k = 0; k <= n; ++k) {
@@ -1746,16 +1672,12 @@ kfbi_status box_create(kfbi_problem* p) {
   KFBI_CUDA(p, cudaMemcpy(B->s64, sv.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice));
   KFBI_CUDA(p, cudaMemcpy(B->s32, sv32.data(), sizeof(float) * (n + 1), cudaMemcpyHostToDevice));
   KFBI_CUDA(p, dalloc(&B->tw64, 2 * B->L));
-  KFBI_CUDA(p, dalloc(&B->tw32, 2 * B->L));
-  KFBI_CUDA(p, dalloc(&B->cosv, n + 1));
   KFBI_CUDA(p, cudaMemcpy(B->tw64, tw.data(), sizeof(double) * 2 * B->L, cudaMemcpyHostToDevice));
-  KFBI_CUDA(p, cudaMemcpy(B->tw32, tw32.data(), sizeof(float) * 2 * B->L, cudaMemcpyHostToDevice));
   {
     const std::vector<float> ts = stage_twiddles(B->logL);
     KFBI_CUDA(p, dalloc(&B->twst, ts.size()));
     KFBI_CUDA(p, cudaMemcpy(B->twst, ts.data(), sizeof(float) * ts.size(), cudaMemcpyHostToDevice));
   }
-  KFBI_CUDA(p, cudaMemcpy(B->cosv, cs.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice));
   const long long nodes = g.nodes();
   if (p->cfg.precision == KFBI_MIXED) {
     KFBI_CUDA(p, dalloc(&B->work32, nodes));
@@ -1837,10 +1759,10 @@ kfbi_status box_create(kfbi_problem* p) {
                 p->cfg.precision == KFBI_MIXED ? "N too large for the shared-memory DST on this device"
                                                : "N too large for the FP64 shared-memory DST on this device "
                                                  "(2D: N <= 2048; the mixed path goes to 4096)");
-  KFBI_CUDA(p, (set_smem<double, 1>(optin)));
-  KFBI_CUDA(p, (set_smem<double, 2>(optin)));
-  KFBI_CUDA(p, (set_smem<double, 4>(optin)));
-  KFBI_CUDA(p, (set_smem<double, 8>(optin)));
+  KFBI_CUDA(p, set_smem<1>(optin));
+  KFBI_CUDA(p, set_smem<2>(optin));
+  KFBI_CUDA(p, set_smem<4>(optin));
+  KFBI_CUDA(p, set_smem<8>(optin));
   KFBI_CUDA(p, (set_smem_mma<6, 4>()));
   KFBI_CUDA(p, (set_smem_mma<7, 4>()));
   KFBI_CUDA(p, (set_smem_mma<8, 4>()));
@@ -1856,9 +1778,7 @@ void box_destroy(kfbi_problem* p) {
   BoxSolver* B = p->box;
   if (!B) return;
   cudaFree(B->tw64);
-  cudaFree(B->tw32);
   cudaFree(B->twst);
-  cudaFree(B->cosv);
   cudaFree(B->s64);
   cudaFree(B->s32);
   cudaFree(B->scale64);
@@ -1919,7 +1839,7 @@ kfbi_status box_steps_total(kfbi_problem* p, long long* out) {
 // write it (the FP64 transform)
 kfbi_status box_solve_interior(kfbi_problem* p, const double* rhs, double* u) {
   if (p->mg || p->cfg.precision == KFBI_MIXED) return box_solve(p, rhs, u);
-  return dst_solve_t<double>(p, rhs, 1, u, 0, nullptr);
+  return dst_solve64(p, rhs, u);
 }
 
 kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
@@ -1930,7 +1850,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   BoxSolver* B = p->box;
   const Grid g = p->g;
   if (p->cfg.precision != KFBI_MIXED) {
-    KFBI_TRY(dst_solve_t<double>(p, rhs, 1, u, 0, nullptr));
+    KFBI_TRY(dst_solve64(p, rhs, u));
     return launch_set_boundary(p, u, nullptr);
   }
   // mixed: u0 = DST32^{-1}(R) (FP32, in place in the work grid); fixed-point
@@ -1946,27 +1866,20 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
   unsigned long long* slot = B->nrm + 9;   // step s: slot + 2 s
   const double margin = first_margin(p);
   {
-    PassPlan P0 = plan_passes<float>(p, rhs, 1, u, 0, nullptr, slot);
+    PassPlan P0 = plan_passes<float>(p, rhs, 1, B->work32, nullptr);
     P0.args[0].zero_nrm = B->nrm;
     P0.args[0].zero_conv = B->conv;
-    PassArgs& last = P0.args[P0.npass - 1];
-    last.dst = B->work32;
-    last.dst64 = 0;
-    last.accumulate = 0;
-    last.corr_max = slot;
-    for (int k = 0; k < P0.npass; ++k) launch_pass<float>(p, P0.args[k], P0.npairs, P0.na, st, P0.pmin[k]);
+    P0.args[P0.npass - 1].corr_max = slot;
+    for (int k = 0; k < P0.npass; ++k) launch_pass32(p, P0.args[k], P0.npairs, P0.na, st);
   }
   launch_fix0(p, g, B->work32, rhs, slot + 1, B->multh2, B->kc, B->fixd, B->fixf, B->ufix, B->rfix,
               B->refine_steps > 1 ? nullptr : u, st);
   if (B->refine_steps == 1)
     KFBI_LAUNCH(p, KFBI_KC_RESIDUAL, k_check<<<1, 1, 0, st>>>(StepCheck{B->nrm, B->tol_dev, B->conv, margin, 0, false}));
   float* r32 = reinterpret_cast<float*>(B->res);
-  PassPlan PK = plan_passes<float>(p, r32, 0, u, 0, B->conv, nullptr);
+  PassPlan PK = plan_passes<float>(p, r32, 0, nullptr, B->conv);
   {
     PassArgs& last = PK.args[PK.npass - 1];
-    last.dst = nullptr;
-    last.dst64 = 0;
-    last.accumulate = 1;
     last.dstfix = B->ufix;
     last.fixf = B->fixf;
     last.fixd = B->fixd;
@@ -1978,7 +1891,7 @@ kfbi_status box_solve(kfbi_problem* p, const double* rhs, double* u) {
     PassArgs& last = PK.args[PK.npass - 1];
     last.corr_max = slot + 2 * it;
     last.uout = it + 1 < B->refine_steps ? nullptr : u;   // the last step also writes the FP64 solution
-    for (int k = 0; k < PK.npass; ++k) launch_pass<float>(p, PK.args[k], PK.npairs, PK.na, st, PK.pmin[k]);
+    for (int k = 0; k < PK.npass; ++k) launch_pass32(p, PK.args[k], PK.npairs, PK.na, st);
   }
   KFBI_CUDA(p, cudaGetLastError());
   return KFBI_OK;
@@ -2159,7 +2072,7 @@ template <int P>
 void noalloc_pass(const PassArgs& A, int npairs, int na, cudaStream_t st) {
   dim3 grid((unsigned)((npairs + P - 1) / P), (unsigned)na);
   size_t smem = sizeof(Cx<double>) * (size_t)(2 * A.n) * P * 2;
-  k_dst_pass<double, P><<<grid, 256, smem, st>>>(A);
+  k_dst_pass<P><<<grid, 256, smem, st>>>(A);
 }
 
 void noalloc_launch(const PassArgs& A, int npairs, int na, cudaStream_t st, int pmin) {
@@ -2206,10 +2119,10 @@ extern "C" kfbi_status kfbi_box_solve_noalloc(int dim, int n, double lo, double 
       int optin = 0;
       if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return KFBI_ERR_CUDA;
-      if (cudaFuncSetAttribute(k_dst_pass<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
-          cudaFuncSetAttribute(k_dst_pass<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
-          cudaFuncSetAttribute(k_dst_pass<double, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
-          cudaFuncSetAttribute(k_dst_pass<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
+      if (cudaFuncSetAttribute(k_dst_pass<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+          cudaFuncSetAttribute(k_dst_pass<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+          cudaFuncSetAttribute(k_dst_pass<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+          cudaFuncSetAttribute(k_dst_pass<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return KFBI_ERR_CUDA;
       g_noalloc_ptr[dev] = ptr;
     }
@@ -2241,29 +2154,26 @@ extern "C" kfbi_status kfbi_box_solve_noalloc(int dim, int n, double lo, double 
   A.order = order;
   const int npairs = n / 2;
   const int n1 = n + 1;
-  auto io = [&](const void* s, void* d, int d64) {
+  auto io = [&](const void* s, void* d) {
     A.src = s;
-    A.src64 = 1;
     A.dst = d;
-    A.dst64 = d64;
-    A.accumulate = 0;
   };
   if (dim == 2) {
-    io(rhs, work, 1);
+    io(rhs, work);
     A.sa = 0; A.sb = n1; A.es = 1; A.fused = 0;
     noalloc_launch(A, npairs, 1, st, 1);
-    io(work, work, 1);
+    io(work, work);
     A.sa = 0; A.sb = 1; A.es = n1; A.fused = 1;
     noalloc_launch(A, npairs, 1, st, 2);
-    io(work, u, 1);
+    io(work, u);
     A.sa = 0; A.sb = n1; A.es = 1; A.fused = 0;
     noalloc_launch(A, npairs, 1, st, 1);
   } else {
     const long long s0 = (long long)n1 * n1;
-    io(rhs, work, 1);
+    io(rhs, work);
     A.sa = s0; A.sb = n1; A.es = 1; A.fused = 0;
     noalloc_launch(A, npairs, n - 1, st, 1);
-    io(work, work, 1);
+    io(work, work);
     A.sa = s0; A.sb = 1; A.es = n1;
     noalloc_launch(A, npairs, n - 1, st, 2);
     A.sa = n1; A.sb = 1; A.es = s0; A.fused = 1;
@@ -2271,7 +2181,7 @@ extern "C" kfbi_status kfbi_box_solve_noalloc(int dim, int n, double lo, double 
     A.fused = 0;
     A.sa = s0; A.sb = 1; A.es = n1;
     noalloc_launch(A, npairs, n - 1, st, 2);
-    io(work, u, 1);
+    io(work, u);
     A.sa = s0; A.sb = n1; A.es = 1;
     noalloc_launch(A, npairs, n - 1, st, 1);
   }
@@ -2324,7 +2234,7 @@ __global__ void k_zero_batched(const BoxDesc* __restrict__ D, int ninst, const i
 }
 
 // the batched check after refinement step `step`, with the rules of
-// check_body (the first FP32 solve stops on the observed error estimate)
+// step_stop (the first FP32 solve stops on the observed error estimate)
 __global__ void k_check_batched(const BoxDesc* __restrict__ D, int ninst, int step) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ninst) return;
@@ -2506,20 +2416,11 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
                   "batched solves need mixed-precision DST problems of one dimension with N <= 1024");
     BoxSolver* B = p->box;
     float* r32 = reinterpret_cast<float*>(B->res);
-    plan0[i] = plan_passes<float>(p, rhs[i], 1, p->ugrid, 0, B->conv, B->nrm + 3);
-    {
-      PassArgs& last = plan0[i].args[plan0[i].npass - 1];
-      last.dst = B->work32;
-      last.dst64 = 0;
-      last.accumulate = 0;
-      last.corr_max = B->nrm + 3;
-    }
-    plank[i] = plan_passes<float>(p, r32, 0, p->ugrid, 0, B->conv, B->nrm + 3);
+    plan0[i] = plan_passes<float>(p, rhs[i], 1, B->work32, B->conv);
+    plan0[i].args[plan0[i].npass - 1].corr_max = B->nrm + 3;
+    plank[i] = plan_passes<float>(p, r32, 0, nullptr, B->conv);
     {
       PassArgs& last = plank[i].args[plank[i].npass - 1];
-      last.dst = nullptr;
-      last.dst64 = 0;
-      last.accumulate = 1;
       last.dstfix = B->ufix;
       last.fixf = B->fixf;
       last.fixd = B->fixd;
