@@ -923,7 +923,11 @@ static_assert(Reg<4, batch_pairs(4)>::THREADS == kBatchPassThreads && Reg<8, bat
 // up to L = 2048 uses 160 threads and at most 20.2 KB per work item
 // (P = batch_pairs(LOGL)), so one kernel takes the work items of all
 // instances (item -> instance by binary search in `start`) and dispatches on
-// the instance's LOGL.
+// the instance's LOGL.  The caps of 72 and 64 registers make the eight inlined
+// bodies spill (2.0 and 4.9 KB of stores over all of them, by -Xptxas -v), and are
+// the faster for it, the passes being bound by latency: 64 stars 37.6, 34.4, 32.8 ms
+// at two, three and four CTAs per SM (one kernel for both directions), 31.7 ms with a
+// kernel each at five and six.
 template <bool STR>
 __global__ void __launch_bounds__(kBatchPassThreads, STR ? 6 : 5)
     k_dst32_batched(const PassArgs* __restrict__ args, const int* __restrict__ start, int ninst) {
