@@ -36,10 +36,10 @@ struct kfbi_batch {
   int n = 0, m = 0, maxnb = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;
-  kfbi::BatchBox* bb = nullptr;        // box solves of the GMRES loop (each problem's RHS buffer)
-  kfbi::BatchBox* bb_data = nullptr;   // box solves with data (buffers of the batch)
+  kfbi::BatchBox* bb = nullptr;        // box solves of the GMRES loop (sparse RHS buffers)
+  kfbi::BatchBox* bb_data = nullptr;   // box solves with data (each problem's RHS buffer)
   kfbi::BatchHot* bh = nullptr;
-  std::vector<double*> rhs_data;
+  std::vector<double*> rhs_loop;
   kfbi::ArnDesc* darn = nullptr;
   kfbi::BatchInst* dinst = nullptr;
   kfbi::BatchInst* hinst = nullptr;    // pinned staging of the per-call pointers
@@ -136,8 +136,8 @@ static bool build_loop(kfbi_batch* b) {
 }
 
 // Potentials with data of every instance: per instance the correction values
-// (a, b, f~ from data[k]) and the corrected right-hand side into the batch's
-// buffer for it, then one batched box solve into each problem's grid,
+// (a, b, f~ from data[k]) and the corrected right-hand side into the
+// problem's RHS buffer, then one batched box solve into each problem's grid,
 // whose boundary layer stays zero.
 static kfbi_status batch_potentials(kfbi_batch* b, const double* const* a, const double* const* bb,
                                     const kfbi_data* data, bool use_gb) {
@@ -147,7 +147,7 @@ static kfbi_status batch_potentials(kfbi_batch* b, const double* const* a, const
     kfbi_data dd = data[k];
     if (!use_gb) dd.g_b = nullptr;
     KFBI_TRY(launch_correction_values_data(p, a ? a[k] : nullptr, bb ? bb[k] : nullptr, &dd, p->cvals));
-    KFBI_TRY(launch_rhs(p, p->cvals, &dd, b->rhs_data[k]));
+    KFBI_TRY(launch_rhs(p, p->cvals, &dd, p->rhs));
   }
   return batch_box_solve(p0, b->bb_data, b->zeros, b->stream);
 }
@@ -174,7 +174,7 @@ kfbi_status kfbi_destroy_batch(kfbi_batch* b) {
   batch_box_destroy(b->bb);
   batch_box_destroy(b->bb_data);
   batch_hot_destroy(b->bh);
-  for (double* r : b->rhs_data) cudaFree(r);
+  for (double* r : b->rhs_loop) cudaFree(r);
   cudaFree(b->darn);
   cudaFree(b->dinst);
   cudaFree(b->jdev);
@@ -227,19 +227,21 @@ kfbi_status kfbi_create_batch(kfbi_problem* const* problems, int count, kfbi_bat
                        "N_b <= 32768"));
     b->maxnb = std::max(b->maxnb, p->nb);
   }
-  std::vector<double*> xs, ys, rhs_loop;
+  std::vector<double*> xs, ys, rhs_data;
   for (kfbi_problem* p : b->ps) {
     double* r = nullptr;
     if (dalloc(&r, p->g.nodes()) != cudaSuccess)
       return bail(fail(p0, KFBI_ERR_CUDA, "out of device memory"));
-    b->rhs_data.push_back(r);
+    b->rhs_loop.push_back(r);
+    // zero once: inside GMRES only the irregular entries are ever written
+    if (cudaMemset(r, 0, sizeof(double) * p->g.nodes()) != cudaSuccess)
+      return bail(fail(p0, KFBI_ERR_CUDA, "memset failed"));
     xs.push_back(p->xbuf);
     ys.push_back(p->ybuf);
-    // zero off the irregular nodes, the only ones written inside GMRES
-    rhs_loop.push_back(p->rhs);
+    rhs_data.push_back(p->rhs);
   }
   kfbi_status s;
-  if ((s = batch_hot_create(p0, b->ps.data(), count, xs.data(), ys.data(), rhs_loop.data(), &b->bh)) != KFBI_OK)
+  if ((s = batch_hot_create(p0, b->ps.data(), count, xs.data(), ys.data(), b->rhs_loop.data(), &b->bh)) != KFBI_OK)
     return bail(s);
   // per-instance refinement tolerances of the loop's box solves (each
   // problem's box_rtol, relaxed inside GMRES when relax > 0)
@@ -252,9 +254,9 @@ kfbi_status kfbi_create_batch(kfbi_problem* const* problems, int count, kfbi_bat
         cudaMemcpy(b->tol_base, base.data(), sizeof(double) * count, cudaMemcpyHostToDevice) != cudaSuccess)
       return bail(fail(p0, KFBI_ERR_CUDA, "out of device memory"));
   }
-  if ((s = batch_box_create(p0, b->ps.data(), count, rhs_loop.data(), &b->bb, b->tol)) != KFBI_OK)
+  if ((s = batch_box_create(p0, b->ps.data(), count, b->rhs_loop.data(), &b->bb, b->tol)) != KFBI_OK)
     return bail(s);
-  if ((s = batch_box_create(p0, b->ps.data(), count, b->rhs_data.data(), &b->bb_data)) != KFBI_OK) return bail(s);
+  if ((s = batch_box_create(p0, b->ps.data(), count, rhs_data.data(), &b->bb_data)) != KFBI_OK) return bail(s);
   std::vector<ArnDesc> ad(count);
   for (int k = 0; k < count; ++k) {
     kfbi_problem* p = b->ps[k];
@@ -277,16 +279,15 @@ kfbi_status kfbi_create_batch(kfbi_problem* const* problems, int count, kfbi_bat
       cudaMemset(b->ctl, 0, sizeof(int) * 4) != cudaSuccess)
     return bail(fail(p0, KFBI_ERR_CUDA, "descriptor upload failed"));
   // pick the box solve's launch shapes for this batch (before the capture,
-  // which records them), every instance active, on the batch's own buffers; the
-  // loop's solves share them
+  // which records them), every instance active; the data solves share them
   {
     // the tuning solves are set-up work: no per-launch timing events for them
     const bool prof_on = p0->prof.on;
     p0->prof.on = false;
-    s = batch_box_autotune(p0, b->bb_data, b->ps.data(), b->rhs_data.data(), b->done, b->stream);
+    s = batch_box_autotune(p0, b->bb, b->ps.data(), b->rhs_loop.data(), b->done, b->stream);
     p0->prof.on = prof_on;
     if (s != KFBI_OK) return bail(s);
-    batch_box_copy_tiles(b->bb, b->bb_data);
+    batch_box_copy_tiles(b->bb_data, b->bb);
   }
   if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
     return bail(fail(p0, KFBI_ERR_CUDA, "stream creation failed"));

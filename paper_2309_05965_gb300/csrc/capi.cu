@@ -22,7 +22,7 @@ kfbi_status fail(kfbi_problem* p, kfbi_status s, const std::string& msg) {
 // [u] = a, [d_n u] = b and no sources, then its four one-sided traces.
 static kfbi_status potential_traces(kfbi_problem* q, const double* a, const double* b, double* T) {
   const int nb = q->nb;
-  KFBI_TRY(launch_correction_values(q, a, b, nullptr, q->cvals));
+  KFBI_TRY(launch_correction_values_operator(q, a, b, q->cvals));
   KFBI_TRY(launch_rhs_operator(q, q->cvals));
   KFBI_TRY(box_solve_interior(q, q->rhs, q->ugrid));
   return launch_traces(q, q->ugrid, q->cvals, T, T + nb, T + 2 * nb, T + 3 * nb);
@@ -50,7 +50,7 @@ kfbi_status apply_operator_impl(kfbi_problem* p, const double* x, double* y) {
   const bool dir = p->cfg.kind == KFBI_DIRICHLET_INTERIOR;
   const bool neu = p->cfg.kind == KFBI_NEUMANN_INTERIOR;
   // Step 3.1 (fitted and evaluated at the irregular nodes)
-  KFBI_TRY(launch_correction_values(p, dir ? x : nullptr, dir ? nullptr : x, nullptr, p->cvals));
+  KFBI_TRY(launch_correction_values_operator(p, dir ? x : nullptr, dir ? nullptr : x, p->cvals));
   // Step 3.2
   KFBI_TRY(launch_rhs_operator(p, p->cvals));
   // Step 3.3
@@ -106,11 +106,8 @@ static kfbi_status potential_with_data(kfbi_problem* p, const double* a, const d
   if (data) dd = *data;
   if (!use_gb) dd.g_b = nullptr;
   KFBI_TRY(launch_correction_values_data(p, a, b, &dd, p->cvals));
-  kfbi_status s = launch_rhs(p, p->cvals, &dd, p->rhs);
-  if (s == KFBI_OK) s = box_solve(p, p->rhs, u);
-  const kfbi_status r = reset_rhs(p, &dd);
-  if (s != KFBI_OK) return s;
-  KFBI_TRY(r);
+  KFBI_TRY(launch_rhs(p, p->cvals, &dd, p->rhs));
+  KFBI_TRY(box_solve(p, p->rhs, u));
   return launch_set_boundary(p, u, use_gb ? dd.g_b : nullptr);
 }
 
@@ -341,6 +338,7 @@ static kfbi_status alloc_work(kfbi_problem* p) {
   p->nx = p->cfg.kind == KFBI_INTERFACE_GENERAL ? 2 * p->nb : p->nb;
   const long long nodes = p->g.nodes();
   if ((!p->rhs && dalloc(&p->rhs, nodes) != cudaSuccess) ||
+      (!p->rhs_dirty && dalloc(&p->rhs_dirty, 1) != cudaSuccess) ||
       (!p->ugrid && dalloc(&p->ugrid, nodes) != cudaSuccess) ||
       galloc(p, &p->cvals, p->nent) != cudaSuccess || galloc(p, &p->tvals, p->nb) != cudaSuccess ||
       galloc(p, &p->bvec, p->nx) != cudaSuccess || galloc(p, &p->xbuf, p->nx) != cudaSuccess ||
@@ -350,6 +348,7 @@ static kfbi_status alloc_work(kfbi_problem* p) {
   // what the operator expects to find: R zero off the (new) irregular nodes, u
   // zero on the boundary layer
   KFBI_CUDA(p, cudaMemsetAsync(p->rhs, 0, sizeof(double) * nodes, p->stream));
+  KFBI_CUDA(p, cudaMemsetAsync(p->rhs_dirty, 0, sizeof(int), p->stream));
   KFBI_TRY(launch_set_boundary(p, p->ugrid, nullptr));
   return gmres_create(p, kMaxKrylov);
 }
@@ -485,7 +484,7 @@ kfbi_status kfbi_destroy_problem(kfbi_problem* p) {
   box_destroy(p);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   if (p->ls_samples) cudaFree(p->ls_samples);
-  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->ugrid, p->ftilde, p->stencil_dev};
+  void* bufs[] = {p->nb_off, p->nb_coef, p->rhs, p->rhs_dirty, p->ugrid, p->ftilde, p->stencil_dev};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t e : p->prof.pool) cudaEventDestroy(e);

@@ -207,7 +207,8 @@ struct kfbi_problem {
   // box solver + work
   kfbi::BoxSolver* box = nullptr;
   double* cvals = nullptr;       // [n_ent]
-  double* rhs = nullptr;         // grid, between calls zero off the irregular nodes (reset_rhs)
+  double* rhs = nullptr;         // grid
+  int* rhs_dirty = nullptr;      // 1 while data with sources or outer values are in rhs (launch_rhs_operator)
   double* ugrid = nullptr;       // grid
   double* tvals = nullptr;       // [N_b]
   double* ftilde = nullptr;      // grid scratch
@@ -335,9 +336,8 @@ kfbi_status launch_collocation_fit(kfbi_problem* p, const double* a, const doubl
 kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* data,
                        double* rhs);
 kfbi_status launch_rhs_operator(kfbi_problem* p, const double* cvals);
-// p->rhs back to zero off the irregular nodes, as the operator expects it, after
-// launch_rhs put data with sources or outer values there
-kfbi_status reset_rhs(kfbi_problem* p, const kfbi_data* data);
+// the operator's correction values (no f~), before launch_rhs_operator
+kfbi_status launch_correction_values_operator(kfbi_problem* p, const double* a, const double* b, double* cvals);
 kfbi_status launch_correction_values_data(kfbi_problem* p, const double* a, const double* b,
                                           const kfbi_data* data, double* cvals);
 kfbi_status upload_neighbour_tables(kfbi_problem* p);
