@@ -438,15 +438,21 @@ kfbi_status kfbi_evaluate_batch(kfbi_batch* b, const kfbi_data* data, const doub
     if (mu) bb[k] = densities[k];
   }
   KFBI_TRY(batch_potentials(b, a.data(), mu ? bb.data() : nullptr, data, mu));
-  // every layer before any output: outputs may be the buffers of the outer values
-  if (mu)
+  // outputs that are also buffers of outer values: every layer before any output,
+  // by way of the problems' grids; else each layer after its output, one launch less
+  bool shared = false;
+  for (int k = 0; mu && k < n; ++k)
+    for (int j = 0; data[k].g_b && j < n && !shared; ++j)
+      shared = u_grids[j] < data[k].g_b + b->ps[k]->g.nodes() && data[k].g_b < u_grids[j] + b->ps[j]->g.nodes();
+  if (shared)
     for (int k = 0; k < n; ++k)
       if (data[k].g_b) KFBI_TRY(launch_set_boundary(b->ps[k], b->ps[k]->ugrid, data[k].g_b));
   for (int k = 0; k < n; ++k) {
     kfbi_problem* p = b->ps[k];
     KFBI_CUDA(p0, cudaMemcpyAsync(u_grids[k], p->ugrid, sizeof(double) * p->g.nodes(), cudaMemcpyDeviceToDevice,
                                   b->stream));
-    if (mu) KFBI_TRY(reset_boundary(p, &data[k]));
+    if (mu && data[k].g_b)
+      KFBI_TRY(shared ? launch_set_boundary(p, p->ugrid, nullptr) : launch_set_boundary(p, u_grids[k], data[k].g_b));
   }
   return KFBI_OK;
 }
