@@ -222,22 +222,12 @@ __global__ void k_traces4(int nb, TraceCSR tp, TraceCSR tm, const double* __rest
   int lane = threadIdx.x & 31;
   if (i >= nb) return;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int e = tp.ptr[i] + lane; e < tp.mid[i]; e += 32) {
-    const double w = u[tp.node[e]];
-    s[0] += tp.wv[e] * w;
-    s[1] += tp.wn[e] * w;
-  }
-  for (int e = tp.mid[i] + lane; e < tp.ptr[i + 1]; e += 32) {
+  for (int e = tp.ptr[i] + lane; e < tp.ptr[i + 1]; e += 32) {
     const double w = trace_datum<MULTI, false>(tp, e, u, cv);
     s[0] += tp.wv[e] * w;
     s[1] += tp.wn[e] * w;
   }
-  for (int e = tm.ptr[i] + lane; e < tm.mid[i]; e += 32) {
-    const double w = u[tm.node[e]];
-    s[2] += tm.wv[e] * w;
-    s[3] += tm.wn[e] * w;
-  }
-  for (int e = tm.mid[i] + lane; e < tm.ptr[i + 1]; e += 32) {
+  for (int e = tm.ptr[i] + lane; e < tm.ptr[i + 1]; e += 32) {
     const double w = trace_datum<MULTI, true>(tm, e, u, cv);
     s[2] += tm.wv[e] * w;
     s[3] += tm.wn[e] * w;
