@@ -442,10 +442,22 @@ size_t coarse_smem(const LvlArgs<T>& A, int lstart) {
   return b;
 }
 
-// f(t) at every interior node t of a grid of n = 2^ln
-template <typename F>
+// f(x, y, z, t) at every interior node t of a grid of n = 2^ln: in FP32 by shifts, over
+// the boundary indices 0 too; in FP64, bound by its pipe (16 cycles a warp
+// instruction), by divisions, so that the lanes are full (16^3 2nd order, 40
+// cycles: 2.05 ms by shifts).
+template <typename T, typename F>
 __device__ __forceinline__ void for_interior(int d, int ln, F&& f) {
   const int n = 1 << ln, n1 = n + 1, mask = n - 1;
+  if (sizeof(T) == 8) {
+    const unsigned m = n - 1, tot = d == 3 ? m * m * m : m * m;
+    for (unsigned q = threadIdx.x; q < tot; q += kCoarseThreads) {
+      const unsigned r = q / m, zz = r / m;
+      const int x = (int)(q - r * m) + 1, y = (int)(d == 3 ? r - zz * m : r) + 1, z = d == 3 ? (int)zz + 1 : 1;
+      f(x, y, z, d == 3 ? (z * n1 + y) * n1 + x : y * n1 + x);
+    }
+    return;
+  }
   for (int q = threadIdx.x; q < 1 << (d * ln); q += kCoarseThreads) {
     const int x = q & mask, y = (q >> ln) & mask, z = d == 3 ? q >> (2 * ln) : 1;
     if (x == 0 || y == 0 || z == 0) continue;
@@ -455,12 +467,13 @@ __device__ __forceinline__ void for_interior(int d, int ln, F&& f) {
 
 // Jacobi (mode 0: out = uin + omega/c0 (f - A uin)) or residual (mode 1) at every
 // interior node.  At 16^3 a thread marches over four nodes of a column with the
-// slice sums of k_march (9 loads a node instead of 27).
+// slice sums of k_march (9 loads a node instead of 27), but for the 7-point operator
+// in FP64, whose sums are fewer than the slices' (16^3: 3.25 ms marching).
 template <typename T>
 __device__ void blk_sweep(int d, int order, const Lvl<T>& L, int ln, const T* uin, const T* f, T* out, int mode) {
   const int n1 = (1 << ln) + 1;
   const T dw = L.dinv_w;
-  if (d == 3 && ln == 4) {
+  if (d == 3 && ln == 4 && (order == 4 || sizeof(T) == 4)) {
     const int x = threadIdx.x & 15, y = (threadIdx.x >> 4) & 15, zc = (threadIdx.x >> 8) * 4;
     if (x > 0 && y > 0) {
       const int plane = n1 * n1, z0 = max(zc, 1);
@@ -477,7 +490,7 @@ __device__ void blk_sweep(int d, int order, const Lvl<T>& L, int ln, const T* ui
       }
     }
   } else {
-    for_interior(d, ln, [&](int, int, int, int t) {
+    for_interior<T>(d, ln, [&](int, int, int, int t) {
       const T au = apply_at<T>(d, order, n1, L.c, uin + t);
       out[t] = mode == 0 ? uin[t] + dw * (f[t] - au) : f[t] - au;
     });
@@ -521,7 +534,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
     T* t = C[k].t;
     // two sweeps, u -> t -> u (kNu = 2); corrections start from zero
     if (k > 0 || start_zero) {
-      for_interior(d, ln, [&](int, int, int, int q) { t[q] = L.dinv_w * f[q]; });
+      for_interior<T>(d, ln, [&](int, int, int, int q) { t[q] = L.dinv_w * f[q]; });
       __syncthreads();
     } else {
       blk_sweep<T>(d, A.order, L, ln, C[k].u, f, t, 0);
@@ -530,7 +543,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
     // residual into t, restricted to the next f
     blk_sweep<T>(d, A.order, L, ln, C[k].u, f, t, 1);
     T* fc = C[k + 1].f;
-    for_interior(d, C[k + 1].ln, [&](int x, int y, int z, int q) {
+    for_interior<T>(d, C[k + 1].ln, [&](int x, int y, int z, int q) {
       T acc = (T)0;
       if (d == 2) {
         const T* r = t + 2 * y * n1 + 2 * x;
@@ -572,7 +585,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
     const int nc1 = A.L[lstart + k + 1].n + 1;
     const T* uc = C[k + 1].u;
     T* u = C[k].u;
-    for_interior(d, C[k].ln, [&](int x, int y, int z, int q) {
+    for_interior<T>(d, C[k].ln, [&](int x, int y, int z, int q) {
       const int ox = x & 1, oy = y & 1, oz = d == 3 ? z & 1 : 0;
       const T* c = uc + ((d == 3 ? (z >> 1) * nc1 : 0) + (y >> 1)) * nc1 + (x >> 1);
       T acc = (T)0;
