@@ -1484,8 +1484,9 @@ void launch_pass32(kfbi_problem* p, const PassArgs& A, int npairs_b, int na, cud
   }
 }
 
-// The FP64 pass on the tensor cores (dst_mma.cuh), N = 64..1024; below and
-// above (2D 2048, whose lines do not fit beside their digits) the FFT kernel stays.
+// The FP64 pass on the tensor cores (dst_mma.cuh), N = 64..1024 (3D: ..512); below
+// and above (2D 2048, whose lines do not fit beside their digits) the FFT kernel
+// stays: a dense product costs N per element, an FFT log N (1024^3 505 ms, products 516).
 // Measured, FFT -> products, FP64 box solve: 256^3 6709 -> 2116 us, 128^3 845 ->
 // 234, 64^3 124 -> 50, 1024^2 414 -> 412, 512^2 116 -> 85, 256^2 52 -> 35, 64^2
 // 33 -> 27; relative error against a quad-precision solve 4e-16..9e-16 -> 1e-16..3e-16.
@@ -1720,7 +1721,7 @@ kfbi_status box_create(kfbi_problem* p) {
     k_scale_table<<<std::min(div_up(nm, 256), 152 * 16), 256>>>(g.d, p->cfg.order, n, p->kt * g.h * g.h,
                                                                 gh2, B->s64, B->scale64);
     KFBI_CUDA(p, cudaGetLastError());
-    if (n >= kMmaMinN && n <= kMmaMaxN) {
+    if (n >= kMmaMinN && n <= (g.d == 2 ? kMmaMaxN2 : kMmaMaxN3)) {
       // round(2^62 sin(pi i / N)), i = 0..N
       std::vector<long long> sq(n + 1);
       const long double pi = acosl(-1.0L);

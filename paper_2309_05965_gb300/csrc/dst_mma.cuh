@@ -26,7 +26,7 @@
 namespace kfbi {
 namespace {
 
-constexpr int kMmaMinN = 64, kMmaMaxN = 1024;   // box sizes the kernel takes
+constexpr int kMmaMinN = 64, kMmaMaxN2 = 1024, kMmaMaxN3 = 512;   // box sizes the kernel takes
 
 // (T 2^32 + L) 2^e rounded half up to FP64, |T| < 2^46, |L| < 2^50, by
 // assembling the bits; overflow gives an infinity

@@ -1,4 +1,4 @@
-"""Mixed box solves at the largest 3D grid the library takes, by both solvers."""
+"""Box solves at the largest 3D grid the library takes."""
 import math
 
 import pytest
@@ -6,17 +6,17 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("box", ["dst", "mg"])
-def test_mixed_box_solve_1024_cubed(box):
+@pytest.mark.parametrize("box,precision,tol", [("dst", 1, 5e-12), ("mg", 1, 5e-12), ("dst", 0, 1e-12)])
+def test_box_solve_1024_cubed(box, precision, tol):
     """The right-hand side of one discrete sine mode, whose solution is that mode.
-    Bound: the mixed box solve's 5e-12 of the oracle tests."""
+    Bounds: those of the oracle tests."""
     import torch
     from paper_2309_05965_gb300 import kfbi
     n, kappa, mode = 1024, 1.0, (3, 5, 2)
     if torch.cuda.mem_get_info()[0] < 110e9:
         pytest.skip("needs 110 GB of free device memory")
     G = kfbi.Problem(3, n, -1.0, 1.0, 3, [0.0, 0.0, 0.0, 0.05, 0.05, 0.05], kfbi.DIRICHLET_INTERIOR, kappa=kappa,
-                     precision=kfbi.MIXED, box_solver=kfbi.BOX_MG if box == "mg" else kfbi.BOX_DST)
+                     precision=precision, box_solver=kfbi.BOX_MG if box == "mg" else kfbi.BOX_DST)
     x = torch.arange(n + 1, dtype=torch.float64, device="cuda")
     ax = [torch.sin(x * (math.pi * k / n)).reshape([-1 if i == j else 1 for j in range(3)])
           for i, k in enumerate(mode)]
@@ -33,4 +33,4 @@ def test_mixed_box_solve_1024_cubed(box):
     G.close()
     del u, ax
     torch.cuda.empty_cache()
-    assert err < 5e-12
+    assert err < tol
