@@ -297,6 +297,13 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
   const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int peers = scale ? (int)gridDim.z : 1;        // the cluster is the grid's z extent
+  // spectral scale of accumulator v of a tile (1 off the grid)
+  auto scale_at = [&](const MmaTile& m, int v) {
+    const int b = b0 + 2 * c + (v & 1), k = m.k0 + m.kstep * (g + 8 * (v >> 1)), m1 = n - 1;
+    if (b >= n || k >= n) return 1.0;
+    return __ldg(A.scale64 + (A.d == 2 ? (k - 1) * m1 + b - 1 : ((k - 1) * m1 + a - 1) * m1 + b - 1));
+  };
+  constexpr bool AHEAD = LOGN > 9;
   bool waited = false;
   for (int t = t0; t < n / 16; t += ts) {
     const MmaTile m = mma_tile(n, t);
@@ -311,6 +318,12 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
     if (BIG)
 #pragma unroll
       for (int v = 0; v < 4; ++v) sT[v] = sL[v] = 0ll;
+    // N = 1024: the tile's scales before its products, which hide their latency (one
+    // CTA per SM does not; smaller N have no registers left for them)
+    double scl[AHEAD ? 4 : 1];
+    if (AHEAD && scale)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) scl[v] = scale_at(m, v);
     uint4 fa[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) fa[q] = __ldg(fr + 32 * q);
@@ -367,7 +380,7 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
     }
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      const int q = 2 * c + (v & 1), b = b0 + q;
+      const int q = 2 * c + (v & 1);
       const int k = m.k0 + m.kstep * (g + 8 * (v >> 1));
       if (k >= n) continue;
       long long T, L;
@@ -384,11 +397,7 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
       // units: digits 7 of both factors 2^56, the matrix 2^62, the line 2^(1082 - e)
       double r = sum_value(T, L, e - 1088);
       if (e == 0x7ff) r = __longlong_as_double(0x7ff8000000000000LL);   // a non-finite line
-      if (scale && b < n) {
-        const int m1 = n - 1;
-        const int at = A.d == 2 ? (k - 1) * m1 + b - 1 : ((k - 1) * m1 + a - 1) * m1 + b - 1;
-        r *= __ldg(A.scale64 + at);
-      }
+      if (scale) r *= AHEAD ? scl[AHEAD ? v : 0] : scale_at(m, v);
       if (peers == 1) {
         raw[q * pr + k - 1] = r;
       } else {
