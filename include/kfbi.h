@@ -361,12 +361,12 @@ typedef struct kfbi_batch kfbi_batch;
  * batch's own grids (kfbi_batch_tiles) and synchronises the stream. */
 kfbi_status kfbi_create_batch(kfbi_problem* const* problems, int count, kfbi_batch** out);
 kfbi_status kfbi_destroy_batch(kfbi_batch* batch);
-/* The launch shapes the autotuner picked at kfbi_create_batch: the CTA count
- * of the persistent FP32 transform pass (half, once or twice the CTAs the GPU
- * holds at once) and of the fixed-point row kernel (4, 8, 16 or 32 per SM),
- * each the fastest of its candidates in timed batched box solves with a
- * synthetic right-hand side.  The shapes only distribute work items; results
- * do not depend on them.  Host integers out; KFBI_ERR_ARG on NULL. */
+/* The launch shapes of the batched box solve: the CTAs of the FP32 transform
+ * pass that the GPU holds at once (it takes an item per CTA, in rows of so many),
+ * and the CTA count of the fixed-point row kernel (4, 8, 16 or 32 per SM, the
+ * fastest in timed batched box solves with a synthetic right-hand side at
+ * kfbi_create_batch).  The shapes only distribute work items; results do not
+ * depend on them.  Host integers out; KFBI_ERR_ARG on NULL. */
 kfbi_status kfbi_batch_tiles(const kfbi_batch* batch, int* pass_ctas, int* row_ctas);
 /* Algorithm 1 for every instance k: data[k] (host array of count kfbi_data
  * with device pointers as in kfbi_gmres_solve), x0s (host array of count

@@ -5,7 +5,7 @@
 // instances is one CUDA graph body:
 //   copy V_j -> x (all instances)        one launch
 //   C at irregular nodes, sparse RHS     two launches over all instances
-//   mixed box solves                     persistent launches over all
+//   mixed box solves                     one launch per pass over all
 //                                        instances' line pairs per pass
 //   traces + BIE combination             one launch over all DOFs
 //   copy y -> V_{j+1}, Arnoldi step      two launches (a CTA per instance)

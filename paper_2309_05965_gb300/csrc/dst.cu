@@ -919,44 +919,41 @@ static_assert(Reg<4, batch_pairs(4)>::THREADS == kBatchPassThreads && Reg<8, bat
               Reg<9, batch_pairs(9)>::THREADS == kBatchPassThreads && Reg<10, batch_pairs(10)>::THREADS == kBatchPassThreads &&
               Reg<11, batch_pairs(11)>::THREADS == kBatchPassThreads, "one CTA shape for every length");
 
-// Persistent FP32 pass over many independent grids: every transform length
-// up to L = 2048 uses 160 threads and at most 20.2 KB per work item
-// (P = batch_pairs(LOGL)), so one kernel takes the work items of all
-// instances (item -> instance by binary search in `start`) and dispatches on
-// the instance's LOGL.  The caps of 72 and 64 registers make the eight inlined
-// bodies spill (2.0 and 4.9 KB of stores over all of them, by -Xptxas -v), and are
-// the faster for it, the passes being bound by latency: 64 stars 37.6, 34.4, 32.8 ms
-// at two, three and four CTAs per SM (one kernel for both directions), 31.7 ms with a
-// kernel each at five and six.
+// FP32 pass over many independent grids: every transform length up to L = 2048
+// uses 160 threads and at most 20.2 KB per work item (P = batch_pairs(LOGL)), so one
+// kernel takes the work items of all instances (item -> instance by binary search
+// in `start`) and dispatches on the instance's LOGL.  An item per CTA: in a loop
+// over items the compiler keeps what it can lift out of every length's body, 209
+// registers against 94 for one length, or at the cap 2.0 and 4.9 KB of spills.  Against
+// persistent CTAs, whole solves: 64 stars with evaluation 29.1 -> 23.7 ms, one 1024^2
+// 5.29 -> 3.71, four 512^2 4.99 -> 3.62, 16 of 256^2 5.05 -> 3.98, 64 of 64^2 5.10 -> 4.87.
 template <bool STR>
-__global__ void __launch_bounds__(kBatchPassThreads, STR ? 6 : 5)
+__global__ void __launch_bounds__(kBatchPassThreads, 5)
     k_dst32_batched(const PassArgs* __restrict__ args, const int* __restrict__ start, int ninst) {
   extern __shared__ unsigned char smraw[];
   Cx<float>* sm = reinterpret_cast<Cx<float>*>(smraw);
-  const int total = start[ninst];
-  for (int item = blockIdx.x; item < total; item += gridDim.x) {
-    int lo = 0, hi = ninst;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (start[mid] <= item) lo = mid; else hi = mid;
-    }
-    const PassArgs& A = args[lo];
-    if (A.skip && *A.skip) continue;
-    const int local = item - start[lo];
-    const int p = batch_pairs(A.logL);
-    const int nbx = (A.n / 2 + p - 1) / p;
-    const int bx = local % nbx, by = local / nbx;
-    switch (A.logL) {
-      case 4: dst32_body<4, batch_pairs(4), STR>(A, bx, by, sm); break;
-      case 5: dst32_body<5, batch_pairs(5), STR>(A, bx, by, sm); break;
-      case 6: dst32_body<6, batch_pairs(6), STR>(A, bx, by, sm); break;
-      case 7: dst32_body<7, batch_pairs(7), STR>(A, bx, by, sm); break;
-      case 8: dst32_body<8, batch_pairs(8), STR>(A, bx, by, sm); break;
-      case 9: dst32_body<9, batch_pairs(9), STR>(A, bx, by, sm); break;
-      case 10: dst32_body<10, batch_pairs(10), STR>(A, bx, by, sm); break;
-      default: dst32_body<11, batch_pairs(11), STR>(A, bx, by, sm); break;
-    }
-    __syncthreads();
+  const int item = blockIdx.y * gridDim.x + blockIdx.x;
+  if (item >= start[ninst]) return;
+  int lo = 0, hi = ninst;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (start[mid] <= item) lo = mid; else hi = mid;
+  }
+  const PassArgs& A = args[lo];
+  if (A.skip && *A.skip) return;
+  const int local = item - start[lo];
+  const int p = batch_pairs(A.logL);
+  const int nbx = (A.n / 2 + p - 1) / p;
+  const int bx = local % nbx, by = local / nbx;
+  switch (A.logL) {
+    case 4: dst32_body<4, batch_pairs(4), STR>(A, bx, by, sm); break;
+    case 5: dst32_body<5, batch_pairs(5), STR>(A, bx, by, sm); break;
+    case 6: dst32_body<6, batch_pairs(6), STR>(A, bx, by, sm); break;
+    case 7: dst32_body<7, batch_pairs(7), STR>(A, bx, by, sm); break;
+    case 8: dst32_body<8, batch_pairs(8), STR>(A, bx, by, sm); break;
+    case 9: dst32_body<9, batch_pairs(9), STR>(A, bx, by, sm); break;
+    case 10: dst32_body<10, batch_pairs(10), STR>(A, bx, by, sm); break;
+    default: dst32_body<11, batch_pairs(11), STR>(A, bx, by, sm); break;
   }
 }
 
@@ -2197,7 +2194,7 @@ extern "C" kfbi_status kfbi_box_solve_noalloc(int dim, int n, double lo, double 
 // Batched mixed-precision box solve: many independent grids (different N),
 // the same steps as the single solve (FP32 solve, fixed-point scale, exact
 // residual, FP32 corrections), each step one launch over all instances: the
-// passes by persistent CTAs over all instances' line pairs, the grid kernels
+// passes by a CTA per item of all instances' line pairs, the grid kernels
 // over all instances' rows, with per-instance convergence flags.
 // ---------------------------------------------------------------------------
 namespace kfbi {
@@ -2384,23 +2381,21 @@ struct BatchBox {
   BoxDesc* dbox = nullptr;     // [ninst]
   int* drstart = nullptr;      // [ninst + 1] items of the row kernels
   bool str[5] = {};            // the pass's lines are strided
-  int grid = 0, rgrid = 0;     // CTAs of the contiguous passes and of the row kernels
-  int grid_s = 0;              // CTAs of the strided passes
-  int res_c = 0, res_s = 0;    // CTAs the GPU holds at once
+  int items = 0;               // of a pass
+  int grid = 0, rgrid = 0;     // CTAs in a row of the passes' grid (as many as the GPU holds at once), of the row kernels
 };
 
 void batch_launch_pass(kfbi_problem* p0, const BatchBox* bb, int v, const PassArgs* args, cudaStream_t st) {
-  if (bb->str[v])
-    KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<true><<<bb->grid_s, kBatchPassThreads, kBatchPassSmem, st>>>(
-        args, bb->dstart, bb->ninst));
-  else
-    KFBI_LAUNCH(p0, KFBI_KC_DST, k_dst32_batched<false><<<bb->grid, kBatchPassThreads, kBatchPassSmem, st>>>(
-        args, bb->dstart, bb->ninst));
+  const int g = std::min(bb->grid, bb->items);
+  const dim3 grid((unsigned)g, (unsigned)div_up(bb->items, g));
+  auto launch = [&](auto kernel) {
+    KFBI_LAUNCH(p0, KFBI_KC_DST, kernel<<<grid, kBatchPassThreads, kBatchPassSmem, st>>>(args, bb->dstart, bb->ninst));
+  };
+  bb->str[v] ? launch(k_dst32_batched<true>) : launch(k_dst32_batched<false>);
 }
 
 void batch_box_copy_tiles(BatchBox* dst, const BatchBox* src) {
   dst->grid = src->grid;
-  dst->grid_s = src->grid_s;
   dst->rgrid = src->rgrid;
 }
 
@@ -2459,13 +2454,11 @@ kfbi_status batch_box_create(kfbi_problem* p0, kfbi_problem* const* ps, int nins
   int dev = 0, sms = 0;
   KFBI_CUDA(p0, cudaGetDevice(&dev));
   KFBI_CUDA(p0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int per_c = 0, per_s = 0;
-  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_c, k_dst32_batched<false>, kBatchPassThreads,
+  int per = 0;
+  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_dst32_batched<false>, kBatchPassThreads,
                                                               kBatchPassSmem));
-  KFBI_CUDA(p0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_s, k_dst32_batched<true>, kBatchPassThreads,
-                                                              kBatchPassSmem));
-  bb->grid = bb->res_c = sms * std::max(1, per_c);
-  bb->grid_s = bb->res_s = sms * std::max(1, per_s);
+  bb->grid = sms * std::max(1, per);
+  bb->items = start[ninst];
   for (int v = 0; v < bb->npass; ++v) bb->str[v] = plan0[0].args[v].es != 1;
   bb->rgrid = sms * 8;
   return KFBI_OK;
@@ -2480,13 +2473,11 @@ __global__ void k_fill_pattern(long long tot, double* __restrict__ R) {
 }
 }  // namespace
 
-// Autotuner of the batched box solve's launch shapes: the CTA count of the
-// persistent transform pass (half, once or twice the CTAs resident on the
-// GPU) and of the row kernel (4, 8, 16 or 32 CTAs per SM), each timed on the
-// batch's own grids (a synthetic right-hand side, one warm-up and two timed
-// box solves per candidate, CUDA events) and the fastest kept.  The shapes
-// change only how the work items are spread, not the arithmetic.  rhs is
-// zeroed again afterwards.
+// Autotuner of the batched box solve's launch shapes: the CTA count of the row
+// kernel (4, 8, 16 or 32 CTAs per SM), each timed on the batch's own grids (a
+// synthetic right-hand side, one warm-up and two timed box solves per candidate,
+// CUDA events) and the fastest kept.  The shapes change only how the work items
+// are spread, not the arithmetic.  rhs is zeroed again afterwards.
 kfbi_status batch_box_autotune(kfbi_problem* p0, BatchBox* bb, kfbi_problem* const* ps, double* const* rhs,
                                const int* done, cudaStream_t st) {
   int dev = 0, sms = 0;
@@ -2509,23 +2500,8 @@ kfbi_status batch_box_autotune(kfbi_problem* p0, BatchBox* bb, kfbi_problem* con
     KFBI_CUDA(p0, cudaEventElapsedTime(ms, e0, e1));
     return KFBI_OK;
   };
-  const int resident = bb->res_c;
   kfbi_status s = KFBI_OK;
   float best = 1e30f;
-  int best_grid = resident;
-  for (int g : {std::max(1, resident / 2), resident, 2 * resident}) {
-    bb->grid = g;
-    bb->grid_s = std::max(1, (int)((long long)g * bb->res_s / bb->res_c));
-    float ms = 0.f;
-    if ((s = time_solve(&ms)) != KFBI_OK) break;
-    if (ms < best) {
-      best = ms;
-      best_grid = g;
-    }
-  }
-  bb->grid = best_grid;
-  bb->grid_s = std::max(1, (int)((long long)best_grid * bb->res_s / bb->res_c));
-  best = 1e30f;
   int best_rgrid = 8 * sms;
   for (int per : {4, 8, 16, 32}) {
     if (s != KFBI_OK) break;
