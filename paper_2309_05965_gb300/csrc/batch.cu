@@ -5,8 +5,8 @@
 // instances is one CUDA graph body:
 //   copy V_j -> x (all instances)        one launch
 //   C at irregular nodes, sparse RHS     two launches over all instances
-//   mixed box solves                     one launch per pass over all
-//                                        instances' line pairs per pass
+//   mixed box solves                     one launch per pass over the
+//                                        line pairs of all instances
 //   traces + BIE combination             one launch over all DOFs
 //   copy y -> V_{j+1}, Arnoldi step      two launches (a CTA per instance)
 //   convergence control                  one launch

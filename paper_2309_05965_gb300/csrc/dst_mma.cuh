@@ -410,6 +410,22 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
   if (!waited) cluster_wait();
 }
 
+// 2D, N = 1024: the digit table (2.2 MB) and the CTA's spectral scales on their way
+// into L2.  All CTAs walk the table in step, so where other grids have pushed it out,
+// it is else a chain of misses: operator on a problem not used just before 442 ->
+// 420 us (by FFT 428).  At 512^2 (0.6 MB) the requests cost more than they bring (86.0
+// against 85.3 us).
+template <int LOGN, int W>
+__device__ __forceinline__ void mma_prefetch(const PassArgs& A, const uint4* frag, int b0) {
+  using M = Mma<LOGN, W>;
+  constexpr int n = M::N;
+  auto fetch = [](const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); };
+  const int cta = blockIdx.z * gridDim.x + blockIdx.x, t = cta * M::THREADS + threadIdx.x;
+  for (int k = t; k < (int)(mma_frag_count(n) / 8); k += gridDim.x * gridDim.z * M::THREADS) fetch(frag + 8 * (long long)k);
+  if (A.fused)
+    for (int k = threadIdx.x; k < n - 1; k += M::THREADS) fetch(A.scale64 + (long long)k * (n - 1) + b0 - 1);
+}
+
 // One pass over the 8 lines b0.. of family a: W warps; the gridDim.z CTAs of a
 // cluster all read the lines and share their modes.
 template <int LOGN, int W>
@@ -425,6 +441,7 @@ __global__ void __launch_bounds__(32 * W, LOGN > 9 ? 1 : W == 8 ? 2 : 4) k_dst_m
   const int sb = (int)A.sb, es = (int)A.es, off0 = a * (int)A.sa + b0 * sb;   // 32-bit: at most 1025^3 nodes
   const bool contig = es == 1;
   if (threadIdx.x < NL) sexp[threadIdx.x] = 1;
+  if (LOGN > 9 && A.d == 2) mma_prefetch<LOGN, W>(A, frag, b0);
   double x[VALS];
   {
     const double* src = static_cast<const double*>(A.src) + off0;
