@@ -442,26 +442,27 @@ size_t coarse_smem(const LvlArgs<T>& A, int lstart) {
   return b;
 }
 
-// f(x, y, z, t) at every interior node t of a grid of n = 2^ln: in FP32 by shifts, over
-// the boundary indices 0 too; in FP64, bound by its pipe (16 cycles a warp
+// f(x, y, z, t) at every interior node t of a grid of n = 2^ln: by shifts, over the
+// boundary indices 0 too; 3D in FP64, bound by its pipe (16 cycles a warp
 // instruction), by divisions, so that the lanes are full (16^3 2nd order, 40
-// cycles: 2.05 ms by shifts).
-template <typename T, typename F>
-__device__ __forceinline__ void for_interior(int d, int ln, F&& f) {
+// cycles: 2.05 -> 1.83 ms).  In 2D, with a lane in 32 idle, divisions cost more
+// than they bring (128^2 3.28 -> 3.95 ms).
+template <typename T, int D, typename F>
+__device__ __forceinline__ void for_interior(int ln, F&& f) {
   const int n = 1 << ln, n1 = n + 1, mask = n - 1;
-  if (sizeof(T) == 8) {
-    const unsigned m = n - 1, tot = d == 3 ? m * m * m : m * m;
-    for (unsigned q = threadIdx.x; q < tot; q += kCoarseThreads) {
+  if (sizeof(T) == 8 && D == 3) {
+    const unsigned m = n - 1;
+    for (unsigned q = threadIdx.x; q < m * m * m; q += kCoarseThreads) {
       const unsigned r = q / m, zz = r / m;
-      const int x = (int)(q - r * m) + 1, y = (int)(d == 3 ? r - zz * m : r) + 1, z = d == 3 ? (int)zz + 1 : 1;
-      f(x, y, z, d == 3 ? (z * n1 + y) * n1 + x : y * n1 + x);
+      const int x = (int)(q - r * m) + 1, y = (int)(r - zz * m) + 1, z = (int)zz + 1;
+      f(x, y, z, (z * n1 + y) * n1 + x);
     }
     return;
   }
-  for (int q = threadIdx.x; q < 1 << (d * ln); q += kCoarseThreads) {
-    const int x = q & mask, y = (q >> ln) & mask, z = d == 3 ? q >> (2 * ln) : 1;
+  for (int q = threadIdx.x; q < 1 << (D * ln); q += kCoarseThreads) {
+    const int x = q & mask, y = (q >> ln) & mask, z = D == 3 ? q >> (2 * ln) : 1;
     if (x == 0 || y == 0 || z == 0) continue;
-    f(x, y, z, d == 3 ? (z * n1 + y) * n1 + x : y * n1 + x);
+    f(x, y, z, D == 3 ? (z * n1 + y) * n1 + x : y * n1 + x);
   }
 }
 
@@ -469,11 +470,11 @@ __device__ __forceinline__ void for_interior(int d, int ln, F&& f) {
 // interior node.  At 16^3 a thread marches over four nodes of a column with the
 // slice sums of k_march (9 loads a node instead of 27), but for the 7-point operator
 // in FP64, whose sums are fewer than the slices' (16^3: 3.25 ms marching).
-template <typename T>
-__device__ void blk_sweep(int d, int order, const Lvl<T>& L, int ln, const T* uin, const T* f, T* out, int mode) {
+template <typename T, int D>
+__device__ void blk_sweep(int order, const Lvl<T>& L, int ln, const T* uin, const T* f, T* out, int mode) {
   const int n1 = (1 << ln) + 1;
   const T dw = L.dinv_w;
-  if (d == 3 && ln == 4 && (order == 4 || sizeof(T) == 4)) {
+  if (D == 3 && ln == 4 && (order == 4 || sizeof(T) == 4)) {
     const int x = threadIdx.x & 15, y = (threadIdx.x >> 4) & 15, zc = (threadIdx.x >> 8) * 4;
     if (x > 0 && y > 0) {
       const int plane = n1 * n1, z0 = max(zc, 1);
@@ -490,8 +491,8 @@ __device__ void blk_sweep(int d, int order, const Lvl<T>& L, int ln, const T* ui
       }
     }
   } else {
-    for_interior<T>(d, ln, [&](int, int, int, int t) {
-      const T au = apply_at<T>(d, order, n1, L.c, uin + t);
+    for_interior<T, D>(ln, [&](int, int, int, int t) {
+      const T au = apply_at<T>(D, order, n1, L.c, uin + t);
       out[t] = mode == 0 ? uin[t] + dw * (f[t] - au) : f[t] - au;
     });
   }
@@ -501,12 +502,13 @@ __device__ void blk_sweep(int d, int order, const Lvl<T>& L, int ln, const T* ui
 // The V-cycle from level lstart down to the coarsest and back, in one CTA.
 // start_zero: the iterate at lstart starts from zero (a coarse correction, or
 // the first cycle on a grid that is coarse from the start).
-template <typename T>
+template <typename T, int D>
 __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, int lstart, int start_zero,
                                                                  const int* skip) {
   if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int d = A.d, nl = A.nlev - lstart;
+  constexpr int d = D;
+  const int nl = A.nlev - lstart;
   CoarseLvl<T> C[kMaxCoarse];
   {
     T* at = reinterpret_cast<T*>(smraw);
@@ -534,16 +536,16 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
     T* t = C[k].t;
     // two sweeps, u -> t -> u (kNu = 2); corrections start from zero
     if (k > 0 || start_zero) {
-      for_interior<T>(d, ln, [&](int, int, int, int q) { t[q] = L.dinv_w * f[q]; });
+      for_interior<T, D>(ln, [&](int, int, int, int q) { t[q] = L.dinv_w * f[q]; });
       __syncthreads();
     } else {
-      blk_sweep<T>(d, A.order, L, ln, C[k].u, f, t, 0);
+      blk_sweep<T, D>(A.order, L, ln, C[k].u, f, t, 0);
     }
-    blk_sweep<T>(d, A.order, L, ln, t, f, C[k].u, 0);
+    blk_sweep<T, D>(A.order, L, ln, t, f, C[k].u, 0);
     // residual into t, restricted to the next f
-    blk_sweep<T>(d, A.order, L, ln, C[k].u, f, t, 1);
+    blk_sweep<T, D>(A.order, L, ln, C[k].u, f, t, 1);
     T* fc = C[k + 1].f;
-    for_interior<T>(d, C[k + 1].ln, [&](int x, int y, int z, int q) {
+    for_interior<T, D>(C[k + 1].ln, [&](int x, int y, int z, int q) {
       T acc = (T)0;
       if (d == 2) {
         const T* r = t + 2 * y * n1 + 2 * x;
@@ -585,7 +587,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
     const int nc1 = A.L[lstart + k + 1].n + 1;
     const T* uc = C[k + 1].u;
     T* u = C[k].u;
-    for_interior<T>(d, C[k].ln, [&](int x, int y, int z, int q) {
+    for_interior<T, D>(C[k].ln, [&](int x, int y, int z, int q) {
       const int ox = x & 1, oy = y & 1, oz = d == 3 ? z & 1 : 0;
       const T* c = uc + ((d == 3 ? (z >> 1) * nc1 : 0) + (y >> 1)) * nc1 + (x >> 1);
       T acc = (T)0;
@@ -595,8 +597,8 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_cycle(LvlArgs<T> A, i
       u[q] += (ox ? (T)0.5 : (T)1) * (oy ? (T)0.5 : (T)1) * (oz ? (T)0.5 : (T)1) * acc;
     });
     __syncthreads();
-    blk_sweep<T>(d, A.order, L, C[k].ln, u, C[k].f, C[k].t, 0);
-    blk_sweep<T>(d, A.order, L, C[k].ln, C[k].t, C[k].f, u, 0);
+    blk_sweep<T, D>(A.order, L, C[k].ln, u, C[k].f, C[k].t, 0);
+    blk_sweep<T, D>(A.order, L, C[k].ln, C[k].t, C[k].f, u, 0);
   }
   T* gu = A.L[lstart].u;
   const int n1 = A.L[lstart].n + 1;
@@ -843,7 +845,8 @@ kfbi_status vcycle(kfbi_problem* p, LvlArgs<T>& A, int lcoarse, bool zero_guess,
     KFBI_LAUNCH(p, KFBI_KC_MG, k_restrict<T><<<rg, 128, 0, st>>>(
         d, A.L[l + 1].n, L.t, A.L[l + 1].f, skip));
   }
-  KFBI_LAUNCH(p, KFBI_KC_MG, k_coarse_cycle<T><<<1, kCoarseThreads, coarse_smem(A, lcoarse), st>>>(
+  auto coarse = d == 2 ? k_coarse_cycle<T, 2> : k_coarse_cycle<T, 3>;
+  KFBI_LAUNCH(p, KFBI_KC_MG, coarse<<<1, kCoarseThreads, coarse_smem(A, lcoarse), st>>>(
       A, lcoarse, (lcoarse > 0 || zero_guess) ? 1 : 0, skip));
   for (int l = lcoarse - 1; l >= 0; --l) {
     Lvl<T>& L = A.L[l];
@@ -906,9 +909,9 @@ kfbi_status build_levels(kfbi_problem* p, MgSolver* M, LvlArgs<T>& A, T** cinv, 
   KFBI_CUDA(p, cudaMemcpy(*cinv, cit.data(), sizeof(T) * cit.size(), cudaMemcpyHostToDevice));
   M->bufs.push_back(*cinv);
   A.cinv = *cinv;
-  // one limit for all problems: the largest coarse part, from 16^3
-  KFBI_CUDA(p, cudaFuncSetAttribute(k_coarse_cycle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(3 * sizeof(T) * (17 * 17 * 17 + 9 * 9 * 9 + 5 * 5 * 5))));
+  // one limit for all problems: the largest coarse part, from 16^3 (in 2D 36 KB at most)
+  KFBI_CUDA(p, (cudaFuncSetAttribute(k_coarse_cycle<T, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(3 * sizeof(T) * (17 * 17 * 17 + 9 * 9 * 9 + 5 * 5 * 5)))));
   return KFBI_OK;
 }
 
