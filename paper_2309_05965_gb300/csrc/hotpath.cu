@@ -20,7 +20,8 @@ namespace {
 // of the owner's collocation system (eq. (cau-ls)), one thread per correction
 // entry.  f~ = fa/sa - fb/sb at the PDE nodes (either pointer may be null);
 // fa holds one grid per interface when fstride > 0 (the entry's interface's).
-// With dirty (the operator): the grid R is cleared first if data left anything in it.
+// OP (the operator): the grid R is cleared first if data left anything in it.
+template <bool OP>
 __global__ void k_cvals(int nirr, int npde, int ndir, int nneu, double h,
                         const int32_t* __restrict__ owner, const double* __restrict__ W,
                         const int32_t* __restrict__ pde_node, const int32_t* __restrict__ dir_idx,
@@ -30,7 +31,7 @@ __global__ void k_cvals(int nirr, int npde, int ndir, int nneu, double h,
                         const int32_t* __restrict__ eiface, long long fstride, const int* __restrict__ dirty,
                         double* __restrict__ R, int tot) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (dirty && *dirty)
+  if (OP && *dirty)
     for (int t = q; t < tot; t += gridDim.x * blockDim.x) R[t] = 0.0;
   if (q >= nirr) return;
   int i = owner[q];
@@ -102,10 +103,9 @@ __global__ void k_rhs_source(Grid g, int order, const uint8_t* __restrict__ insi
                              const double* __restrict__ li, const double* __restrict__ lo_,
                              double rsi, double rso, double h2_12, const double* __restrict__ gb,
                              const double* __restrict__ nbc, const int8_t* __restrict__ nboff,
-                             int nnb, double* __restrict__ R, long long fstride, int* __restrict__ dirty) {
+                             int nnb, double* __restrict__ R, long long fstride) {
   const int tot = (int)g.nodes();
   const int n1 = g.n + 1;
-  if (dirty && blockIdx.x == 0 && threadIdx.x == 0) *dirty = 1;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += gridDim.x * blockDim.x) {
     int idx[3];
     if (g.d == 2) {
@@ -163,7 +163,7 @@ __global__ void k_rhs_correct(int nirr, int nnb, const int32_t* __restrict__ lin
                               const double* __restrict__ cv, double* __restrict__ R, int add,
                               int* __restrict__ dirty) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (dirty && q == 0) *dirty = 0;
+  if (dirty && q == 0) *dirty = add;
   if (q >= nirr) return;
   double acc = 0.0;
   for (int s = 0; s < nnb; ++s) {
@@ -183,7 +183,7 @@ __global__ void k_rhs_correct_multi(int nirr, int nnb, const int32_t* __restrict
                                     const double* __restrict__ nbc, const double* __restrict__ cv,
                                     double* __restrict__ R, int add, int* __restrict__ dirty) {
   int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (dirty && q == 0) *dirty = 0;
+  if (dirty && q == 0) *dirty = add;
   if (q >= nirr) return;
   double acc = 0.0;
   for (int s = 0; s < nnb; ++s) {
@@ -505,7 +505,7 @@ static long long in_stride(const kfbi_problem* p, const kfbi_data* data) {
 
 kfbi_status launch_correction_values(kfbi_problem* p, const double* a, const double* b,
                                      const double* ftilde, double* cvals) {
-  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<<<div_up(p->nent, 128), 128, 0, p->stream>>>(
+  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<false><<<div_up(p->nent, 128), 128, 0, p->stream>>>(
       p->nent, p->npde, p->ndir, p->nneu, p->g.h, p->ent_owner, p->ent_w, p->pde_node,
       p->dir_idx, p->neu_idx, a, b, ftilde, 1.0, nullptr, 1.0, cvals, p->ent_iface, 0, nullptr, nullptr, 0));
   KFBI_CUDA(p, cudaGetLastError());
@@ -513,7 +513,7 @@ kfbi_status launch_correction_values(kfbi_problem* p, const double* a, const dou
 }
 
 kfbi_status launch_correction_values_operator(kfbi_problem* p, const double* a, const double* b, double* cvals) {
-  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<<<div_up(p->nent, 128), 128, 0, p->stream>>>(
+  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<true><<<div_up(p->nent, 128), 128, 0, p->stream>>>(
       p->nent, p->npde, p->ndir, p->nneu, p->g.h, p->ent_owner, p->ent_w, p->pde_node,
       p->dir_idx, p->neu_idx, a, b, nullptr, 1.0, nullptr, 1.0, cvals, p->ent_iface, 0, p->rhs_dirty, p->rhs,
       (int)p->g.nodes()));
@@ -528,7 +528,7 @@ kfbi_status launch_correction_values_data(kfbi_problem* p, const double* a, cons
   const double* fo = data ? data->f_out : nullptr;
   double so = interior_bvp(p) ? 1.0 : p->cfg.sigma_out;
   if (interior_bvp(p)) fo = nullptr;
-  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<<<div_up(p->nent, 128), 128, 0, p->stream>>>(
+  KFBI_LAUNCH(p, KFBI_KC_CORRECTION, k_cvals<false><<<div_up(p->nent, 128), 128, 0, p->stream>>>(
       p->nent, p->npde, p->ndir, p->nneu, p->g.h, p->ent_owner, p->ent_w, p->pde_node,
       p->dir_idx, p->neu_idx, a, b, fi, p->cfg.sigma_in, fo, so, cvals, p->ent_iface,
       in_stride(p, data), nullptr, nullptr, 0));
@@ -569,7 +569,9 @@ kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* da
   const Grid g = p->g;
   const double* d_nbc = p->nb_coef;
   const int8_t* d_off = p->nb_off;
-  if (data && (data->f_in || data->f_out || data->lapf_in || data->lapf_out || data->g_b)) {
+  const bool fills = data && (data->f_in || data->f_out || data->lapf_in || data->lapf_out || data->g_b);
+  int* dirty = fills && rhs == p->rhs ? p->rhs_dirty : nullptr;
+  if (fills) {
     const double* fi = data->f_in;
     const double* fo = interior_bvp(p) ? nullptr : data->f_out;
     const double* li = data->lapf_in;
@@ -577,19 +579,18 @@ kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* da
     double so = interior_bvp(p) ? 1.0 : p->cfg.sigma_out;
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_source<<<std::min(div_up(g.nodes(), 256), 152 * 32), 256, 0, p->stream>>>(
         g, p->cfg.order, p->inside, fi, fo, li, lo_, 1.0 / p->cfg.sigma_in, 1.0 / so, g.h * g.h / 12.0,
-        interior_bvp(p) ? nullptr : data->g_b, d_nbc, d_off, p->n_nb, rhs, in_stride(p, data),
-        rhs == p->rhs ? p->rhs_dirty : nullptr));
+        interior_bvp(p) ? nullptr : data->g_b, d_nbc, d_off, p->n_nb, rhs, in_stride(p, data)));
     KFBI_CUDA(p, cudaGetLastError());
   } else {
     KFBI_CUDA(p, cudaMemsetAsync(rhs, 0, sizeof(double) * g.nodes(), p->stream));
   }
   if (cvals && p->n_iface > 1) {
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct_multi<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
-        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, d_nbc, cvals, rhs, 1, nullptr));
+        p->nirr, p->n_nb, p->irr_lin, p->corr_nb, p->corr_nb2, d_nbc, cvals, rhs, 1, dirty));
     KFBI_CUDA(p, cudaGetLastError());
   } else if (cvals) {
     KFBI_LAUNCH(p, KFBI_KC_RHS, k_rhs_correct<<<div_up(p->nirr, 128), 128, 0, p->stream>>>(
-        p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, d_nbc, cvals, rhs, 1, nullptr));
+        p->nirr, p->n_nb, p->irr_lin, p->irr_inside, p->corr_nb, d_nbc, cvals, rhs, 1, dirty));
     KFBI_CUDA(p, cudaGetLastError());
   }
   return KFBI_OK;
@@ -598,8 +599,8 @@ kfbi_status launch_rhs(kfbi_problem* p, const double* cvals, const kfbi_data* da
 // The operator's right-hand side: the corrections alone, assigned at the
 // irregular nodes of p->rhs, which is zero elsewhere: the kernel of the correction
 // values before this one clears it, but only after data with sources or outer
-// values were there.  That state is a word on the device, set by the kernel that
-// writes the sources and reset here, so that graphs replayed in any order find it.
+// values were there.  That state is a word on the device, set by the corrections after
+// sources (add) and reset by them here, so that graphs replayed in any order find it.
 // (A clearing pass per application is a grid of writes each time; a grid of the
 // operator's own costs its memory, 8.6 GB at 1024^3; a clearing after each use of
 // data 4 us of the 50 us right-hand side at 64^2.)
