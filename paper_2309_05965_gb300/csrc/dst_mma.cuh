@@ -320,8 +320,8 @@ __device__ __forceinline__ void mma_modes(const PassArgs& A, int t0, int ts, con
       for (int v = 0; v < 4; ++v) sT[v] = sL[v] = 0ll;
     // N = 1024: the tile's scales before its products, which hide their latency (one
     // CTA per SM does not; smaller N have no registers left for them).  Two operators'
-    // grids exceed L2: general right-hand side 956 -> 930 us, evaluation 936 -> 914
-    // (by FFT 919 and 908; one operator's 452 -> 448, 446 -> 436, solves 1.6 % faster)
+    // grids exceed L2: general right-hand side 956 -> 930 us, evaluation 936 -> 914,
+    // with mma_prefetch 916 and 897 (by FFT 919 and 908)
     double scl[AHEAD ? 4 : 1];
     if (AHEAD && scale)
 #pragma unroll
